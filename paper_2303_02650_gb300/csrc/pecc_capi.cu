@@ -32,7 +32,7 @@ struct pecc_ctx {
   float2 *x32 = nullptr;
   double2 *x64 = nullptr;
   void *xw = nullptr, *xb = nullptr, *xo = nullptr, *g = nullptr, *gt = nullptr, *d = nullptr, *xbuild = nullptr;
-  void *S = nullptr, *Y = nullptr, *gram = nullptr, *ecirc = nullptr;
+  void *S = nullptr, *gram = nullptr, *ecirc = nullptr;
   int32_t *perm = nullptr, *meta = nullptr;
   uint64_t *skey = nullptr;
   int32_t *rp = nullptr, *col = nullptr, *rp_s = nullptr, *col_s = nullptr;
@@ -288,8 +288,7 @@ pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
   ALC(p, double2, total); ctx->gt = p;
   ALC(p, double2, total); ctx->d = p;
   ALC(p, double2, total); ctx->xbuild = p;
-  ALC(p, char, vec2 * (size_t)m1 * (size_t)total); ctx->S = p;
-  ALC(p, char, vec2 * (size_t)m1 * (size_t)total); ctx->Y = p;
+  ALC(p, char, 2 * vec2 * (size_t)m1 * (size_t)total); ctx->S = p;
   ALC(p, char, vecs * (size_t)gram_off); ctx->gram = p;
   ALC(ctx->meta, int32_t, meta_off);
   ALC(p, double, total); ctx->ecirc = p;
@@ -623,7 +622,7 @@ static DescendParams dparams(pecc_ctx *c, int phase) {
   p.x64 = c->x64;
   p.xw = c->xw; p.xb = c->xb; p.xo = c->xo;
   p.g = c->g; p.gt = c->gt; p.d = c->d;
-  p.S = c->S; p.Y = c->Y;
+  p.S = c->S;
   p.perm = c->perm;
   p.skey = c->skey;
   p.rp = c->rp; p.col = c->col;

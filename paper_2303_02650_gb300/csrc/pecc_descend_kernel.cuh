@@ -41,14 +41,23 @@ namespace {
 
 constexpr int KS = kMaxSlots;     // basis index of Y slot a is KS + a
 constexpr int GI = 2 * kMaxSlots; // basis index of g
-// The dots of the first reduction of a batch step come in chunks of 32 values, one chunk per four
-// physical slots a: in chunk a / 4, from 6 (a % 4): g's_a, g'y_a, s's_a, s'y_a, y's_a, y'y_a, where
-// (s, y) is the pending pair; chunk 0 also carries g'g, s's, s'y and y'y at 24..27.
-constexpr int kSlotsPerChunk = 4;
+// The dots of the first reduction of a batch step come in chunks of 32 values, one chunk per seven
+// physical slots a: in chunk a / 7, from 4 (a % 7): g's_a, g'y_a, y's_a, y'y_a, where (s, y) is the
+// pending pair; chunk 0 also carries g'g, s's, s'y and y'y at 28..31.  The two-loop on the Gram
+// matrix reads an s only against the y's of its own or a newer pair, and no s against another s, so
+// s's_a and s'y_a are not taken: four values per slot instead of six put the six slots of m = 5 in
+// one chunk (one pass over the slots and one reduce-scatter instead of two), the eleven of m = 10
+// in two instead of three.
+constexpr int kSlotsPerChunk = 7;
 constexpr int kChunks = (kMaxSlots + kSlotsPerChunk - 1) / kSlotsPerChunk;
 constexpr int kPA = 32 * kChunks;  // per-warp partial values of the first reduction
-constexpr int PA_GG = 24, PA_SS = 25, PA_SY = 26, PA_YY = 27;
-__device__ __forceinline__ int pa_idx(int a, int kind) { return 32 * (a >> 2) + 6 * (a & 3) + kind; }
+constexpr int PA_GG = 28, PA_SS = 29, PA_SY = 30, PA_YY = 31;
+__device__ __forceinline__ int pa_idx(int a, int kind) {
+  return 32 * (a / kSlotsPerChunk) + 4 * (a % kSlotsPerChunk) + kind;
+}
+// Gram matrix of a batch: s_a'y_b at a KS + b (a not newer than b), then y_a'y_b at KS KS + a KS + b.
+constexpr int kGram = 2 * KS * KS;
+constexpr int kYY = KS * KS;
 constexpr int kRingInts = kMaxSlots + 3;  // count, stage, ring[kMaxSlots], pending
 
 __device__ __forceinline__ uint64_t sortable(double v) {
@@ -76,6 +85,10 @@ template <class A, int W> struct Smem {
   acc_t eA;                    // batch energy of that reduction
   vec_t coef[kBasis];
   unsigned long long hash;
+  // the list builds' scratch (kept here, not in registers: the batch steps never touch it)
+  int32_t *corder, *cells;
+  uint32_t *ckey;
+  typename V2<typename A::pos_t>::type *xs;
   unsigned used;               // physical slots in the current batch's ring (bit mask)
   int32_t sh[40];
   int q;
@@ -133,6 +146,29 @@ __device__ __forceinline__ void row_terms(const PP xi, const uint16_t *__restric
     }
   }
 }
+
+__host__ __device__ inline size_t round16(size_t b) { return (b + 15) & ~size_t(15); }
+
+// Bytes of the room that a batch step's arrays (g, direction, trial gradient of the largest batch,
+// `vec` bytes per circle; the step's start, `pos` bytes) share with the list builds' scratch, k > 1.
+__host__ __device__ inline size_t batch_room(int n, int k, size_t vec, size_t pos) {
+  const size_t nbm = (size_t)(n + k - 1) / k;
+  const size_t step = 3 * round16(nbm * vec) + nbm * pos, build = round16(8 * (size_t)n) + (size_t)n * pos;
+  return step > build ? step : build;
+}
+
+// One secant pair of one circle: s and y side by side, one 16-byte access in binary32 (two in
+// binary64) where separate arrays took two.
+template <typename T> struct alignas(16) SecantPair { v2<T> s, y; };
+__device__ __forceinline__ SecantPair<float> ld_pair(const SecantPair<float> *p) {
+  const float4 v = *(const float4 *)p;
+  return SecantPair<float>{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ SecantPair<double> ld_pair(const SecantPair<double> *p) { return *p; }
+__device__ __forceinline__ void st_pair(SecantPair<float> *p, float2 s, float2 y) {
+  *(float4 *)p = make_float4(s.x, s.y, y.x, y.y);
+}
+__device__ __forceinline__ void st_pair(SecantPair<double> *p, double2 s, double2 y) { p->s = s; p->y = y; }
 
 // Bump allocator over dynamic shared memory; returns the fallback when the request does not fit.
 struct Carve {
@@ -214,40 +250,75 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
     __syncthreads();
     return;
   }
-  vec_t *gram = cv.take<vec_t>((size_t)k * kBasis * kBasis, (vec_t *)P.gram + D.gram_off);
+  vec_t *gram = cv.take<vec_t>((size_t)k * kGram, (vec_t *)P.gram + D.gram_off);
   PP *xw = cv.take<PP>(n, (PP *)((double2 *)P.xw + D.off));
   int32_t *rp = cv.take<int32_t>(n + 1, P.rp + D.rp_off);
-  // two-level lists: the rows of the filtered lists start where the outer list's rows start and
-  // end at re[p]; with one level re = rp + 1 (CSR)
+  // row p of the lists: rl[p] entries from rp[p] on.  With two levels the rows of the filtered
+  // lists start where the outer list's rows start.
   bool two = P.list_outer > 0.0;
-  int32_t *re = two ? cv.take<int32_t>(n, P.rp + D.rp_off + n + 1) : rp + 1;
+  uint16_t *rl = cv.take<uint16_t>(n, (uint16_t *)(P.rp + D.rp_off + n + 1));
   // neighbor indices are 16-bit inside the descent (instances of at most 65535 circles)
   const int cap_s = min(D.cap, 8 * n + 64);  // about 5 neighbors per circle in practice
   uint16_t *col_s = cv.take<uint16_t>(cap_s, (uint16_t *)nullptr);
   uint16_t *const col_g = (uint16_t *)(P.col + D.col_off);  // 2 cap int32 = 4 cap uint16
   uint16_t *col = col_s ? col_s : col_g;
   int cap = col_s ? cap_s : D.cap;
-  VV *g = cv.take<VV>(n, (VV *)((double2 *)P.g + D.off));
-  VV *dv = cv.take<VV>(n, (VV *)((double2 *)P.d + D.off));
-  VV *gt = cv.take<VV>(n, (VV *)((double2 *)P.gt + D.off));
-  PP *xo = cv.take<PP>(n, (PP *)((double2 *)P.xo + D.off));
+  // g, the direction, the trial gradient and the step's start belong to one batch step (indexed from
+  // the batch's first circle), so with k > 1 they take the room of the largest batch only.  The list
+  // builds' scratch (circles in cell order, their cell keys, coordinates in cell order) shares that
+  // room: nothing of it is live while a build runs, except that one-batch steps (k = 1) carry a
+  // gradient across the build at the end of a sweep, where the scratch keeps to the direction and
+  // the step's start.  At k = 2 this and the 16-bit row lengths bring the FP32 working set from
+  // 72 n to 54 n bytes: instances up to about 1000 circles are on chip at four blocks per SM (688
+  // before), and the outer list too up to about 690.
+  const int nbm = (n + k - 1) / k;
+  VV *g, *dv, *gt;
+  PP *xo, *xs;
+  int32_t *corder;
+  uint32_t *ckey;
+  if (k == 1) {
+    g = cv.take<VV>(n, (VV *)((double2 *)P.g + D.off));
+    dv = cv.take<VV>(n, (VV *)((double2 *)P.d + D.off));
+    gt = cv.take<VV>(n, (VV *)((double2 *)P.gt + D.off));
+    xo = cv.take<PP>(n, (PP *)((double2 *)P.xo + D.off));
+    corder = (int32_t *)dv;
+    ckey = (uint32_t *)dv + n;
+    xs = xo;
+  } else {
+    unsigned char *room = cv.take<unsigned char>(batch_room(n, k, sizeof(VV), sizeof(PP)), (unsigned char *)nullptr);
+    if (room) {
+      const size_t vb = round16(nbm * sizeof(VV));
+      g = (VV *)room;
+      dv = (VV *)(room + vb);
+      gt = (VV *)(room + 2 * vb);
+      xo = (PP *)(room + 3 * vb);
+      corder = (int32_t *)room;
+      ckey = (uint32_t *)room + n;
+      xs = (PP *)(room + round16(8 * (size_t)n));
+    } else {
+      g = cv.take<VV>(nbm, (VV *)((double2 *)P.g + D.off));
+      dv = cv.take<VV>(nbm, (VV *)((double2 *)P.d + D.off));
+      gt = cv.take<VV>(nbm, (VV *)((double2 *)P.gt + D.off));
+      PP *const xo_g = (PP *)((double2 *)P.xo + D.off);
+      xo = cv.take<PP>(nbm, xo_g);
+      corder = P.corder + D.off;
+      ckey = P.ckey + D.off;
+      xs = xo_g;
+    }
+  }
   PP *xb = cv.take<PP>(n, (PP *)((double2 *)P.xb + D.off));
   const CellGrid G = (A::kId == 1) ? CellGrid{D.R, D.inv_cs, (float)D.R, D.inv_f, D.ncx_f, true}
                                    : CellGrid{D.R, D.inv_cs, 0.f, 0.f, D.ncx, false};
-  // The list builds' scratch lives in arrays that are dead while a build runs: the circles in
-  // cell order and their cell keys in the direction (8 n bytes at least), the cell table in the
-  // positions at the last build when it fits (they are rewritten right after every build).  The
-  // gradient arrays cannot serve: one-batch steps swap g and gt and carry a gradient across the
-  // build at the end of a sweep.
-  int32_t *corder = (int32_t *)dv;
-  uint32_t *ckey = (uint32_t *)dv + n;
+  // the builds' cell table lives in the positions at the last build when it fits (they are
+  // rewritten right after every build)
   const size_t ncells = 2 * (size_t)G.nc * G.nc + 2;
   int32_t *cells = (ncells * sizeof(int32_t) <= (size_t)n * sizeof(PP)) ? (int32_t *)xb
                                                                        : cv.take<int32_t>(ncells, P.cells + D.cell_off);
+  if (tid == 0) { S.corder = corder; S.ckey = ckey; S.xs = xs; S.cells = cells; }
   // the secant pairs last: on chip when the block's share holds them (few instances per launch, a
   // block alone on its SM), else in global memory; they carry nothing between descent calls
-  VV *Sv = cv.take<VV>((size_t)mm * n, (VV *)P.S + (int64_t)mm * D.off);
-  VV *Yv = cv.take<VV>((size_t)mm * n, (VV *)P.Y + (int64_t)mm * D.off);
+  using SP = SecantPair<vec_t>;
+  SP *SY = cv.take<SP>((size_t)mm * n, (SP *)P.S + (int64_t)mm * D.off);
   // the outer list last: its rows are read once per filtered rebuild
   uint16_t *const colL_g = col_g + 2 * (size_t)D.cap;
   uint16_t *colL_s = nullptr, *colL = nullptr;
@@ -272,7 +343,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
       GL = CellGrid{D.R, inv, 0.f, 0.f, nc, false};
     }
     lc2L = (pos_t)(lb * lb);
-    if (GL.nc > G.nc) { two = false; re = rp + 1; }  // its cell table must fit the scratch
+    if (GL.nc > G.nc) two = false;  // its cell table must fit the scratch
   }
   int32_t *perm = P.perm + D.off;
   // the partition keys borrow the list storage (8 n bytes) before the first build
@@ -322,12 +393,12 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
   // the outer list at the current layout (rows rp, entries colL); the filtered lists take the
   // same room, so they move to global memory with it when it outgrows their share
   auto build_outer = [&]() -> bool {
-    int tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, GL, lc2L, ckey, corder, cells, xo, rp, colL, capL, S.sh,
+    int tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, GL, lc2L, S.ckey, S.corder, S.cells, S.xs, rp, colL, capL, S.sh,
                                                    nullptr, false);
     if (tot > capL && colL_s && colL == colL_s) {
       colL = colL_g;
       capL = D.cap;
-      tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, GL, lc2L, ckey, corder, cells, xo, rp, colL, capL, S.sh,
+      tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, GL, lc2L, S.ckey, S.corder, S.cells, S.xs, rp, colL, capL, S.sh,
                                                  nullptr, false);
     }
     if (tot > capL) return false;
@@ -360,7 +431,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
           }
         }
       }
-      re[p] = w;
+      rl[p] = (uint16_t)(w - rp[p]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
@@ -382,19 +453,22 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
       } else {
         outer_ok = build_outer();
         DL = 0;
-        if (!outer_ok) { two = false; re = rp + 1; }  // one level from here on
+        if (!outer_ok) two = false;  // one level from here on
       }
       if (two) { filter(); return true; }
     }
-    int tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, G, lc2, ckey, corder, cells, xo, rp, col, cap, S.sh,
+    int tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, G, lc2, S.ckey, S.corder, S.cells, S.xs, rp, col, cap, S.sh,
                                                    &S.hash, false);
     if (tot > cap && col_s && col == col_s) {
       col = col_g;
       cap = D.cap;
-      tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, G, lc2, ckey, corder, cells, xo, rp, col, cap, S.sh,
+      tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, G, lc2, S.ckey, S.corder, S.cells, S.xs, rp, col, cap, S.sh,
                                                  &S.hash, false);
     }
-    return tot <= cap;
+    if (tot > cap) return false;
+    for (int p = tid; p < n; p += T) rl[p] = (uint16_t)(rp[p + 1] - rp[p]);
+    __syncthreads();
+    return true;
   };
   // ANM step (Algorithm ANM): Gamma' replaces Gamma; equal sets double the deferral length
   auto anm_rebuild = [&]() -> bool {
@@ -417,7 +491,8 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
       PP xi = xw[p];
       acc_t e = 0;
       vec_t ux = 0, uy = 0;  // unused
-      row_terms<A, PP>(xi, col, rp[p], re[p], xw, 0, n, p, ux, uy, e);
+      const int t0 = rp[p];
+      row_terms<A, PP>(xi, col, t0, t0 + rl[p], xw, 0, n, p, ux, uy, e);
       vec_t fx, fy;
       acc_t d0 = A::wall(xi, R, Rm1sq, fx, fy);
       a += e + d0 * d0;
@@ -441,7 +516,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
     }
   }
   for (int u = tid; u < k * kRingInts; u += T) rings[u] = 0;
-  for (int u = tid; u < k * kBasis * kBasis; u += T) gram[u] = vec_t(0);
+  for (int u = tid; u < k * kGram; u += T) gram[u] = vec_t(0);
   __syncthreads();
 
   const int q_ = n / k, r_ = n % k;
@@ -462,72 +537,100 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
         fresh = false;
       }
       int *ring = rings + p * kRingInts;  // [0] count, [1] stage, [2..] slots, [2 + KS] pending
-      vec_t *Gm = gram + (size_t)p * kBasis * kBasis;
+      vec_t *Gm = gram + (size_t)p * kGram;
       const int count0 = ring[0], st = ring[1], pending = ring[2 + kMaxSlots];
 
       // ---- pass A: batch energy (Eq. 7) and gradient, then the dots of g and of the pair (s, y)
-      // written by this batch's previous step with every stored vector (the pair's curvature is
-      // tested here).  The pair is staged in the direction and trial-gradient arrays (both free
-      // until pass B and pass D), and the dots are taken four slots at a time, each chunk of 32
-      // values reduce-scattered over the warp: few live accumulators, many loads in flight.
+      // written by this batch's previous step with the stored vectors (the pair's curvature is tested
+      // here): one walk over the batch for the first seven slots, a second one for the slots beyond
+      // (m > 6).  The values of a chunk are reduce-scattered over the warp.  Dots in the walk of the
+      // gradient itself cost registers: 215.1 ms per 4096-instance batch against 211.2 (spills).
       if (fresh) { VV *t_ = g; g = gt; gt = t_; }
-      acc_t aA = 0;
-      vec_t xgg = 0, xss = 0, xsy = 0, xyy = 0;
-      for (int pos = b + tid; pos < e; pos += T) {
-        PP xi = xw[pos];
-        xo[pos] = xi;
-        VV gi;
-        if (!fresh) {
-          vec_t gx = 0, gy = 0;
-          acc_t ei = 0;
-          row_terms<A, PP>(xi, col, rp[pos], re[pos], xw, b, e, pos, gx, gy, ei);
-          vec_t fx, fy;
-          acc_t d0 = A::wall(xi, R, Rm1sq, fx, fy);
-          gx += fx; gy += fy;
-          aA += ei + d0 * d0;
-          gi.x = gx; gi.y = gy;
-          g[pos] = gi;
-        } else {
-          gi = g[pos];
-        }
-        xgg += gi.x * gi.x + gi.y * gi.y;
-        if (pending) {
-          const VV sp = Sv[(int64_t)st * n + pos], yp = Yv[(int64_t)st * n + pos];
-          dv[pos] = sp;
-          gt[pos] = yp;
-          xss += sp.x * sp.x + sp.y * sp.y;
-          xsy += sp.x * yp.x + sp.y * yp.y;
-          xyy += yp.x * yp.x + yp.y * yp.y;
-        }
-      }
+      const int nb = e - b;
       const int nch = (mm + kSlotsPerChunk - 1) / kSlotsPerChunk;
-      for (int c = 0; c < nch; ++c) {
+      acc_t aA = 0;
+      {
+        vec_t xgg = 0;
+        for (int i = tid; i < nb; i += T) {
+          const int pos = b + i;
+          PP xi = xw[pos];
+          xo[i] = xi;
+          VV gi;
+          if (!fresh) {
+            vec_t gx = 0, gy = 0;
+            acc_t ei = 0;
+            const int t0 = rp[pos];
+            row_terms<A, PP>(xi, col, t0, t0 + rl[pos], xw, b, e, pos, gx, gy, ei);
+            vec_t fx, fy;
+            acc_t d0 = A::wall(xi, R, Rm1sq, fx, fy);
+            gx += fx; gy += fy;
+            aA += ei + d0 * d0;
+            gi.x = gx; gi.y = gy;
+            g[i] = gi;
+          } else {
+            gi = g[i];
+          }
+          xgg += gi.x * gi.x + gi.y * gi.y;
+        }
         vec_t v[32];
 #pragma unroll
         for (int u = 0; u < 32; ++u) v[u] = 0;
-        if (c == 0) { v[PA_GG] = xgg; v[PA_SS] = xss; v[PA_SY] = xsy; v[PA_YY] = xyy; }
-        for (int pos = b + tid; pos < e; pos += T) {
-          const VV gi = g[pos];
-          VV sp{}, yp{};
-          if (pending) { sp = dv[pos]; yp = gt[pos]; }
+        v[PA_GG] = xgg;
+        for (int i = tid; i < nb; i += T) {
+          const int pos = b + i;
+          const VV gi = g[i];
+          VV yp{};
+          if (pending) {
+            const SP pp = ld_pair(SY + st * n + pos);
+            const VV sp = pp.s;
+            yp = pp.y;
+            v[PA_SS] += sp.x * sp.x + sp.y * sp.y;
+            v[PA_SY] += sp.x * yp.x + sp.y * yp.y;
+            v[PA_YY] += yp.x * yp.x + yp.y * yp.y;
+          }
 #pragma unroll
-          for (int j = 0; j < kSlotsPerChunk; ++j) {
-            const int a = c * kSlotsPerChunk + j;
+          for (int a = 0; a < kSlotsPerChunk; ++a) {
             if (a < mm) {
-              const VV s_ = Sv[(int64_t)a * n + pos], y_ = Yv[(int64_t)a * n + pos];
-              v[6 * j + 0] += gi.x * s_.x + gi.y * s_.y;
-              v[6 * j + 1] += gi.x * y_.x + gi.y * y_.y;
+              const SP pr = ld_pair(SY + a * n + pos);
+              const VV s_ = pr.s, y_ = pr.y;
+              v[4 * a + 0] += gi.x * s_.x + gi.y * s_.y;
+              v[4 * a + 1] += gi.x * y_.x + gi.y * y_.y;
               if (pending) {
-                v[6 * j + 2] += sp.x * s_.x + sp.y * s_.y;
-                v[6 * j + 3] += sp.x * y_.x + sp.y * y_.y;
-                v[6 * j + 4] += yp.x * s_.x + yp.y * s_.y;
-                v[6 * j + 5] += yp.x * y_.x + yp.y * y_.y;
+                v[4 * a + 2] += yp.x * s_.x + yp.y * s_.y;
+                v[4 * a + 3] += yp.x * y_.x + yp.y * y_.y;
               }
             }
           }
         }
         warp_reduce_scatter<vec_t, 32>(v);
-        pa[warp * kPA + c * 32 + lane] = v[0];
+        pa[warp * kPA + lane] = v[0];
+      }
+      if (nch > 1) {
+        vec_t v[32];
+#pragma unroll
+        for (int u = 0; u < 32; ++u) v[u] = 0;
+        for (int i = tid; i < nb; i += T) {
+          const int pos = b + i;
+          const VV gi = g[i];
+          VV yp{};
+          if (pending) yp = ld_pair(SY + st * n + pos).y;
+#pragma unroll
+          for (int j = 0; j < kMaxSlots - kSlotsPerChunk; ++j) {
+            const int a = kSlotsPerChunk + j;
+            if (a < mm) {
+              const SP pr = ld_pair(SY + a * n + pos);
+              const VV s_ = pr.s, y_ = pr.y;
+              v[4 * j + 0] += gi.x * s_.x + gi.y * s_.y;
+              v[4 * j + 1] += gi.x * y_.x + gi.y * y_.y;
+              if (pending) {
+                v[4 * j + 2] += yp.x * s_.x + yp.y * s_.y;
+                v[4 * j + 3] += yp.x * y_.x + yp.y * y_.y;
+              }
+            }
+          }
+        }
+        warp_reduce_scatter<vec_t, 32>(v);
+        pa[warp * kPA + 32 + lane] = v[0];
       }
       {
         const acc_t ws = warp_sum(aA);
@@ -560,15 +663,12 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
           if (push) {
             if (lane < count0) {
               const int sl = ring[2 + lane];
-              Gm[st * kBasis + sl] = Gm[sl * kBasis + st] = S.ob[pa_idx(sl, 2)];
-              Gm[st * kBasis + KS + sl] = Gm[(KS + sl) * kBasis + st] = S.ob[pa_idx(sl, 3)];
-              Gm[(KS + st) * kBasis + sl] = Gm[sl * kBasis + KS + st] = S.ob[pa_idx(sl, 4)];
-              Gm[(KS + st) * kBasis + KS + sl] = Gm[(KS + sl) * kBasis + KS + st] = S.ob[pa_idx(sl, 5)];
+              Gm[sl * KS + st] = S.ob[pa_idx(sl, 2)];
+              Gm[kYY + st * KS + sl] = Gm[kYY + sl * KS + st] = S.ob[pa_idx(sl, 3)];
             }
             if (lane == 0) {
-              Gm[st * kBasis + st] = ss;
-              Gm[st * kBasis + KS + st] = Gm[(KS + st) * kBasis + st] = sy;
-              Gm[(KS + st) * kBasis + KS + st] = yy;
+              Gm[st * KS + st] = sy;
+              Gm[kYY + st * KS + st] = yy;
             }
           }
           __syncwarp();
@@ -605,24 +705,24 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
         // Lane c holds row c; each substitution step is one broadcast.
         const bool act = lane < count;
         const int sl = act ? ring[2 + lane] : 0;
-        const vec_t rho = act ? vec_t(1) / Gm[sl * kBasis + KS + sl] : vec_t(0);
+        const vec_t rho = act ? vec_t(1) / Gm[sl * KS + sl] : vec_t(0);
         vec_t acc = act ? S.ob[pa_idx(sl, 0)] : vec_t(0);
         vec_t my_alpha = 0, my_w = 0, gam = 1;
         for (int cc = count - 1; cc >= 0; --cc) {
           const vec_t a = __shfl_sync(0xffffffffu, rho * acc, cc);
           if (lane == cc) my_alpha = a;
           const int slc = ring[2 + cc];
-          if (lane < cc) acc -= a * Gm[sl * kBasis + KS + slc];
+          if (lane < cc) acc -= a * Gm[sl * KS + slc];
         }
         if (count > 0) {
           const int nw_ = ring[2 + count - 1];
-          gam = Gm[nw_ * kBasis + KS + nw_] / Gm[(KS + nw_) * kBasis + KS + nw_];
+          gam = Gm[nw_ * KS + nw_] / Gm[kYY + nw_ * KS + nw_];
         }
         vec_t t = act ? S.ob[pa_idx(sl, 1)] : vec_t(0);
         for (int dd = 0; dd < count; ++dd) {
           const vec_t ad = __shfl_sync(0xffffffffu, my_alpha, dd);
           const int sld = ring[2 + dd];
-          if (act) t -= ad * Gm[(KS + sl) * kBasis + KS + sld];
+          if (act) t -= ad * Gm[kYY + sl * KS + sld];
         }
         vec_t acc2 = gam * t;
         for (int cc = 0; cc < count; ++cc) {
@@ -630,7 +730,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
           const vec_t w = __shfl_sync(0xffffffffu, my_alpha, cc) - bcc;
           if (lane == cc) my_w = w;
           const int slc = ring[2 + cc];
-          if (act && lane > cc) acc2 += w * Gm[slc * kBasis + KS + sl];
+          if (act && lane > cc) acc2 += w * Gm[slc * KS + sl];
         }
         if (act) {
           S.coef[sl] = -my_w;
@@ -672,19 +772,19 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
           const unsigned used = S.used;
           gdB = 0;
           dmB = 0;
-          for (int pos = b + tid; pos < e; pos += 2 * T) {
-            const int p2 = pos + T;
-            const bool h2 = p2 < e;
-            const int q2 = h2 ? p2 : pos;
-            const VV gi = g[pos], gi2 = g[q2];
+          for (int i = tid; i < nb; i += 2 * T) {
+            const int i2 = i + T;
+            const bool h2 = i2 < nb;
+            const int pos = b + i, q2 = h2 ? b + i2 : pos;
+            const VV gi = g[i], gi2 = g[h2 ? i2 : i];
             const vec_t cg = S.coef[GI];
             vec_t dx = cg * gi.x, dy = cg * gi.y;
             vec_t dx2 = cg * gi2.x, dy2 = cg * gi2.y;
 #pragma unroll
             for (int a = 0; a < kMaxSlots; ++a) {
               if (a < mm && ((used >> a) & 1u)) {
-                const VV s_ = Sv[(int64_t)a * n + pos], y_ = Yv[(int64_t)a * n + pos];
-                const VV s2 = Sv[(int64_t)a * n + q2], y2 = Yv[(int64_t)a * n + q2];
+                const SP p1 = ld_pair(SY + a * n + pos), p2 = ld_pair(SY + a * n + q2);
+                const VV s_ = p1.s, y_ = p1.y, s2 = p2.s, y2 = p2.y;
                 const vec_t cs = S.coef[a], cy = S.coef[KS + a];
                 dx += cs * s_.x + cy * y_.x;
                 dy += cs * s_.y + cy * y_.y;
@@ -693,12 +793,12 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
               }
             }
             VV dd; dd.x = dx; dd.y = dy;
-            dv[pos] = dd;
+            dv[i] = dd;
             gdB += (acc_t)(gi.x * dx + gi.y * dy);
             dmB = max(dmB, dx * dx + dy * dy);
             if (h2) {
               VV d2; d2.x = dx2; d2.y = dy2;
-              dv[p2] = d2;
+              dv[i2] = d2;
               gdB += (acc_t)(gi2.x * dx2 + gi2.y * dy2);
               dmB = max(dmB, dx2 * dx2 + dy2 * dy2);
             }
@@ -717,29 +817,31 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
         sc_t al = (dmax > step_max) ? step_max / dmax : sc_t(1);
         for (int tr = 0; tr < P.max_trials; ++tr) {
           // ---- pass C: trial coordinates
-          for (int pos = b + tid; pos < e; pos += T) {
-            PP xo_ = xo[pos];
-            VV dd = dv[pos];
+          for (int i = tid; i < nb; i += T) {
+            PP xo_ = xo[i];
+            VV dd = dv[i];
             PP v;
             v.x = xo_.x + (pos_t)(al * (sc_t)dd.x);
             v.y = xo_.y + (pos_t)(al * (sc_t)dd.y);
-            xw[pos] = v;
+            xw[b + i] = v;
           }
           __syncthreads();
           // ---- pass D: trial batch energy and gradient, displacement since the build
           acc_t aD = 0;
           vec_t cD = 0;
-          for (int pos = b + tid; pos < e; pos += T) {
+          for (int i = tid; i < nb; i += T) {
+            const int pos = b + i;
             PP xi = xw[pos];
             vec_t gx = 0, gy = 0;
             acc_t ei = 0;
-            row_terms<A, PP>(xi, col, rp[pos], re[pos], xw, b, e, pos, gx, gy, ei);
+            const int t0 = rp[pos];
+            row_terms<A, PP>(xi, col, t0, t0 + rl[pos], xw, b, e, pos, gx, gy, ei);
             vec_t fx, fy;
             acc_t d0 = A::wall(xi, R, Rm1sq, fx, fy);
             gx += fx; gy += fy;
             aD += ei + d0 * d0;
             VV gg_; gg_.x = gx; gg_.y = gy;
-            gt[pos] = gg_;
+            gt[i] = gg_;
             PP x0 = xb[pos];
             vec_t ex = (vec_t)(xi.x - x0.x), ey = (vec_t)(xi.y - x0.y);
             cD = max(cD, ex * ex + ey * ey);
@@ -755,7 +857,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
           al *= sc_t(0.5);
         }
         if (!accepted) {
-          for (int pos = b + tid; pos < e; pos += T) xw[pos] = xo[pos];
+          for (int i = tid; i < nb; i += T) xw[b + i] = xo[i];
           __syncthreads();
         }
       }
@@ -767,13 +869,13 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
       // its dots and its curvature test come with this batch's next step
       {
         const int stg = ring[1];
-        for (int pos = b + tid; pos < e; pos += T) {
-          PP xn = xw[pos], x0 = xo[pos];
+        for (int i = tid; i < nb; i += T) {
+          const int pos = b + i;
+          PP xn = xw[pos], x0 = xo[i];
           VV s_; s_.x = (vec_t)(xn.x - x0.x); s_.y = (vec_t)(xn.y - x0.y);
-          VV gn = gt[pos], go = g[pos];
+          VV gn = gt[i], go = g[i];
           VV y_; y_.x = gn.x - go.x; y_.y = gn.y - go.y;
-          Sv[(int64_t)stg * n + pos] = s_;
-          Yv[(int64_t)stg * n + pos] = y_;
+          st_pair(SY + stg * n + pos, s_, y_);
         }
         // every thread raises the flag: with one batch the next read comes without a barrier in
         // between, and each thread then reads its own store (thread 0 clears the flag only after
@@ -820,7 +922,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
     const int64_t stride = P.dump_stride;
     for (int pos = tid; pos < n; pos += T) {
       const int i = perm[pos];
-      const int b0 = lists_ok ? rp[pos] : 0, len_ = lists_ok ? re[pos] - b0 : 0;
+      const int b0 = lists_ok ? rp[pos] : 0, len_ = lists_ok ? (int)rl[pos] : 0;
       const bool ok = lists_ok && len_ <= P.dump_stride;
       P.dump_cnt[D.off + i] = ok ? len_ : -1;
       if (ok)
@@ -881,13 +983,16 @@ template <int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
 descend_fused_kernel(DescendParams P32, DescendParams P64) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  __shared__ Smem<Arith32, MAXT / 32> S32;
-  __shared__ Smem<ArithMix, MAXT / 32> S64;
+  // the two phases' block states are never live together
+  __shared__ union { double align_; unsigned char a[sizeof(Smem<Arith32, MAXT / 32>)], b[sizeof(Smem<ArithMix, MAXT / 32>)]; } U;
+  __shared__ int next;
+  Smem<Arith32, MAXT / 32> &S32 = *(Smem<Arith32, MAXT / 32> *)U.a;
+  Smem<ArithMix, MAXT / 32> &S64 = *(Smem<ArithMix, MAXT / 32> *)U.b;
   const int num = P32.num_dev ? *P32.num_dev : P32.num;
   for (;;) {
-    if (threadIdx.x == 0) S32.q = atomicAdd(P32.queue, 1);
+    if (threadIdx.x == 0) next = atomicAdd(P32.queue, 1);
     __syncthreads();
-    const int qi = S32.q;
+    const int qi = next;
     __syncthreads();
     if (qi >= num) break;
     const int q = P32.order[qi];
@@ -903,7 +1008,7 @@ template <class A, int MAXT, int MINB> DescendVariant descend_variant() {
 }
 template <int MAXT, int MINB> DescendVariant descend_fused_variant() {
   return DescendVariant{(const void *)descend_fused_kernel<MAXT, MINB>, MAXT, MINB,
-                        sizeof(Smem<Arith32, MAXT / 32>) + sizeof(Smem<ArithMix, MAXT / 32>)};
+                        std::max(sizeof(Smem<Arith32, MAXT / 32>), sizeof(Smem<ArithMix, MAXT / 32>)) + 16};
 }
 
 }  // namespace

@@ -68,7 +68,7 @@ struct DescendParams {
   double2 *x64;
   void *xw, *xb, *xo;    // per-circle positions scratch (sized for double2)
   void *g, *gt, *d;      // per-circle vectors (sized for double2)
-  void *S, *Y;           // (m + 1) secant slots per circle
+  void *S;               // (m + 1) secant slots (s and y) per circle; instance q's from 2 (m + 1) off_q vectors on
   int32_t *perm;
   uint64_t *skey;
   int32_t *rp, *col;
