@@ -41,17 +41,17 @@ namespace {
 
 constexpr int KS = kMaxSlots;     // basis index of Y slot a is KS + a
 constexpr int GI = 2 * kMaxSlots; // basis index of g
-// The dots of the first reduction of a batch step come in chunks of 32 values, one chunk per seven
-// physical slots a: in chunk a / 7, from 4 (a % 7): g's_a, g'y_a, y's_a, y'y_a, where (s, y) is the
-// pending pair; chunk 0 also carries g'g, s's, s'y and y'y at 28..31.  The two-loop on the Gram
+// The dots of the first reduction of a batch step come in chunks of 32 values, one chunk per six
+// physical slots a: in chunk a / 6, from 4 (a % 6): g's_a, g'y_a, y's_a, y'y_a, where (s, y) is the
+// pending pair; chunk 0 also carries g'g, s's, s'y and y'y at 24..27.  The two-loop on the Gram
 // matrix reads an s only against the y's of its own or a newer pair, and no s against another s, so
 // s's_a and s'y_a are not taken: four values per slot instead of six put the six slots of m = 5 in
 // one chunk (one pass over the slots and one reduce-scatter instead of two), the eleven of m = 10
 // in two instead of three.
-constexpr int kSlotsPerChunk = 7;
+constexpr int kSlotsPerChunk = 6;
 constexpr int kChunks = (kMaxSlots + kSlotsPerChunk - 1) / kSlotsPerChunk;
 constexpr int kPA = 32 * kChunks;  // per-warp partial values of the first reduction
-constexpr int PA_GG = 28, PA_SS = 29, PA_SY = 30, PA_YY = 31;
+constexpr int PA_GG = 24, PA_SS = 25, PA_SY = 26, PA_YY = 27;
 __device__ __forceinline__ int pa_idx(int a, int kind) {
   return 32 * (a / kSlotsPerChunk) + 4 * (a % kSlotsPerChunk) + kind;
 }
@@ -169,6 +169,18 @@ __device__ __forceinline__ void st_pair(SecantPair<float> *p, float2 s, float2 y
   *(float4 *)p = make_float4(s.x, s.y, y.x, y.y);
 }
 __device__ __forceinline__ void st_pair(SecantPair<double> *p, double2 s, double2 y) { p->s = s; p->y = y; }
+
+// The pairs of circle pos in the physical slots [A0, A0 + N), of mm in all.  Every load is issued
+// whether its slot is in use or not (its value is then ignored; a slot past the last is read as slot
+// 0), so that all of them are in flight together: behind a test of its own each slot waited for its
+// own L2 round trip (the 4096-instance batch at m = 5: 210.5 ms, with the groups 191.2).  Six slots
+// per group, those of m = 5, and one circle per thread at a time: seven slots, or two circles, take
+// registers the kernel does not have (196.0 and 192.6 ms, and a single instance gets slower).
+template <int A0, int N, typename T>
+__device__ __forceinline__ void load_slots(const SecantPair<T> *SY, int mm, int n, int pos, SecantPair<T> *pr) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) pr[j] = ld_pair(SY + (A0 + j < mm ? A0 + j : 0) * n + pos);
+}
 
 // Bump allocator over dynamic shared memory; returns the fallback when the request does not fit.
 struct Carve {
@@ -542,8 +554,8 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
 
       // ---- pass A: batch energy (Eq. 7) and gradient, then the dots of g and of the pair (s, y)
       // written by this batch's previous step with the stored vectors (the pair's curvature is tested
-      // here): one walk over the batch for the first seven slots, a second one for the slots beyond
-      // (m > 6).  The values of a chunk are reduce-scattered over the warp.  Dots in the walk of the
+      // here): one walk over the batch for the first six slots, a second one for the slots beyond
+      // (m > 5).  The values of a chunk are reduce-scattered over the warp.  Dots in the walk of the
       // gradient itself cost registers: 215.1 ms per 4096-instance batch against 211.2 (spills).
       if (fresh) { VV *t_ = g; g = gt; gt = t_; }
       const int nb = e - b;
@@ -578,6 +590,8 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
         v[PA_GG] = xgg;
         for (int i = tid; i < nb; i += T) {
           const int pos = b + i;
+          SP pr[kSlotsPerChunk];
+          load_slots<0, kSlotsPerChunk>(SY, mm, n, pos, pr);
           const VV gi = g[i];
           VV yp{};
           if (pending) {
@@ -591,8 +605,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
 #pragma unroll
           for (int a = 0; a < kSlotsPerChunk; ++a) {
             if (a < mm) {
-              const SP pr = ld_pair(SY + a * n + pos);
-              const VV s_ = pr.s, y_ = pr.y;
+              const VV s_ = pr[a].s, y_ = pr[a].y;
               v[4 * a + 0] += gi.x * s_.x + gi.y * s_.y;
               v[4 * a + 1] += gi.x * y_.x + gi.y * y_.y;
               if (pending) {
@@ -611,6 +624,8 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
         for (int u = 0; u < 32; ++u) v[u] = 0;
         for (int i = tid; i < nb; i += T) {
           const int pos = b + i;
+          SP pr[kMaxSlots - kSlotsPerChunk];
+          load_slots<kSlotsPerChunk, kMaxSlots - kSlotsPerChunk>(SY, mm, n, pos, pr);
           const VV gi = g[i];
           VV yp{};
           if (pending) yp = ld_pair(SY + st * n + pos).y;
@@ -618,8 +633,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
           for (int j = 0; j < kMaxSlots - kSlotsPerChunk; ++j) {
             const int a = kSlotsPerChunk + j;
             if (a < mm) {
-              const SP pr = ld_pair(SY + a * n + pos);
-              const VV s_ = pr.s, y_ = pr.y;
+              const VV s_ = pr[j].s, y_ = pr[j].y;
               v[4 * j + 0] += gi.x * s_.x + gi.y * s_.y;
               v[4 * j + 1] += gi.x * y_.x + gi.y * y_.y;
               if (pending) {
@@ -763,45 +777,37 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
           for (int u = tid; u < kBasis; u += T) S.coef[u] = (u == GI) ? vec_t(-1) : vec_t(0);
           __syncthreads();
         }
-        // ---- pass B: direction, g'd and the largest per-circle move.  Two positions per thread at a
-        // time, so that the secant-slot loads of both are in flight together; g'd takes the positions
-        // in the same order as one at a time.
+        // ---- pass B: direction, g'd and the largest per-circle move
         acc_t gdB = 0;
         vec_t dmB = 0;
         for (int round = 0; round < 2; ++round) {
           const unsigned used = S.used;
           gdB = 0;
           dmB = 0;
-          for (int i = tid; i < nb; i += 2 * T) {
-            const int i2 = i + T;
-            const bool h2 = i2 < nb;
-            const int pos = b + i, q2 = h2 ? b + i2 : pos;
-            const VV gi = g[i], gi2 = g[h2 ? i2 : i];
+          for (int i = tid; i < nb; i += T) {
+            const int pos = b + i;
+            SP pr[kSlotsPerChunk];
+            load_slots<0, kSlotsPerChunk>(SY, mm, n, pos, pr);
+            const VV gi = g[i];
             const vec_t cg = S.coef[GI];
             vec_t dx = cg * gi.x, dy = cg * gi.y;
-            vec_t dx2 = cg * gi2.x, dy2 = cg * gi2.y;
 #pragma unroll
             for (int a = 0; a < kMaxSlots; ++a) {
+              if (a == kSlotsPerChunk) {
+                if (mm <= kSlotsPerChunk) break;
+                load_slots<kSlotsPerChunk, kMaxSlots - kSlotsPerChunk>(SY, mm, n, pos, pr);
+              }
               if (a < mm && ((used >> a) & 1u)) {
-                const SP p1 = ld_pair(SY + a * n + pos), p2 = ld_pair(SY + a * n + q2);
-                const VV s_ = p1.s, y_ = p1.y, s2 = p2.s, y2 = p2.y;
+                const VV s_ = pr[a % kSlotsPerChunk].s, y_ = pr[a % kSlotsPerChunk].y;
                 const vec_t cs = S.coef[a], cy = S.coef[KS + a];
                 dx += cs * s_.x + cy * y_.x;
                 dy += cs * s_.y + cy * y_.y;
-                dx2 += cs * s2.x + cy * y2.x;
-                dy2 += cs * s2.y + cy * y2.y;
               }
             }
             VV dd; dd.x = dx; dd.y = dy;
             dv[i] = dd;
             gdB += (acc_t)(gi.x * dx + gi.y * dy);
             dmB = max(dmB, dx * dx + dy * dy);
-            if (h2) {
-              VV d2; d2.x = dx2; d2.y = dy2;
-              dv[i2] = d2;
-              gdB += (acc_t)(gi2.x * dx2 + gi2.y * dy2);
-              dmB = max(dmB, dx2 * dx2 + dy2 * dy2);
-            }
           }
           reduce_sm<A, W>(S, rbuf, gdB, dmB);
           if (gdB < acc_t(0) || round == 1) break;
