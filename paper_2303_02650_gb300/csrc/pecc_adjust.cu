@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
     // list build with ANM bookkeeping; false on a capacity overflow
     auto rebuild = [&](bool anm) -> bool {
       const int tot = cta_build_neighbors<double, int32_t>(x, n, G, lc2, ckey, corder, cells, xs, rp, col, cap, S.sh,
-                                                          &S.hash, false);
+                                                          &S.hash);
       if (tot > cap) return false;
       if (anm) {
         const unsigned long long h = S.hash;

@@ -49,7 +49,9 @@ struct pecc_ctx {
   bool radius_host_known = false;  // radius_host holds the radii of the last pecc_solve_host
   std::vector<double> radius_host;
   int lists_prec = -1;  // precision of the standalone lists: 0 FP64, 1 FP32
-  int block = 0, bps = 0, grid = 0, block_build = 256;
+  int block = 0, bps = 0, grid = 0;
+  LargeTiles lt{};   // tiles of the instances past kCellsBlockN circles (standalone kernels)
+  int n_small = -1;  // the largest instance that is not one of them
   // per arithmetic (0 FP64, 1 FP32, 2 polish) and 3 = FP32 descent + polish fused in one kernel
   struct Launch { int block = 0, bps = 0, grid = 0, var = 0; size_t smem = 0; } lc[4];
   bool lc_ready = false;
@@ -325,6 +327,42 @@ pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
     ctx->gb.kmax = kmax;
     ALC(ctx->gctl, GridCtl, 1);
   }
+  // tiles of the instances the standalone kernels give several blocks
+  std::vector<int2> row_tiles, cell_tiles;
+  for (int q = 0; q < ctx->num; ++q) {
+    const int n = ctx->n[q];
+    if (n <= kCellsBlockN) {
+      ctx->n_small = std::max(ctx->n_small, n);
+      continue;
+    }
+    const int64_t cap_c = cell_grid_cap(n), nct = (cap_c * cap_c + kTileCells - 1) / kTileCells;
+    for (int t = 0; t < (n + kTileRows - 1) / kTileRows; ++t) row_tiles.push_back(make_int2(q, t));
+    for (int64_t t = 0; t < nct; ++t) cell_tiles.push_back(make_int2(q, (int)t));
+  }
+  if (!row_tiles.empty()) {
+    LargeTiles &L = ctx->lt;
+    L.nrows = (int)row_tiles.size();
+    L.ncells = (int)cell_tiles.size();
+    int2 *rt = nullptr, *ct = nullptr;
+    ALC(rt, int2, row_tiles.size());
+    ALC(ct, int2, cell_tiles.size());
+    ALC(L.row_total, int32_t, row_tiles.size());
+    ALC(L.cell_total, int32_t, cell_tiles.size());
+    ALC(L.go, int32_t, ctx->num);
+    ALC(L.hits, unsigned long long, ctx->num);
+    ALC(L.smin, unsigned long long, ctx->num);
+    ALC(L.rmax, unsigned long long, ctx->num);
+    ALC(L.smin32, uint32_t, ctx->num);
+    ALC(L.rmax32, uint32_t, ctx->num);
+    ALC(L.bad, int32_t, ctx->num);
+    L.rows = rt;
+    L.cells = ct;
+    L.rank = ctx->perm;             // the descent's scratch, free between its calls
+    L.tmp = (int32_t *)ctx->skey;
+    if (cudaMemcpy(rt, row_tiles.data(), sizeof(int2) * row_tiles.size(), cudaMemcpyHostToDevice) ||
+        cudaMemcpy(ct, cell_tiles.data(), sizeof(int2) * cell_tiles.size(), cudaMemcpyHostToDevice))
+      return bail(fail(ctx, PECC_ERR_CUDA, "upload tiles"));
+  }
 #undef ALC
   // instance of every circle, processing order (largest first)
   std::vector<int32_t> inst_of(total);
@@ -437,7 +475,7 @@ pecc_status pecc_rebuild_neighbors_ex(pecc_ctx *ctx, int32_t eval, int32_t force
   int prec = eval == PECC_FP32 ? 1 : 0;
   if (prec == 1 && !ctx->x32) return fail(ctx, PECC_ERR_ARG, "FP32 lists need an FP32 context");
   if (ctx->lists_prec != prec) force = 1;
-  CK(launch_build(sparams(ctx), prec, force, rebuilt_dev, nullptr, ctx->block_build, ctx->stream));
+  CK(launch_build(sparams(ctx), ctx->lt, ctx->n_small, ctx->num_sms, prec, force, rebuilt_dev, ctx->stream));
   ctx->lists_prec = prec;
   return PECC_OK;
 }
@@ -1119,12 +1157,12 @@ pecc_status pecc_warm_start_ex(pecc_ctx *ctx, pecc_mlp *mlp, int32_t rounds, dou
   if ((s = mlp_scratch(ctx))) return s;
   StandaloneParams sp = sparams(ctx);
   for (int r = 0; r < rounds; ++r) {
-    CK(launch_build(sp, 1, 1, nullptr, nullptr, ctx->block_build, ctx->stream));
+    CK(launch_build(sp, ctx->lt, ctx->n_small, ctx->num_sms, 1, 1, nullptr, ctx->stream));
     CK(energy_grad_launch(ctx, sp, 1, ctx->Eb, ctx->g));
     CK(mlp_features(sp, ctx->feat, ctx->stream));
     CK(mlp_forward(mlp->wb, mlp->params, ctx->feat, ctx->total, ctx->dout, mlp->sms, ctx->stream));
     CK(mlp_apply(sp, ctx->dout, ctx->backup, (float)max_move, ctx->stream));
-    CK(launch_build(sp, 1, 1, nullptr, nullptr, ctx->block_build, ctx->stream));
+    CK(launch_build(sp, ctx->lt, ctx->n_small, ctx->num_sms, 1, 1, nullptr, ctx->stream));
     CK(energy_grad_launch(ctx, sp, 1, ctx->Ea, ctx->g));
     CK(mlp_revert(sp, ctx->backup, ctx->Eb, ctx->Ea, accepted_dev, ctx->stream));
   }
@@ -1135,8 +1173,8 @@ pecc_status pecc_warm_start_ex(pecc_ctx *ctx, pecc_mlp *mlp, int32_t rounds, dou
 pecc_status pecc_check_feasible(pecc_ctx *ctx, double tol, uint8_t *feasible_dev, double *max_overlap_dev) {
   pecc_status s = need_radius(ctx);
   if (s) return s;
-  CK(launch_feasible(sparams(ctx), ctx->cfg.precision == PECC_FP32 ? 1 : 0, tol, feasible_dev, max_overlap_dev,
-                     ctx->block_build, ctx->stream));
+  CK(launch_feasible(sparams(ctx), ctx->lt, ctx->n_small, ctx->num_sms, ctx->cfg.precision == PECC_FP32 ? 1 : 0, tol,
+                     feasible_dev, max_overlap_dev, ctx->stream));
   return PECC_OK;
 }
 

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kDT, 2) dense_kernel(DenseParams P) {
     bool ok = true;
     auto rebuild = [&](bool anm) -> bool {
       const int tot = cta_build_neighbors<double, int32_t>(x, n, G, lc2, ckey, corder, cells, xs, rp, col, cap, S.sh,
-                                                          &S.hash, false);
+                                                          &S.hash);
       ++builds;
       if (tot > cap) return false;
       if (anm) {

@@ -406,12 +406,12 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
   // same room, so they move to global memory with it when it outgrows their share
   auto build_outer = [&]() -> bool {
     int tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, GL, lc2L, S.ckey, S.corder, S.cells, S.xs, rp, colL, capL, S.sh,
-                                                   nullptr, false);
+                                                   nullptr);
     if (tot > capL && colL_s && colL == colL_s) {
       colL = colL_g;
       capL = D.cap;
       tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, GL, lc2L, S.ckey, S.corder, S.cells, S.xs, rp, colL, capL, S.sh,
-                                                 nullptr, false);
+                                                 nullptr);
     }
     if (tot > capL) return false;
     if (tot > cap && col_s && col == col_s) {
@@ -470,12 +470,12 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
       if (two) { filter(); return true; }
     }
     int tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, G, lc2, S.ckey, S.corder, S.cells, S.xs, rp, col, cap, S.sh,
-                                                   &S.hash, false);
+                                                   &S.hash);
     if (tot > cap && col_s && col == col_s) {
       col = col_g;
       cap = D.cap;
       tot = cta_build_neighbors<pos_t, uint16_t>(xw, n, G, lc2, S.ckey, S.corder, S.cells, S.xs, rp, col, cap, S.sh,
-                                                 &S.hash, false);
+                                                 &S.hash);
     }
     if (tot > cap) return false;
     for (int p = tid; p < n; p += T) rl[p] = (uint16_t)(rp[p + 1] - rp[p]);

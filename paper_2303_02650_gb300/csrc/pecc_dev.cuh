@@ -226,8 +226,7 @@ __device__ __forceinline__ unsigned long long mix32(uint32_t x) {
 // one instance; lists go to rp[0..n], col[0..cap).  cells: 2 * nc^2 + 2 int32 of scratch;
 // ckey/corder: n each; xs: n positions of scratch (the coordinates in cell order, so that
 // the three cells of a row of the 3x3 block are one contiguous range).  All pointers may
-// be shared or global memory.  sort_rows: rows ascending in j (else in cell-scan order,
-// still deterministic).  Returns the number of entries (block-uniform); > cap means
+// be shared or global memory.  Rows come in cell-scan order (deterministic).  Returns the number of entries (block-uniform); > cap means
 // overflow and the rows are then not written.  hash (shared, may be null) receives an
 // order-independent 64-bit digest of the pair set, used to tell Gamma' from Gamma.
 // Cell binning and stable key sort of one instance (the first half of a list build): ckey[i]
@@ -273,7 +272,7 @@ __device__ void cta_cell_sort(const v2<T> *__restrict__ x, int n, const CellGrid
 template <typename T, typename IdxT>
 __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const CellGrid &G, T lc2,
                                    uint32_t *ckey, int32_t *corder, int32_t *cells, v2<T> *xs, int32_t *rp,
-                                   IdxT *col, int cap, int32_t *sh, unsigned long long *hash, bool sort_rows) {
+                                   IdxT *col, int cap, int32_t *sh, unsigned long long *hash) {
   const int T_ = blockDim.x, t = threadIdx.x;
   const int nc = G.nc;
   int32_t *cstart = cells;
@@ -316,14 +315,6 @@ __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const Cel
             col[w++] = (IdxT)j;
             if (hash) h += mix32((uint32_t)i * 0x9E3779B1u ^ (uint32_t)j);
           }
-        }
-      }
-      if (sort_rows) {
-        for (int a = first + 1; a < w; ++a) {
-          IdxT v = col[a];
-          int b = a - 1;
-          while (b >= first && col[b] > v) { col[b + 1] = col[b]; --b; }
-          col[b + 1] = v;
         }
       }
     }

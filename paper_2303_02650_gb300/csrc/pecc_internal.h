@@ -216,6 +216,25 @@ int adjust_max_m();
 // Largest instance whose coordinates the block energy + gradient kernel stages in shared memory.
 inline int energy_stage_n(int eval) { return (int)(PECC_ENERGY_STAGE_BYTES / (eval == 1 ? 8 : 16)); }
 
+// Cell binning in the standalone kernels (pecc_cells.cuh, pecc_kernels.cu): instances of at most
+// kCellsBlockN circles by one block each, in shared memory; larger ones by one kernel per step over tiles
+// of kTileRows circles (or kTileCells cells) of all of them.
+constexpr int kCellsBlockN = 2048;
+constexpr int kTileRows = 256;
+constexpr int kTileCells = 1024;
+struct LargeTiles {
+  const int2 *rows, *cells;  // {instance, tile of the instance}, in instance order
+  int nrows, ncells;
+  int32_t *row_total, *cell_total;  // per tile
+  int32_t *go;                      // per instance: the list is to be rebuilt
+  int32_t *rank, *tmp;              // per circle
+  // feasibility check, per instance: entries; smallest squared distance and largest squared radius in
+  // binary32 (bits) and in binary64 (bits); a coordinate is not finite
+  unsigned long long *hits, *smin, *rmax;
+  uint32_t *smin32, *rmax32;
+  int32_t *bad;
+};
+
 struct StandaloneParams {
   const InstDesc *desc;
   InstOut *out;
@@ -243,12 +262,13 @@ cudaError_t launch_get_positions(const StandaloneParams &p, double *xy, int from
 // Radii and cell grids of every instance from device radii (stream-ordered); a radius that is not
 // finite and > 0 leaves R = NaN and a one-cell grid.
 cudaError_t launch_set_radius(InstDesc *desc, const double *R, int num, double l_cut, cudaStream_t s);
-cudaError_t launch_build(const StandaloneParams &p, int prec, int force, int32_t *rebuilt, int32_t *status,
-                         int block, cudaStream_t s);
+// n_small: the largest instance of at most kCellsBlockN circles (-1: none)
+cudaError_t launch_build(const StandaloneParams &p, const LargeTiles &L, int n_small, int sms, int prec, int force,
+                         int32_t *rebuilt, cudaStream_t s);
 cudaError_t launch_energy_grad(const StandaloneParams &p, int eval, double *E, void *grad, void *ecirc,
                                int max_small_n, bool any_large, cudaStream_t s);
-cudaError_t launch_feasible(const StandaloneParams &p, int from32, double tol, uint8_t *feasible,
-                            double *max_overlap, int block, cudaStream_t s);
+cudaError_t launch_feasible(const StandaloneParams &p, const LargeTiles &L, int n_small, int sms, int from32,
+                            double tol, uint8_t *feasible, double *max_overlap, cudaStream_t s);
 cudaError_t launch_export_csr(const StandaloneParams &p, const int64_t *base, int32_t *row_ptr, int32_t *col,
                               cudaStream_t s);
 cudaError_t launch_export_cells(const StandaloneParams &p, uint32_t *key, int32_t *order, cudaStream_t s);

@@ -1,10 +1,13 @@
 // pecc_kernels.cu -- standalone kernels: random init (Sec. 5.1), neighbor build
 // (Sec. 4.3), fused energy + gradient (Eq. 3, Eq. 5), feasibility (Eq. 1, Eq. 2).
+#include "pecc_cells.cuh"
 #include "pecc_internal.h"
 
 namespace pecc {
 
 namespace {
+
+inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 // Asynchronous copy of BYTES (8 or 16) from global to shared memory (cp.async; completed by
 // cp.async.wait_all).  Both addresses must be BYTES-aligned.
@@ -101,40 +104,376 @@ __global__ void set_radius_kernel(InstDesc *desc, const double *__restrict__ R, 
 }
 
 // ----------------------------------------------------------------- build ----
+// Lists of Sec. 4.3 as CSR rows ascending in j, from the cells (pecc_cells.cuh).  A warp takes 32
+// consecutive circles, a lane a row: the lane collects its hits (kRowHits 16- or 32-bit indices at
+// most, a column of the warp's buffer), ranks them among themselves, and the warp writes its 32 rows as
+// one contiguous piece.  A row with more hits sends its warp to the general path below (second walk,
+// entries straight to global memory, insertion sort).
+constexpr int kRowHits = 16;
+
+// Hits of the circle at xi (index i, cell key) over the 3x3 cells, in scan order: f(q) for each.
+template <typename T, typename I, typename F>
+__device__ __forceinline__ void for_neighbors(const Coords<T> &X, typename Coords<T>::point xi, int i, int key, int nc,
+                                              const int32_t *start, const float2 *xs, const I *ord,
+                                              const Near<T> &near, F f) {
+  const int cy = key / nc, cx = key - cy * nc;
+  const int bx0 = max(cx - 1, 0), bx1 = min(cx + 1, nc - 1);
+  for (int by = max(cy - 1, 0); by <= min(cy + 1, nc - 1); ++by) {
+    const int lo = start[by * nc + bx0], hi = start[by * nc + bx1 + 1];
+    for (int q = lo; q < hi; ++q)
+      if (near(xi, xs[q], X, ord, q) && (int)ord[q] != i) f(q);
+  }
+}
+
+// The 32 rows of a warp, once every lane knows where its row starts: buf holds the lane's hits at
+// buf[32 h + lane] (cnt of them when cnt <= kRowHits), row0 is the lane's row start.  Entries at or
+// past cap are not written (an overflowed list).
+template <typename T, typename I>
+__device__ __forceinline__ void write_rows(const Coords<T> &X, bool act, int i, int key, int nc, const int32_t *start,
+                                           const float2 *xs, const I *ord, I *buf, int cnt, int row0, int32_t *col,
+                                           int cap) {
+  const int lane = threadIdx.x & 31;
+  if (__any_sync(0xffffffffu, cnt > kRowHits)) {
+    if (act) {
+      const typename Coords<T>::point xi = X.at(i);
+      Near<T> near;
+      near.init(xi, X.l_cut);
+      int w = row0;
+      for_neighbors<T, I>(X, xi, i, key, nc, start, xs, ord, near, [&](int q) {
+        const int v = (int)ord[q];
+        if (w < cap) {  // insert in ascending order
+          int t = w - 1;
+          while (t >= row0 && col[t] > v) { col[t + 1] = col[t]; --t; }
+          col[t + 1] = v;
+        }
+        ++w;
+      });
+    }
+    return;
+  }
+  // ranks among the lane's own hits, all of them in registers
+  int h[kRowHits], rank[kRowHits];
+#pragma unroll
+  for (int u = 0; u < kRowHits; ++u) {
+    h[u] = u < cnt ? (int)buf[32 * u + lane] : 0x7fffffff;
+    rank[u] = 0;
+  }
+#pragma unroll
+  for (int u = 0; u < kRowHits / 2; ++u)
+#pragma unroll
+    for (int v = u + 1; v < kRowHits / 2; ++v) {
+      const bool less = h[v] < h[u];
+      rank[u] += less;
+      rank[v] += !less;
+    }
+  if (__any_sync(0xffffffffu, cnt > kRowHits / 2)) {
+#pragma unroll
+    for (int v = kRowHits / 2; v < kRowHits; ++v)
+#pragma unroll
+      for (int u = 0; u < v; ++u) {
+        const bool less = h[v] < h[u];
+        rank[u] += less;
+        rank[v] += !less;
+      }
+  }
+  const int base = __shfl_sync(0xffffffffu, row0, 0);
+  const int total = __shfl_sync(0xffffffffu, row0 + cnt, 31) - base;  // lanes past the last row have none
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < kRowHits; ++u)
+    if (u < cnt) buf[row0 - base + rank[u]] = (I)h[u];
+  __syncwarp();
+  for (int t = lane; t < total; t += 32)
+    if (base + t < cap) col[base + t] = (int)buf[t];
+  __syncwarp();  // the next rows' hits go into the same buffer
+}
+
+// Exclusive prefix sum of one value per thread over the block; total: the block's sum.  sh: 33 ints.
+__device__ __forceinline__ int block_exclusive(int v, int32_t *sh, int &total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  __syncthreads();  // the previous call's reads of sh
+  if (lane == 31) sh[w] = incl;
+  __syncthreads();
+  int before = 0;
+  total = 0;
+  for (int u = 0; u < nw; ++u) {
+    const int t = sh[u];
+    before += u < w ? t : 0;
+    total += t;
+  }
+  return before + incl - v;
+}
+
+template <typename T> __device__ __forceinline__ Coords<T> coords_of(const StandaloneParams &P, int64_t off, int from32);
+template <> __device__ __forceinline__ Coords<float> coords_of<float>(const StandaloneParams &P, int64_t off, int) {
+  return Coords<float>{P.x32 + off, P.l_cut};
+}
+template <> __device__ __forceinline__ Coords<double> coords_of<double>(const StandaloneParams &P, int64_t off,
+                                                                        int from32) {
+  return Coords<double>{P.x64 + off, from32 ? P.x32 + off : nullptr, P.l_cut};
+}
+
+// Instances of at most kCellsBlockN circles, one block each, everything on chip: the coordinates come
+// in once, the rows, cells and order go out once.  What bounds it is the latency of the block's chain
+// (cell counts, two scans, candidate walks).  The 4096-instance batch's new positions, lists, energy and
+// gradient take 216 us with it, about 160 us of them here; 966 us with the kernel it replaced (lists
+// built and sorted in global memory, 901 us).
+constexpr int kBuildWarpBytes = 32 * kRowHits * (int)sizeof(uint16_t);
 template <typename T>
-__global__ void build_kernel(StandaloneParams P, int force, int32_t *rebuilt, int32_t *status) {
+__global__ void __launch_bounds__(512) build_block_kernel(StandaloneParams P, int force, int32_t *rebuilt) {
+  extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int32_t sh[40];
   using PP = v2<T>;
-  const int q = blockIdx.x;
-  const InstDesc D = P.desc[q];
+  const int q = P.eorder[blockIdx.x];
+  const InstDesc &D = P.desc[q];
   const int n = D.n;
-  const PP *x;
-  if constexpr (sizeof(T) == 4) x = (const PP *)(P.x32 + D.off);
-  else x = (const PP *)(P.x64 + D.off);
-  PP *xb = (PP *)P.xbuild + D.off;
+  if (n > kCellsBlockN) return;
+  const int64_t off = D.off;
+  const Coords<T> X = coords_of<T>(P, off, 0);
+  PP *xb = (PP *)P.xbuild + off;
   int go = force;
   if (!go) {
     // largest displacement since the last standalone build
     double m = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      PP a = x[i], b = xb[i];
-      double dx = (double)a.x - (double)b.x, dy = (double)a.y - (double)b.y;
+      const PP a = X.at(i), b = xb[i];
+      const double dx = (double)a.x - (double)b.x, dy = (double)a.y - (double)b.y;
       m = fmax(m, dx * dx + dy * dy);
     }
     go = __syncthreads_or(m > P.rebuild_disp * P.rebuild_disp);
   }
-  if (go) {
-    const T lc2 = (T)(P.l_cut * P.l_cut);
-    CellGrid G{D.R, D.inv_cs, 0.f, 0.f, D.ncx, false};
-    int tot = cta_build_neighbors<T, int32_t>(x, n, G, lc2, P.ckey + D.off, P.corder + D.off, P.cells + D.cell_off,
-                                     (PP *)P.xtmp + D.off, P.rp + D.off + q, P.col + D.col_s_off, D.cap, sh,
-                                     nullptr, true);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) xb[i] = x[i];
-    if (threadIdx.x == 0 && status) status[q] = tot > D.cap ? 4 : 0;
-  } else if (threadIdx.x == 0 && status) {
-    status[q] = 0;
-  }
   if (threadIdx.x == 0 && rebuilt) rebuilt[q] = go;
+  if (!go) return;
+  const int nc = D.ncx, cap = D.cap;
+  const size_t extra = (size_t)(blockDim.x >> 5) * kBuildWarpBytes;
+  const BlockCells C = block_cells<T>(X, n, D.R, D.inv_cs, nc, sm, extra, P.cells + D.cell_off, P.ckey + off,
+                                      P.corder + off, sh, [&](int i, PP p) { xb[i] = p; });
+  int32_t *rp = P.rp + off + q, *col = P.col + D.col_s_off;
+  uint16_t *buf = (uint16_t *)(C.extra + (threadIdx.x >> 5) * kBuildWarpBytes);
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) rp[0] = 0;
+  int run = 0;
+  for (int i0 = 0; i0 < n; i0 += blockDim.x) {
+    const int i = i0 + threadIdx.x;
+    const bool act = i < n;
+    int cnt = 0, key = 0;
+    if (act) {
+      const PP xi = X.at(i);
+      key = C.key[i];
+      Near<T> near;
+      near.init(xi, P.l_cut);
+      for_neighbors<T, uint16_t>(X, xi, i, key, nc, C.start, C.xs, C.ord, near, [&](int qq) {
+        if (cnt < kRowHits) buf[32 * cnt + lane] = C.ord[qq];
+        ++cnt;
+      });
+    }
+    int total;
+    const int row0 = run + block_exclusive(cnt, sh, total);
+    if (act) rp[i + 1] = row0 + cnt;
+    write_rows<T, uint16_t>(X, act, i, key, nc, C.start, C.xs, C.ord, buf, cnt, row0, col, cap);
+    run += total;
+  }
+}
+
+// ---- larger instances: one kernel per step over tiles of all of them (pecc_cells.cuh); each step reads
+// what the one before it wrote.  One block per instance left the GPU idle: new positions, lists, energy
+// and gradient of 100000 circles took 3842 us, now 88 us, most of it the launches' own latency.  The line
+// to the block form is where its shared memory and one block's time end; from 1000 circles on a block
+// takes longer than the eight launches, but a batch of such instances fills the GPU with blocks.
+struct LargeDest { uint32_t *ckey; int32_t *corder; float2 *xs; };  // per circle (offset by the instance)
+
+template <typename T>
+__global__ void __launch_bounds__(kTileRows) large_go_kernel(StandaloneParams P, LargeTiles L, int force) {
+  const int2 t = L.rows[blockIdx.x];
+  const InstDesc &D = P.desc[t.x];
+  const int i = t.y * kTileRows + threadIdx.x, n = D.n;
+  // the instance's cell counters, four per thread of its row tiles, the last tile to the end
+  int32_t *cells = P.cells + D.cell_off;
+  const int ncell = D.ncx * D.ncx, last = (n - 1) / kTileRows;
+  const int c1 = t.y == last ? ncell + 1 : min(ncell + 1, (t.y + 1) * 4 * kTileRows);
+  for (int c = t.y * 4 * kTileRows + threadIdx.x; c < c1; c += kTileRows) cells[c] = 0;
+  int go = force;
+  if (!go) {
+    using PP = v2<T>;
+    double m = 0.0;
+    if (i < n) {
+      const PP a = coords_of<T>(P, D.off, 0).at(i), b = ((const PP *)P.xbuild + D.off)[i];
+      const double dx = (double)a.x - (double)b.x, dy = (double)a.y - (double)b.y;
+      m = dx * dx + dy * dy;
+    }
+    go = __syncthreads_or(m > P.rebuild_disp * P.rebuild_disp);
+  }
+  if (threadIdx.x == 0 && go) atomicOr(&L.go[t.x], 1);  // cleared before this launch
+}
+
+// cells of every circle and its arrival rank in its cell; for the list build also the reference
+// coordinates, for the feasibility check the largest radius and the finiteness
+template <typename T, bool CHECK>
+__global__ void __launch_bounds__(kTileRows) large_key_kernel(StandaloneParams P, LargeTiles L, LargeDest O, int from32,
+                                                              v2<T> *xbuild) {
+  const int2 t = L.rows[blockIdx.x];
+  if (!CHECK && !L.go[t.x]) return;
+  const InstDesc &D = P.desc[t.x];
+  const int i = t.y * kTileRows + threadIdx.x;
+  float r2 = 0.f;
+  int bad = 0;
+  if (i < D.n) {
+    const typename Coords<T>::point p = coords_of<T>(P, D.off, from32).at(i);
+    const int key = cell_key_fast(p, D.R, D.inv_cs, D.ncx);
+    O.ckey[D.off + i] = (uint32_t)key;
+    L.rank[D.off + i] = atomicAdd(P.cells + D.cell_off + key + 1, 1);
+    if (xbuild) xbuild[D.off + i] = p;
+    if (CHECK) {
+      const float fx = (float)p.x, fy = (float)p.y;
+      r2 = fx * fx + fy * fy;
+      bad = !(isfinite(p.x) && isfinite(p.y));
+    }
+  }
+  if (CHECK) {
+    bad = __syncthreads_or(bad);
+    r2 = warp_max(r2);
+    if ((threadIdx.x & 31) == 0 && r2 > 0.f) atomicMax(&L.rmax32[t.x], __float_as_uint(r2));
+    if (threadIdx.x == 0 && bad) atomicOr(&L.bad[t.x], 1);
+  }
+}
+
+// inclusive sums of the cell counts within a tile of cells, and the tile's total
+__global__ void __launch_bounds__(256) large_cells_kernel(StandaloneParams P, LargeTiles L) {
+  __shared__ int32_t sh[40];
+  const int2 t = L.cells[blockIdx.x];
+  if (!L.go[t.x]) return;
+  const InstDesc &D = P.desc[t.x];
+  const int ncell = D.ncx * D.ncx, c0 = t.y * kTileCells;
+  int32_t *a = P.cells + D.cell_off + 1 + c0;
+  const int m = min(kTileCells, ncell - c0);
+  int v[4], s = 0;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int c = 4 * threadIdx.x + u;
+    v[u] = c < m ? a[c] : 0;
+    s += v[u];
+  }
+  int total, run = block_exclusive(s, sh, total);
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int c = 4 * threadIdx.x + u;
+    run += v[u];
+    if (c < m) a[c] = run;
+  }
+  if (threadIdx.x == 0) L.cell_total[blockIdx.x] = m > 0 ? total : 0;
+}
+
+// Sum of the totals of the earlier tiles of tile b's instance (its tile t.y of the instance).
+__device__ __forceinline__ int tiles_before(const int32_t *total, int b, int ty, int32_t *sh) {
+  int s = 0;
+  for (int u = threadIdx.x; u < ty; u += blockDim.x) s += total[b - ty + u];
+  int all;
+  block_exclusive(s, sh, all);
+  return all;
+}
+
+__global__ void __launch_bounds__(256) large_cells_base_kernel(StandaloneParams P, LargeTiles L) {
+  __shared__ int32_t sh[40];
+  const int2 t = L.cells[blockIdx.x];
+  if (!L.go[t.x]) return;
+  const InstDesc &D = P.desc[t.x];
+  const int ncell = D.ncx * D.ncx, c0 = t.y * kTileCells;
+  if (c0 >= ncell) return;
+  const int base = tiles_before(L.cell_total, blockIdx.x, t.y, sh);
+  int32_t *a = P.cells + D.cell_off + 1 + c0;
+  for (int c = threadIdx.x; c < min(kTileCells, ncell - c0); c += blockDim.x) a[c] += base;
+}
+
+__global__ void __launch_bounds__(kTileRows) large_scatter_kernel(StandaloneParams P, LargeTiles L, LargeDest O) {
+  const int2 t = L.rows[blockIdx.x];
+  if (!L.go[t.x]) return;
+  const InstDesc &D = P.desc[t.x];
+  const int i = t.y * kTileRows + threadIdx.x;
+  if (i < D.n) L.tmp[D.off + P.cells[D.cell_off + O.ckey[D.off + i]] + L.rank[D.off + i]] = i;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kTileRows) large_order_kernel(StandaloneParams P, LargeTiles L, LargeDest O,
+                                                                int from32) {
+  const int2 t = L.rows[blockIdx.x];
+  if (!L.go[t.x]) return;
+  const InstDesc &D = P.desc[t.x];
+  const int p = t.y * kTileRows + threadIdx.x;
+  if (p >= D.n) return;
+  const int32_t *tmp = L.tmp + D.off, *start = P.cells + D.cell_off;
+  const int i = tmp[p], c = (int)O.ckey[D.off + i];
+  int r = start[c];
+  for (int q = start[c], hi = start[c + 1]; q < hi; ++q) r += tmp[q] < i;
+  O.corder[D.off + r] = i;
+  O.xs[D.off + r] = coords_of<T>(P, D.off, from32).low(i);
+}
+
+// FILL = false: the entries of every tile of rows; true: the rows.
+template <typename T, bool FILL>
+__global__ void __launch_bounds__(kTileRows) large_rows_kernel(StandaloneParams P, LargeTiles L, LargeDest O) {
+  __shared__ int32_t sh[40];
+  __shared__ int32_t bufs[FILL ? kTileRows * kRowHits : 1];
+  const int2 t = L.rows[blockIdx.x];
+  if (!L.go[t.x]) return;
+  const InstDesc &D = P.desc[t.x];
+  const int n = D.n, i = t.y * kTileRows + threadIdx.x, lane = threadIdx.x & 31, nc = D.ncx;
+  const Coords<T> X = coords_of<T>(P, D.off, 0);
+  const int32_t *start = P.cells + D.cell_off, *ord = O.corder + D.off;
+  const float2 *xs = O.xs + D.off;
+  int32_t *buf = bufs + (FILL ? (threadIdx.x >> 5) * 32 * kRowHits : 0);
+  const bool act = i < n;
+  int cnt = 0, key = 0;
+  if (act) {
+    const typename Coords<T>::point xi = X.at(i);
+    key = (int)O.ckey[D.off + i];
+    Near<T> near;
+    near.init(xi, P.l_cut);
+    for_neighbors<T, int32_t>(X, xi, i, key, nc, start, xs, ord, near, [&](int q) {
+      if (FILL && cnt < kRowHits) buf[32 * cnt + lane] = ord[q];
+      ++cnt;
+    });
+  }
+  if (!FILL) {
+    int total;
+    block_exclusive(cnt, sh, total);
+    if (threadIdx.x == 0) L.row_total[blockIdx.x] = total;
+    return;
+  }
+  const int base = tiles_before(L.row_total, blockIdx.x, t.y, sh);
+  int total;
+  const int row0 = base + block_exclusive(cnt, sh, total);
+  int32_t *rp = P.rp + D.off + t.x;
+  if (act) rp[i + 1] = row0 + cnt;
+  if (i == 0) rp[0] = 0;
+  write_rows<T, int32_t>(X, act, i, key, nc, start, xs, ord, buf, cnt, row0, P.col + D.col_s_off, D.cap);
+}
+
+__global__ void large_rebuilt_kernel(StandaloneParams P, LargeTiles L, int32_t *rebuilt) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= L.nrows) return;
+  const int2 t = L.rows[b];
+  if (t.y == 0) rebuilt[t.x] = L.go[t.x];
+}
+
+// Cells, order and sorted coordinates of every large instance (flags in L.go, or all of them).
+template <typename T, bool CHECK>
+cudaError_t large_cells(const StandaloneParams &p, const LargeTiles &L, const LargeDest &O, int from32, int force,
+                        v2<T> *xbuild, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(L.go, 0, sizeof(int32_t) * (size_t)p.num, s);
+  if (e != cudaSuccess) return e;
+  large_go_kernel<T><<<L.nrows, kTileRows, 0, s>>>(p, L, force);
+  large_key_kernel<T, CHECK><<<L.nrows, kTileRows, 0, s>>>(p, L, O, from32, xbuild);
+  large_cells_kernel<<<L.ncells, 256, 0, s>>>(p, L);
+  large_cells_base_kernel<<<L.ncells, 256, 0, s>>>(p, L);
+  large_scatter_kernel<<<L.nrows, kTileRows, 0, s>>>(p, L, O);
+  large_order_kernel<T><<<L.nrows, kTileRows, 0, s>>>(p, L, O, from32);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------- fused energy + gradient ----
@@ -318,54 +657,206 @@ __global__ void __launch_bounds__(1024) energy_reduce_kernel(StandaloneParams P,
 }
 
 // ----------------------------------------------------------- feasibility ----
-// A fresh FP64 list with cutoff l_cut > 2 holds every pair with l_ij < 2, so the largest
-// depth over the list equals the largest over all pairs (Eq. 1); walls per circle (Eq. 2).
-__global__ void feasible_kernel(StandaloneParams P, int from32, double tol, uint8_t *feasible,
-                                double *max_overlap) {
-  __shared__ int32_t sh[40];
-  __shared__ double red[32];
-  const int q = P.eorder[blockIdx.x];  // largest instance first
-  const InstDesc D = P.desc[q];
-  const int n = D.n;
-  double2 *x = (double2 *)P.xtmp + D.off;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    if (from32) { float2 f = P.x32[D.off + i]; x[i] = make_double2((double)f.x, (double)f.y); }
-    else x[i] = P.x64[D.off + i];
+// The largest overlap depth over all pairs (Eq. 1) and walls (Eq. 2), with correctly rounded binary64
+// operations: a pair's depth fl(2 - fl(sqrt(s))) never rises with its squared distance s, a wall's never
+// falls with the squared radius, so the two extremes decide and only they take the square root.  The
+// search runs in binary32; the binary64 values are formed for the pairs and circles whose binary32 ones
+// lie within the slack of the extreme.  The entries a list with cutoff l_cut > 2 would hold (it holds
+// every overlapping pair) are counted: past twice the capacity the instance is not checkable.
+// The 4096-instance batch: 187 us, against 2212 us for a binary64 list build and a walk over it, which
+// the two binary64 lanes of an SM bound.
+__device__ __forceinline__ double dist2_exact(double2 a, double2 b) {
+  const double dx = __dsub_rn(a.x, b.x), dy = __dsub_rn(a.y, b.y);
+  return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+}
+__device__ __forceinline__ double norm2_exact(double2 a) { return __dadd_rn(__dmul_rn(a.x, a.x), __dmul_rn(a.y, a.y)); }
+
+// v = the larger of 0 and the two depths; s2 / r2: smallest squared distance (below 4, or infinity) and
+// largest squared radius
+__device__ __forceinline__ void feasible_result(const StandaloneParams &P, int q, double R, bool bad, double s2,
+                                                double r2, double tol, uint8_t *feasible, double *max_overlap) {
+  double v = 0.0;
+  if (s2 < 4.0) v = fmax(v, __dsub_rn(2.0, __dsqrt_rn(s2)));
+  const double d = __dsub_rn(__dadd_rn(__dsqrt_rn(r2), 1.0), R);
+  v = fmax(v, d > 0.0 ? d : 0.0);
+  if (P.desc[q].n == 0) v = 0.0;
+  if (bad) v = __longlong_as_double(0x7ff8000000000000ll);  // NaN: not checkable
+  const bool ok = !bad && v <= tol;
+  if (feasible) feasible[q] = ok ? 1 : 0;
+  if (max_overlap) max_overlap[q] = v;
+  P.out[q].max_overlap = v;
+}
+
+// Bounds for the exact pass from the extremes of the binary32 search: pairs up to *s_hi, circles from
+// *r_lo on.  m: the slack at the instance's largest coordinate.
+__device__ __forceinline__ void exact_bounds(float smin, float rmax, float *s_hi, float *r_lo) {
+  const float r = sqrtf(rmax), m = dist_slack(1.5f * r, 2.f);
+  const bool ok = m <= 0.25f;  // else every pair and circle in binary64
+  const float l = sqrtf(smin) + 2.f * m, w = fmaxf(r - 2.f * m, 0.f);
+  *s_hi = ok ? fminf(l * l, (2.f + m) * (2.f + m)) : __int_as_float(0x7f800000);
+  *r_lo = ok ? w * w : -1.f;
+}
+
+// Visit the circles around sorted position p: f(q, squared distance in binary32) for every other circle
+// of its 3x3 cells.
+template <typename I, typename F>
+__device__ __forceinline__ void for_candidates(int p, int key, int nc, const int32_t *start, const float2 *xs,
+                                               const I *, F f) {
+  const int cy = key / nc, cx = key - cy * nc;
+  const int bx0 = max(cx - 1, 0), bx1 = min(cx + 1, nc - 1);
+  const float2 a = xs[p];
+  for (int by = max(cy - 1, 0); by <= min(cy + 1, nc - 1); ++by) {
+    const int lo = start[by * nc + bx0], hi = start[by * nc + bx1 + 1];
+    for (int q = lo; q < hi; ++q) {
+      if (q == p) continue;
+      const float dx = a.x - xs[q].x, dy = a.y - xs[q].y;
+      f(q, dx * dx + dy * dy);
+    }
   }
-  __syncthreads();
-  int32_t *rp = P.rp_t + D.rp_off;
-  int32_t *cl = P.col_t + D.col_off;
-  const double lc2 = P.l_cut * P.l_cut;
-  CellGrid G{D.R, D.inv_cs, 0.f, 0.f, D.ncx, false};
-  int tot = cta_build_neighbors<double, int32_t>(x, n, G, lc2, P.ckey_t + D.off, P.corder_t + D.off, P.cells + D.cell_off,
-                                        (double2 *)P.xtmp2 + D.off, rp, cl, 2 * D.cap, sh, nullptr, false);
-  double m = 0.0;
+}
+
+__global__ void __launch_bounds__(512) feasible_block_kernel(StandaloneParams P, int from32, double tol,
+                                                             uint8_t *feasible, double *max_overlap) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ int32_t sh[40];
+  __shared__ float f_s[32], f_r[32];
+  __shared__ int h_n[32];
+  __shared__ double d_s[32], d_r[32];
+  const int q = P.eorder[blockIdx.x];  // largest instance first
+  const InstDesc &D = P.desc[q];
+  const int n = D.n;
+  if (n > kCellsBlockN) return;
+  const Coords<double> X = coords_of<double>(P, D.off, from32);
+  const int nc = D.ncx, lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  float rmax = 0.f;
   int bad = 0;
-  if (tot <= 2 * D.cap) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      double2 xi = x[i];
-      bad |= !(isfinite(xi.x) && isfinite(xi.y));
-      for (int t = rp[i]; t < rp[i + 1]; ++t) {
-        int j = cl[t];
-        if (j > i) m = fmax(m, pair_depth_exact(xi, x[j]));
-      }
-      m = fmax(m, wall_depth_exact(xi, D.R));
+  const BlockCells C =
+      block_cells<double>(X, n, D.R, D.inv_cs, nc, sm, 0, P.cells + D.cell_off, nullptr, nullptr, sh,
+                          [&](int, double2 p) {
+                            const float fx = (float)p.x, fy = (float)p.y;
+                            rmax = fmaxf(rmax, fx * fx + fy * fy);
+                            bad |= !(isfinite(p.x) && isfinite(p.y));
+                          });
+  const float inf = __int_as_float(0x7f800000);
+  float smin = inf;
+  int hits = 0;
+  for (int p = threadIdx.x; p < n; p += blockDim.x) {
+    const int i = C.ord[p];
+    Near<double> near;
+    const float2 a = C.xs[p];
+    near.init(make_double2((double)a.x, (double)a.y), P.l_cut);  // lo and hi allow for the rounding
+    for_candidates(p, (int)C.key[i], nc, C.start, C.xs, C.ord, [&](int qq, float s) {
+      smin = fminf(smin, s);
+      if (s > near.hi) return;
+      hits += (s < near.lo) || nbr_pred(X.at(i), X.at(C.ord[qq]), near.lc2);
+    });
+  }
+  const float my_s = smin;
+  smin = -warp_max(-smin);
+  rmax = warp_max(rmax);
+  hits = warp_sum(hits);
+  if (lane == 0) { f_s[w] = smin; f_r[w] = rmax; h_n[w] = hits; }
+  bad = __syncthreads_or(bad);
+  long long tot = 0;
+  for (int u = 0; u < nw; ++u) {
+    smin = fminf(smin, f_s[u]);
+    rmax = fmaxf(rmax, f_r[u]);
+    tot += h_n[u];
+  }
+  bad |= tot > 2ll * D.cap;
+  double s2 = (double)inf, r2 = 0.0;
+  if (!bad) {
+    float s_hi, r_lo;
+    exact_bounds(smin, rmax, &s_hi, &r_lo);
+    const bool pairs = !(my_s > s_hi);
+    for (int p = threadIdx.x; p < n; p += blockDim.x) {
+      const float2 a = C.xs[p];
+      const int i = C.ord[p];
+      if (!(a.x * a.x + a.y * a.y < r_lo)) r2 = fmax(r2, norm2_exact(X.at(i)));
+      if (pairs)
+        for_candidates(p, (int)C.key[i], nc, C.start, C.xs, C.ord, [&](int qq, float s) {
+          if (!(s > s_hi)) s2 = fmin(s2, dist2_exact(X.at(i), X.at(C.ord[qq])));
+        });
+    }
+  }
+  s2 = -warp_max(-s2);
+  r2 = warp_max(r2);
+  if (lane == 0) { d_s[w] = s2; d_r[w] = r2; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int u = 1; u < nw; ++u) { s2 = fmin(s2, d_s[u]); r2 = fmax(r2, d_r[u]); }
+    feasible_result(P, q, D.R, bad, s2, r2, tol, feasible, max_overlap);
+  }
+}
+
+// the same over the tiles of the larger instances: the binary32 search, the exact pass, the result
+template <bool EXACT>
+__global__ void __launch_bounds__(kTileRows) large_check_kernel(StandaloneParams P, LargeTiles L, LargeDest O,
+                                                                int from32) {
+  const int2 t = L.rows[blockIdx.x];
+  const InstDesc &D = P.desc[t.x];
+  const int n = D.n, p = t.y * kTileRows + threadIdx.x, nc = D.ncx, lane = threadIdx.x & 31;
+  const Coords<double> X = coords_of<double>(P, D.off, from32);
+  const int32_t *start = P.cells + D.cell_off, *ord = O.corder + D.off;
+  const float2 *xs = O.xs + D.off;
+  const float inf = __int_as_float(0x7f800000);
+  if (!EXACT) {
+    float smin = inf;
+    int hits = 0;
+    if (p < n) {
+      const int i = ord[p];
+      Near<double> near;
+      const float2 a = xs[p];
+      near.init(make_double2((double)a.x, (double)a.y), P.l_cut);
+      for_candidates(p, (int)O.ckey[D.off + i], nc, start, xs, ord, [&](int q, float s) {
+        smin = fminf(smin, s);
+        if (s > near.hi) return;
+        hits += (s < near.lo) || nbr_pred(X.at(i), X.at(ord[q]), near.lc2);
+      });
+    }
+    smin = -warp_max(-smin);
+    hits = warp_sum(hits);
+    if (lane == 0) {
+      atomicMin(&L.smin32[t.x], __float_as_uint(smin));
+      if (hits) atomicAdd(&L.hits[t.x], (unsigned long long)hits);
     }
   } else {
-    bad = 1;
+    if (L.bad[t.x] || L.hits[t.x] > 2ull * (unsigned long long)D.cap) return;
+    float s_hi, r_lo;
+    exact_bounds(__uint_as_float(L.smin32[t.x]), __uint_as_float(L.rmax32[t.x]), &s_hi, &r_lo);
+    if (p >= n) return;
+    const int i = ord[p];
+    const float2 a = xs[p];
+    if (!(a.x * a.x + a.y * a.y < r_lo))
+      atomicMax(&L.rmax[t.x], (unsigned long long)__double_as_longlong(norm2_exact(X.at(i))));
+    for_candidates(p, (int)O.ckey[D.off + i], nc, start, xs, ord, [&](int q, float s) {
+      if (!(s > s_hi))
+        atomicMin(&L.smin[t.x], (unsigned long long)__double_as_longlong(dist2_exact(X.at(i), X.at(ord[q]))));
+    });
   }
-  m = warp_max(m);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  bad = __syncthreads_or(bad);
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmax(v, red[w]);
-    if (bad) v = __longlong_as_double(0x7ff8000000000000ll);  // NaN: not checkable
-    bool ok = !bad && v <= tol;
-    if (feasible) feasible[q] = ok ? 1 : 0;
-    if (max_overlap) max_overlap[q] = v;
-    P.out[q].max_overlap = v;
-  }
+}
+__global__ void large_check_init_kernel(StandaloneParams P, LargeTiles L) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= L.nrows) return;
+  const int2 t = L.rows[b];
+  if (t.y) return;
+  L.hits[t.x] = 0;
+  L.smin[t.x] = 0x7ff0000000000000ull;
+  L.rmax[t.x] = 0;
+  L.smin32[t.x] = 0x7f800000u;
+  L.rmax32[t.x] = 0;
+  L.bad[t.x] = 0;
+}
+__global__ void large_check_result_kernel(StandaloneParams P, LargeTiles L, double tol, uint8_t *feasible,
+                                          double *max_overlap) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= L.nrows) return;
+  const int2 t = L.rows[b];
+  if (t.y) return;
+  const InstDesc &D = P.desc[t.x];
+  const bool bad = L.bad[t.x] || L.hits[t.x] > 2ull * (unsigned long long)D.cap;
+  feasible_result(P, t.x, D.R, bad, __longlong_as_double((long long)L.smin[t.x]),
+                  __longlong_as_double((long long)L.rmax[t.x]), tol, feasible, max_overlap);
 }
 
 // ---------------------------------------------------------------- export ----
@@ -421,8 +912,6 @@ __global__ void stats_kernel(const InstOut *out, int num, int32_t *st) {
   r[5] = o.resets; r[6] = o.stalls; r[7] = o.polished; r[8] = o.iters32; r[9] = o.trials32;
 }
 
-inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
-
 }  // namespace
 
 cudaError_t launch_init(const StandaloneParams &p, uint64_t seed, int mode, int prec, cudaStream_t s) {
@@ -445,12 +934,39 @@ cudaError_t launch_set_radius(InstDesc *desc, const double *R, int num, double l
   return cudaGetLastError();
 }
 
-cudaError_t launch_build(const StandaloneParams &p, int prec, int force, int32_t *rebuilt, int32_t *status,
-                         int block, cudaStream_t s) {
-  if (p.num <= 0) return cudaSuccess;
-  if (prec == 1) build_kernel<float><<<p.num, block, 0, s>>>(p, force, rebuilt, status);
-  else build_kernel<double><<<p.num, block, 0, s>>>(p, force, rebuilt, status);
+// Threads of a block per instance: one circle per thread up to 256; 512 when the instances leave SMs
+// idle anyway.
+static int cells_threads(int n_small, int num, int sms) {
+  if (n_small > 512 && num <= sms) return 512;
+  return n_small <= 64 ? 64 : (n_small <= 128 ? 128 : 256);
+}
+
+template <typename T>
+static cudaError_t build_t(const StandaloneParams &p, const LargeTiles &L, int n_small, int sms, int force,
+                           int32_t *rebuilt, cudaStream_t s) {
+  if (n_small >= 0) {
+    const int block = cells_threads(n_small, p.num, sms);
+    const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kBuildWarpBytes);
+    cudaError_t e = cudaFuncSetAttribute(build_block_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    build_block_kernel<T><<<p.num, block, smem, s>>>(p, force, rebuilt);
+  }
+  if (L.nrows > 0) {
+    const LargeDest O{p.ckey, p.corder, (float2 *)p.xtmp};
+    cudaError_t e = large_cells<T, false>(p, L, O, 0, force, (v2<T> *)p.xbuild, s);
+    if (e != cudaSuccess) return e;
+    large_rows_kernel<T, false><<<L.nrows, kTileRows, 0, s>>>(p, L, O);
+    large_rows_kernel<T, true><<<L.nrows, kTileRows, 0, s>>>(p, L, O);
+    if (rebuilt) large_rebuilt_kernel<<<blocks_for(L.nrows, 128), 128, 0, s>>>(p, L, rebuilt);
+  }
   return cudaGetLastError();
+}
+
+cudaError_t launch_build(const StandaloneParams &p, const LargeTiles &L, int n_small, int sms, int prec, int force,
+                         int32_t *rebuilt, cudaStream_t s) {
+  if (p.num <= 0) return cudaSuccess;
+  return prec == 1 ? build_t<float>(p, L, n_small, sms, force, rebuilt, s)
+                   : build_t<double>(p, L, n_small, sms, force, rebuilt, s);
 }
 
 template <class A> static cudaError_t launch_eg_block(const StandaloneParams &p, int stage_n, size_t smem,
@@ -487,9 +1003,25 @@ cudaError_t launch_energy_grad(const StandaloneParams &p, int eval, double *E, v
   return cudaGetLastError();
 }
 
-cudaError_t launch_feasible(const StandaloneParams &p, int from32, double tol, uint8_t *feasible,
-                            double *max_overlap, int block, cudaStream_t s) {
-  if (p.num > 0) feasible_kernel<<<p.num, block, 0, s>>>(p, from32, tol, feasible, max_overlap);
+cudaError_t launch_feasible(const StandaloneParams &p, const LargeTiles &L, int n_small, int sms, int from32,
+                            double tol, uint8_t *feasible, double *max_overlap, cudaStream_t s) {
+  if (p.num <= 0) return cudaSuccess;
+  if (n_small >= 0) {
+    const size_t smem = cells_smem(n_small, 0);
+    cudaError_t e = cudaFuncSetAttribute(feasible_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    feasible_block_kernel<<<p.num, cells_threads(n_small, p.num, sms), smem, s>>>(p, from32, tol, feasible, max_overlap);
+  }
+  if (L.nrows > 0) {
+    const LargeDest O{p.ckey_t, p.corder_t, (float2 *)p.xtmp2};
+    const unsigned nb = blocks_for(L.nrows, 128);
+    large_check_init_kernel<<<nb, 128, 0, s>>>(p, L);
+    cudaError_t e = large_cells<double, true>(p, L, O, from32, 1, nullptr, s);
+    if (e != cudaSuccess) return e;
+    large_check_kernel<false><<<L.nrows, kTileRows, 0, s>>>(p, L, O, from32);
+    large_check_kernel<true><<<L.nrows, kTileRows, 0, s>>>(p, L, O, from32);
+    large_check_result_kernel<<<nb, 128, 0, s>>>(p, L, tol, feasible, max_overlap);
+  }
   return cudaGetLastError();
 }
 

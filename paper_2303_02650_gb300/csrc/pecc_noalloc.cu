@@ -54,7 +54,7 @@ __global__ void noalloc_feasible_kernel(unsigned char *scratch, const double *__
   // the build zeroes the cell counters it uses and overwrites everything else it reads
   const int tot = cta_build_neighbors<double, int32_t>(
       x, n, G, lc2, (uint32_t *)(scratch + kOffKey), (int32_t *)(scratch + kOffOrd), (int32_t *)(scratch + kOffCells),
-      (double2 *)(scratch + kOffXs), rp, col, cap, sh, nullptr, false);
+      (double2 *)(scratch + kOffXs), rp, col, cap, sh, nullptr);
   double m = 0.0;
   int bad = 0;
   if (tot <= cap) {
