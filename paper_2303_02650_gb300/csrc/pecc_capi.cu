@@ -1133,7 +1133,7 @@ pecc_status pecc_features(pecc_ctx *ctx, const float *unused, float *feat_dev) {
   pecc_status s = need_fp32(ctx);
   if (s) return s;
   if (ctx->total > 0 && !feat_dev) return fail(ctx, PECC_ERR_ARG, "feat_dev is NULL");
-  CK(mlp_features(sparams(ctx), feat_dev, ctx->stream));
+  CK(mlp_features(sparams(ctx), ctx->lt, ctx->n_small, feat_dev, ctx->stream));
   return PECC_OK;
 }
 
@@ -1159,7 +1159,7 @@ pecc_status pecc_warm_start_ex(pecc_ctx *ctx, pecc_mlp *mlp, int32_t rounds, dou
   for (int r = 0; r < rounds; ++r) {
     CK(launch_build(sp, ctx->lt, ctx->n_small, ctx->num_sms, 1, 1, nullptr, ctx->stream));
     CK(energy_grad_launch(ctx, sp, 1, ctx->Eb, ctx->g));
-    CK(mlp_features(sp, ctx->feat, ctx->stream));
+    CK(mlp_features(sp, ctx->lt, ctx->n_small, ctx->feat, ctx->stream));
     CK(mlp_forward(mlp->wb, mlp->params, ctx->feat, ctx->total, ctx->dout, mlp->sms, ctx->stream));
     CK(mlp_apply(sp, ctx->dout, ctx->backup, (float)max_move, ctx->stream));
     CK(launch_build(sp, ctx->lt, ctx->n_small, ctx->num_sms, 1, 1, nullptr, ctx->stream));

@@ -265,6 +265,9 @@ cudaError_t launch_set_radius(InstDesc *desc, const double *R, int num, double l
 // n_small: the largest instance of at most kCellsBlockN circles (-1: none)
 cudaError_t launch_build(const StandaloneParams &p, const LargeTiles &L, int n_small, int sms, int prec, int force,
                          int32_t *rebuilt, cudaStream_t s);
+// cells, order and sorted coordinates of the larger instances' binary32 layouts into ckey_t, corder_t
+// and xtmp (float2 per circle)
+cudaError_t launch_large_cells32(const StandaloneParams &p, const LargeTiles &L, cudaStream_t s);
 cudaError_t launch_energy_grad(const StandaloneParams &p, int eval, double *E, void *grad, void *ecirc,
                                int max_small_n, bool any_large, cudaStream_t s);
 cudaError_t launch_feasible(const StandaloneParams &p, const LargeTiles &L, int n_small, int sms, int from32,
@@ -283,7 +286,7 @@ int mlp_num_bf16();
 int mlp_train_blocks(int sms);
 cudaError_t mlp_init(float *params, __nv_bfloat16 *wb, uint64_t seed, cudaStream_t s);
 cudaError_t mlp_sync_bf16(const float *params, __nv_bfloat16 *wb, cudaStream_t s);
-cudaError_t mlp_features(const StandaloneParams &p, float *feat, cudaStream_t s);
+cudaError_t mlp_features(const StandaloneParams &p, const LargeTiles &L, int n_small, float *feat, cudaStream_t s);
 cudaError_t mlp_targets(const StandaloneParams &p, const double *xbefore, float *target, cudaStream_t s);
 cudaError_t mlp_forward(const __nv_bfloat16 *wb, const float *params, const float *feat, int64_t rows, float *out,
                         int sms, cudaStream_t s, float *trace = nullptr);

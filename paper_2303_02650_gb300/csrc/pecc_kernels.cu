@@ -969,6 +969,10 @@ cudaError_t launch_build(const StandaloneParams &p, const LargeTiles &L, int n_s
                    : build_t<double>(p, L, n_small, sms, force, rebuilt, s);
 }
 
+cudaError_t launch_large_cells32(const StandaloneParams &p, const LargeTiles &L, cudaStream_t s) {
+  return large_cells<float, false>(p, L, LargeDest{p.ckey_t, p.corder_t, (float2 *)p.xtmp}, 0, 1, nullptr, s);
+}
+
 template <class A> static cudaError_t launch_eg_block(const StandaloneParams &p, int stage_n, size_t smem,
                                                      void *grad, double *E, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(energy_grad_block_kernel<A>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -12,6 +12,7 @@
 // displacement in the same frame.
 #include <cuda_bf16.h>
 
+#include "pecc_cells.cuh"
 #include "pecc_internal.h"
 #include "pecc_tc.cuh"
 
@@ -47,72 +48,122 @@ __device__ __forceinline__ float2 frame_er(float2 c) {
   return make_float2(__fdiv_rn(c.x, r), __fdiv_rn(c.y, r));
 }
 
-// One block per instance: cell sort (grid side >= 2.5, so 4.5 is within two cells), then per
-// circle the 12 nearest within 4.5 and the wall distance.
-__global__ void features_kernel(StandaloneParams P, float *feat) {
-  __shared__ int32_t sh[40];
-  const int q = blockIdx.x;
-  const InstDesc D = P.desc[q];
-  const int n = D.n;
-  const float2 *x = P.x32 + D.off;
-  float2 *xs = (float2 *)P.xtmp + D.off;
-  const CellGrid G{D.R, D.inv_cs, 0.f, 0.f, D.ncx, false};
-  uint32_t *ckey = P.ckey_t + D.off;
-  int32_t *corder = P.corder_t + D.off;
-  int32_t *cells = P.cells + D.cell_off;
-  cta_cell_sort<float>(x, n, G, ckey, corder, cells, xs, sh);
-  const int nc = G.nc;
-  const float Rf = (float)D.R;
-  for (int q0 = threadIdx.x; q0 < n; q0 += blockDim.x) {
-    const int i = corder[q0];
-    const float2 xi = xs[q0];
-    const uint32_t key = ckey[i];
-    const int cx = (int)(key % (uint32_t)nc), cy = (int)(key / (uint32_t)nc);
-    float bs[KNN];
-    int bj[KNN];
-    float bx[KNN], by[KNN];
+// A lane takes one circle: it collects the circles within 4.5 (at most two cells away: the grid's side
+// is at least 2.5) as positions in a column of its warp's buffer, then keeps the twelve least (squared
+// distance, index) of them as ascending 64-bit keys: the distance's bits, then the index (and, where
+// both fit 16 bits, the sorted position, which gives the coordinates without a search).  Collecting first
+// lets the insertions of a warp's lanes run together.  The warp's 32 rows of 25 values leave through
+// shared memory as one contiguous piece.
+constexpr int kKnnBuf = 32;                               // collected per lane before they are inserted
+constexpr int kKnnWarpBytes = 32 * F * (int)sizeof(float);  // the rows of a warp
+static_assert(kKnnWarpBytes >= 32 * kKnnBuf * (int)sizeof(uint16_t), "the rows take the 16-bit buffer's place");
+static_assert(kKnnWarpBytes <= 32 * kKnnBuf * (int)sizeof(int32_t), "and fit the 32-bit one's");
+
+// I: type of the sorted order's entries (16-bit: keys carry the position).
+template <typename I>
+__device__ __forceinline__ void feature_rows(const float2 *__restrict__ x, int n, int i, float Rf, int key, int nc,
+                                             const int32_t *start, const float2 *xs, const I *ord, void *scratch,
+                                             float *__restrict__ feat) {
+  constexpr bool pack = sizeof(I) == 2;
+  const int lane = threadIdx.x & 31;
+  const bool act = i < n;
+  unsigned long long best[KNN];
 #pragma unroll
-    for (int u = 0; u < KNN; ++u) { bs[u] = 3.0e38f; bj[u] = 0x7fffffff; bx[u] = 0.f; by[u] = 0.f; }
-    const int bx0 = max(cx - 2, 0), bx1 = min(cx + 2, nc - 1);
-    for (int yy = max(cy - 2, 0); yy <= min(cy + 2, nc - 1); ++yy) {
-      const int lo = cells[yy * nc + bx0], hi = cells[yy * nc + bx1 + 1];
-      for (int qq = lo; qq < hi; ++qq) {
-        if (qq == q0) continue;
-        const float2 xj = xs[qq];
-        const float dx = __fsub_rn(xj.x, xi.x), dy = __fsub_rn(xj.y, xi.y);
-        const float s = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
-        if (!(s < kKnnR2)) continue;
-        const int j = corder[qq];
-        if (s > bs[KNN - 1] || (s == bs[KNN - 1] && j > bj[KNN - 1])) continue;
-        // insert (s, j) into the ascending list (compare-swap down the unrolled list)
-        float cs = s, cxv = dx, cyv = dy;
-        int cj = j;
+  for (int u = 0; u < KNN; ++u) best[u] = ~0ull;
+  const float2 xi = act ? x[i] : make_float2(0.f, 0.f);
+  if (act) {
+    I *buf = (I *)scratch + lane;
+    int cnt = 0;
+    auto dist2 = [&](int q) {
+      const float2 xj = xs[q];
+      const float dx = __fsub_rn(xj.x, xi.x), dy = __fsub_rn(xj.y, xi.y);
+      return __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
+    };
+    auto insert_all = [&]() {
+      for (int h = 0; h < cnt; ++h) {
+        const int q = (int)buf[32 * h];
+        const int j = (int)ord[q];
+        if (j == i) continue;
+        unsigned long long k = ((unsigned long long)__float_as_uint(dist2(q)) << 32) |
+                               (pack ? ((unsigned)j << 16) | (unsigned)q : (unsigned)j);
 #pragma unroll
         for (int u = 0; u < KNN; ++u) {
-          const bool less = cs < bs[u] || (cs == bs[u] && cj < bj[u]);
-          if (less) {
-            float ts = bs[u], tx = bx[u], ty = by[u];
-            int tj = bj[u];
-            bs[u] = cs; bj[u] = cj; bx[u] = cxv; by[u] = cyv;
-            cs = ts; cj = tj; cxv = tx; cyv = ty;
-          }
+          const unsigned long long b = best[u];
+          const bool less = k < b;
+          best[u] = less ? k : b;
+          k = less ? b : k;
         }
       }
+      cnt = 0;
+    };
+    const int cy = key / nc, cx = key - cy * nc;
+    const int bx0 = max(cx - 2, 0), bx1 = min(cx + 2, nc - 1);
+    for (int yy = max(cy - 2, 0); yy <= min(cy + 2, nc - 1); ++yy) {
+      const int lo = start[yy * nc + bx0], hi = start[yy * nc + bx1 + 1];
+      for (int q = lo; q < hi; ++q) {
+        if (!(dist2(q) < kKnnR2)) continue;
+        buf[32 * cnt] = (I)q;
+        if (++cnt == kKnnBuf) insert_all();
+      }
     }
+    insert_all();
+  }
+  __syncwarp();  // the rows take the buffer's place
+  float *rows = (float *)scratch;
+  if (act) {
     const float2 er = frame_er(xi);
-    float *f = feat + (size_t)(D.off + i) * F;
+    float *f = rows + F * lane;
 #pragma unroll
     for (int u = 0; u < KNN; ++u) {
-      const bool has = bj[u] != 0x7fffffff;
-      const float fu = has ? __fadd_rn(__fmul_rn(bx[u], er.x), __fmul_rn(by[u], er.y)) : 0.f;
-      const float fv = has ? __fsub_rn(__fmul_rn(by[u], er.x), __fmul_rn(bx[u], er.y)) : 0.f;
-      f[2 * u] = fu;
-      f[2 * u + 1] = fv;
+      const bool has = best[u] != ~0ull;
+      float2 xj = xi;
+      if (has) xj = pack ? xs[best[u] & 0xffffu] : x[best[u] & 0xffffffffu];
+      const float dx = __fsub_rn(xj.x, xi.x), dy = __fsub_rn(xj.y, xi.y);
+      f[2 * u] = has ? __fadd_rn(__fmul_rn(dx, er.x), __fmul_rn(dy, er.y)) : 0.f;
+      f[2 * u + 1] = has ? __fsub_rn(__fmul_rn(dy, er.x), __fmul_rn(dx, er.y)) : 0.f;
     }
     const float r = __fsqrt_rn(__fadd_rn(__fmul_rn(xi.x, xi.x), __fmul_rn(xi.y, xi.y)));
     const float b = __fsub_rn(__fsub_rn(Rf, r), 1.0f);
     f[24] = fminf(b, 4.5f);
   }
+  __syncwarp();
+  const int i0 = i - lane, m = min(32, n - i0) * F;
+  for (int t = lane; t < m; t += 32) feat[(size_t)i0 * F + t] = rows[t];
+  __syncwarp();
+}
+
+// Instances of at most kCellsBlockN circles, one block each (pecc_cells.cuh).  Bound by instruction issue
+// of the collecting and inserting walks: 142 us for 665 000 circles in 1024 instances, 460 us when cells
+// and lists lay in global memory and every lane inserted as it walked.
+__global__ void __launch_bounds__(256) features_block_kernel(StandaloneParams P, float *feat) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ int32_t sh[40];
+  const int q = P.eorder[blockIdx.x];
+  const InstDesc &D = P.desc[q];
+  const int n = D.n;
+  if (n > kCellsBlockN) return;
+  const Coords<float> X{P.x32 + D.off, P.l_cut};
+  const size_t extra = (size_t)(blockDim.x >> 5) * kKnnWarpBytes;
+  const BlockCells C = block_cells<float>(X, n, D.R, D.inv_cs, D.ncx, sm, extra, P.cells + D.cell_off, nullptr, nullptr,
+                                          sh, [](int, float2) {});
+  void *scratch = C.extra + (threadIdx.x >> 5) * kKnnWarpBytes;
+  for (int i0 = threadIdx.x & ~31; i0 < n; i0 += blockDim.x) {
+    const int i = i0 + (threadIdx.x & 31);
+    feature_rows<uint16_t>(X.x, n, i, (float)D.R, i < n ? (int)C.key[i] : 0, D.ncx, C.start, C.xs, C.ord, scratch,
+                           feat + (size_t)D.off * F);
+  }
+}
+
+// Tiles of the larger instances, over the cells that launch_large_cells32 left in the scratch.
+__global__ void __launch_bounds__(kTileRows) features_tile_kernel(StandaloneParams P, LargeTiles L, float *feat) {
+  __shared__ __align__(16) unsigned char sm[(kTileRows / 32) * 32 * kKnnBuf * 4];
+  const int2 t = L.rows[blockIdx.x];
+  const InstDesc &D = P.desc[t.x];
+  const int n = D.n, i = t.y * kTileRows + threadIdx.x;
+  if (i - (int)(threadIdx.x & 31) >= n) return;  // the whole warp
+  feature_rows<int32_t>(P.x32 + D.off, n, i, (float)D.R, i < n ? (int)P.ckey_t[D.off + i] : 0, D.ncx,
+                        P.cells + D.cell_off, (const float2 *)P.xtmp + D.off, P.corder_t + D.off,
+                        sm + (threadIdx.x >> 5) * 32 * kKnnBuf * 4, feat + (size_t)D.off * F);
 }
 
 // Target of circle i: its displacement from x_before to now, in the frame of x_before.
@@ -648,8 +699,20 @@ cudaError_t mlp_sync_bf16(const float *params, bf16 *wb, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t mlp_features(const StandaloneParams &p, float *feat, cudaStream_t s) {
-  if (p.num > 0) features_kernel<<<p.num, 256, 0, s>>>(p, feat);
+cudaError_t mlp_features(const StandaloneParams &p, const LargeTiles &L, int n_small, float *feat, cudaStream_t s) {
+  if (p.num <= 0) return cudaSuccess;
+  if (n_small >= 0) {
+    const int block = n_small <= 64 ? 64 : (n_small <= 128 ? 128 : 256);
+    const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kKnnWarpBytes);
+    cudaError_t e = cudaFuncSetAttribute(features_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    features_block_kernel<<<p.num, block, smem, s>>>(p, feat);
+  }
+  if (L.nrows > 0) {
+    cudaError_t e = launch_large_cells32(p, L, s);
+    if (e != cudaSuccess) return e;
+    features_tile_kernel<<<L.nrows, kTileRows, 0, s>>>(p, L, feat);
+  }
   return cudaGetLastError();
 }
 

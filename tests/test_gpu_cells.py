@@ -6,6 +6,7 @@ for bit."""
 import numpy as np
 import pytest
 
+from oracle import mlp as omlp
 from paper_2303_02650_gb300 import synth
 from gpu_util import need_gpu, split
 
@@ -103,3 +104,22 @@ def test_check_nonfinite_overflow_and_near_contact(orc, sizes):
             assert np.isnan(mo2[q]) and feas2[q] == 0
         else:
             assert mo2[q] == ref
+
+
+@pytest.mark.parametrize("sizes", [[1, 64, 65, 2047, 2048], [2049, 2305], [300, 2600, 0, 12]])
+@pytest.mark.parametrize("kind,u", [("plain", 0.83), ("clusters", 0.83), ("grid", 0.83), ("plain", 0.02)])
+def test_features_at_the_edges(sizes, kind, u):
+    """The 25 features bit for bit: full and short rows, more than 32 circles within 4.5 (the buffer
+    of a lane is emptied on the way), equal distances (index order), coincident circles."""
+    torch, pecc = need_gpu()
+    n = np.array(sizes, dtype=np.int32)
+    R = np.array([synth.radius(max(int(v), 1), u) for v in n])
+    xy = _layout(n, R, 23, kind)
+    with pecc.Context(n, precision=1) as c:
+        c.set_radius(R)
+        c.set_positions(torch.from_numpy(xy))
+        xy = c.get_positions().cpu().numpy().astype(np.float32)
+        f = c.features().cpu().numpy()
+    for q, (fq, xq) in enumerate(zip(split(f, n), split(xy, n))):
+        if n[q]:
+            assert np.array_equal(fq, omlp.features(xq, float(R[q]))), q
