@@ -181,9 +181,9 @@ __global__ void targets_kernel(StandaloneParams P, const double *__restrict__ xb
 // ------------------------------------------------------------------ tensor-core network ----
 // Both kernels below keep every weight and activation tile in shared memory in the core layout of
 // pecc_tc.cuh and run the 128-wide GEMMs as tcgen05 MMAs (M = 128 rows of a tile, K = 16 per
-// instruction) issued by thread 0, with FP32 accumulators in TMEM; thread t of the 128 owns row t
-// of a tile (TMEM lane t) in every epilogue.  The 2-wide output layer and its gradient run on the
-// CUDA cores inside the epilogues.
+// instruction) issued by one thread, with FP32 accumulators in TMEM; a thread owns a row of a tile
+// (TMEM lane r) in every epilogue, or a quarter of its columns.  The 2-wide output layer runs on the CUDA
+// cores inside the epilogues.
 constexpr int TM = 128;                  // rows per tile
 constexpr int FPAD = 32;                 // padded input width
 constexpr uint32_t kW1B = TM * FPAD * 2;  // bytes of a [128][32] bf16 core tile
@@ -192,7 +192,8 @@ constexpr long long kWaitNs = 2000000000ll;  // bound of every wait on the MMA b
 constexpr uint32_t kColStep = 2 * 128;       // a K step of 16 along the columns: two cores
 
 // weights of the block: W1 [128][32], W2, W3 [128][128] in the core layout, from the padded bf16
-// copies; biases b1 b2 b3 [128], the output layer W4 [2][128] (bf16 values) and b4 [2] as floats
+// copies; biases b1 b2 b3 [128], the output layer W4 (bf16 values; both rows' entries of a column side
+// by side: [128][2]) and b4 [2] as floats
 __device__ void tc_load_weights(const bf16 *__restrict__ wb, const float *__restrict__ params, unsigned char *w1,
                                 unsigned char *w2, unsigned char *w3, float *fb) {
   for (int u = threadIdx.x; u < TM * (FPAD / 8); u += blockDim.x) {
@@ -208,373 +209,473 @@ __device__ void tc_load_weights(const bf16 *__restrict__ wb, const float *__rest
     fb[u] = params[OB1 + u];
     fb[H + u] = params[OB2 + u];
     fb[2 * H + u] = params[OB3 + u];
-    fb[3 * H + u] = __bfloat162float(wb[BW4 + u]);
-    fb[4 * H + u] = __bfloat162float(wb[BW4 + SA + u]);
+    fb[3 * H + 2 * u] = __bfloat162float(wb[BW4 + u]);
+    fb[3 * H + 2 * u + 1] = __bfloat162float(wb[BW4 + SA + u]);
   }
   if (threadIdx.x < 2) fb[5 * H + threadIdx.x] = params[OB4 + threadIdx.x];
 }
 
-// row r of the tile's input: the 25 features of global row gr (zero past rows and past column 25)
-__device__ __forceinline__ void tc_load_row(const float *__restrict__ feat, int64_t gr, int64_t rows, int r,
-                                            unsigned char *x) {
+// Two floats rounded to bf16, low half first, and back.
+__device__ __forceinline__ uint32_t pack2f(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);  // one conversion instruction
+  return *(const uint32_t *)&v;
+}
+__device__ __forceinline__ float lo2f(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float hi2f(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+
+// 32 bf16 values (16 words) of row r starting at column c0 of a [128][C] core tile
+__device__ __forceinline__ void tc_store32(unsigned char *t, int r, int c0, int C, const uint32_t (&w)[16]) {
 #pragma unroll
-  for (int c8 = 0; c8 < FPAD / 8; ++c8) {
-    uint32_t w[4];
+  for (int c8 = 0; c8 < 4; ++c8)
+    *(uint4 *)(t + tc::core_off(r, c0 + 8 * c8, C)) = make_uint4(w[4 * c8], w[4 * c8 + 1], w[4 * c8 + 2], w[4 * c8 + 3]);
+}
+__device__ __forceinline__ void trace32(float *t, const uint32_t (&w)[16]) {
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const int c = 8 * c8 + 2 * h;
-      const float a = (gr < rows && c < F) ? feat[gr * F + c] : 0.f;
-      const float b = (gr < rows && c + 1 < F) ? feat[gr * F + c + 1] : 0.f;
-      w[h] = pack2(__float2bfloat16_rn(a), __float2bfloat16_rn(b));
-    }
-    *(uint4 *)(x + tc::core_off(r, 8 * c8, FPAD)) = make_uint4(w[0], w[1], w[2], w[3]);
+  for (int j = 0; j < 16; ++j) {
+    t[2 * j] = lo2f(w[j]);
+    t[2 * j + 1] = hi2f(w[j]);
   }
 }
 
-// 32 bf16 values of row r starting at column c0 of a [128][128] core tile
-__device__ __forceinline__ void tc_store32(unsigned char *t, int r, int c0, const float (&v)[32]) {
+// Hidden layer, columns [c0, c0 + 32) of this thread's row: accumulator plus bias, ReLU, rounded to bf16.
+__device__ __forceinline__ void tc_hidden32(uint32_t taddr, const float *bias, uint32_t (&w)[16]) {
+  float v[32];
+  tc::ld32(taddr, v);
 #pragma unroll
-  for (int c8 = 0; c8 < 4; ++c8) {
-    uint32_t w[4];
-#pragma unroll
-    for (int h = 0; h < 4; ++h)
-      w[h] = pack2(__float2bfloat16_rn(v[8 * c8 + 2 * h]), __float2bfloat16_rn(v[8 * c8 + 2 * h + 1]));
-    *(uint4 *)(t + tc::core_off(r, c0 + 8 * c8, H)) = make_uint4(w[0], w[1], w[2], w[3]);
+  for (int j = 0; j < 8; ++j) {
+    const float4 b = *(const float4 *)(bias + 4 * j);
+    w[2 * j] = pack2f(fmaxf(v[4 * j] + b.x, 0.f), fmaxf(v[4 * j + 1] + b.y, 0.f));
+    w[2 * j + 1] = pack2f(fmaxf(v[4 * j + 2] + b.z, 0.f), fmaxf(v[4 * j + 3] + b.w, 0.f));
   }
 }
-__device__ __forceinline__ float tc_get(const unsigned char *t, int r, int c, int C) {
-  return __bfloat162float(*(const bf16 *)(t + tc::core_off(r, c, C)));
+// The output layer over 32 columns: o0 / o1 += h W4^T from the rounded values, columns in order.
+__device__ __forceinline__ void tc_out32(const uint32_t (&w)[16], const float *w4, float &o0, float &o1) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const float4 a = *(const float4 *)(w4 + 4 * j);
+    o0 = fmaf(lo2f(w[j]), a.x, o0);
+    o1 = fmaf(lo2f(w[j]), a.y, o1);
+    o0 = fmaf(hi2f(w[j]), a.z, o0);
+    o1 = fmaf(hi2f(w[j]), a.w, o1);
+  }
 }
 
-// Thread 0 issues D = A B^T over K (K / 16 MMAs) and commits them to the barrier.  The operand
-// descriptors advance by `astep` / `bstep` bytes per K step of 16.
+// One thread issues D = A B^T over K (K / 16 MMAs).  The operand descriptors advance by `astep` /
+// `bstep` bytes per K step of 16.
 __device__ __forceinline__ void tc_gemm(uint32_t d, uint32_t a_addr, bool a_krows, int a_cols, uint32_t astep,
                                         uint32_t b_addr, bool b_krows, int b_cols, uint32_t bstep, int N, int K,
                                         bool accumulate) {
   const uint32_t id = tc::idesc_bf16(TM, N, a_krows ? 1 : 0, b_krows ? 1 : 0);
-  for (int ks = 0; ks < K / 16; ++ks) {
-    const uint32_t aa = a_addr + ks * astep, ba = b_addr + ks * bstep;
-    const uint64_t ad = a_krows ? tc::desc_k_rows(aa, a_cols) : tc::desc_k_cols(aa, a_cols);
-    const uint64_t bd = b_krows ? tc::desc_k_rows(ba, b_cols) : tc::desc_k_cols(ba, b_cols);
+  uint64_t ad = a_krows ? tc::desc_k_rows(a_addr, a_cols) : tc::desc_k_cols(a_addr, a_cols);
+  uint64_t bd = b_krows ? tc::desc_k_rows(b_addr, b_cols) : tc::desc_k_cols(b_addr, b_cols);
+#pragma unroll
+  for (int ks = 0; ks < K / 16; ++ks) {  // the start address is the descriptors' low field, in 16-byte units
     tc::mma(d, ad, bd, id, (accumulate || ks > 0) ? 1 : 0);
+    ad += astep >> 4;
+    bd += bstep >> 4;
   }
 }
 
-// Make this block's shared-memory writes visible to the tensor cores and order TMEM accesses around
-// a block barrier.
-__device__ __forceinline__ void tc_sync() {
+// Barrier of one 128-thread group of the block (named barrier 1 + g; g < 0: of the block); whether any of
+// its threads passed bad.
+__device__ __forceinline__ bool group_any(bool bad, int g) {
+  if (g < 0) return __syncthreads_or(bad);
+  uint32_t any;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.b32 p, %1, 0;\nbarrier.cta.red.or.pred q, %2, 128, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(any)
+      : "r"((uint32_t)bad), "r"(1 + g)
+      : "memory");
+  return any != 0;
+}
+
+// Make this group's shared-memory writes visible to the tensor cores and order TMEM accesses around a
+// barrier of the group (g < 0: of the block).  ok: this thread's waits so far ended in time; returns
+// whether all threads' did.
+__device__ __forceinline__ bool tc_sync(bool ok = true, int g = -1) {
   tc::fence_smem_to_async();
   tc::fence_before();
-  __syncthreads();
+  const bool any = group_any(!ok, g);
   tc::fence_after();
+  return !any;
 }
 
-// Thread 0 commits the MMAs issued so far and waits for them; every thread learns whether the wait
-// ended in time (block-uniform).
-__device__ __forceinline__ bool tc_commit_wait(uint64_t *mbar, uint32_t &phase, int *flag) {
-  if (threadIdx.x == 0) {
-    tc::commit(mbar);
-    *flag = tc::mbar_wait(mbar, phase, kWaitNs) ? 0 : 1;
-  }
+// Every thread waits for the barrier's current phase itself (a wait that runs out is reported to the
+// group at its next barrier, so that all of them leave together).
+__device__ __forceinline__ bool tc_wait(uint64_t *mbar, uint32_t &phase) {
+  const bool ok = tc::mbar_wait(mbar, phase, kWaitNs);
   phase ^= 1u;
-  tc::fence_before();
-  __syncthreads();
+  __syncwarp();  // the TMEM loads that follow are warp-wide instructions
   tc::fence_after();
-  return *flag == 0;
+  return ok;
 }
 
-// Epilogue of a hidden layer: this thread's row of the accumulator plus bias, ReLU, rounded to bf16
-// into tile `t` (and, if set, the rounded values to trace[0..128)); with w4, also the output layer
-// o0 / o1 += h W4^T from the rounded values.
-__device__ __forceinline__ void tc_hidden_epilogue(uint32_t tacc, const float *bias, unsigned char *t, float *trace,
-                                                   const float *w4, float &o0, float &o1) {
-  const int r = threadIdx.x;
-  for (int c0 = 0; c0 < H; c0 += 32) {
-    float v[32];
-    tc::ld32(tacc + ((uint32_t)(r & ~31) << 16) + (uint32_t)c0, v);
+// Forward: out[rows][2] for rows of feat[rows][25]; trace (may be null): float[rows][3][128], the bf16
+// activations of the three hidden layers.  One block per SM, four groups of 128 threads that share the
+// weights; each group takes a tile of 128 rows at a time through the chain MMA, epilogue, MMA by itself,
+// so that three tiles' epilogues run while another's MMAs do.  A group's tile of inputs and its hidden
+// activations take the same 32 KB (the inputs are dead once the first MMAs are done).  The features of
+// the next tile are loaded, coalesced, while the last layer runs.
+// 665 000 rows: 98 us, bound by shared-memory wavefronts and issue of the epilogues; 283 us with one group
+// per SM and row-wise feature loads.
+constexpr int kFwdGroups = 4;
+constexpr int kRowLoads = F;  // 32 rows of F floats per warp, one per lane and load
+constexpr uint32_t kFwdW1 = 0, kFwdW2 = kFwdW1 + kW1B, kFwdW3 = kFwdW2 + kHB, kFwdT = kFwdW3 + kHB,
+                   kFwdF = kFwdT + kFwdGroups * kHB, kFwdBar = kFwdF + (5 * H + 4) * 4;
+constexpr size_t kFwdSmem = (size_t)kFwdBar + 8 * kFwdGroups + 16 + 128;  // barriers, TMEM address; alignment
+
+// the warp's 32 rows from row0 on, coalesced: float e = lane + 32 u of the 800 (zero past rows)
+__device__ __forceinline__ void load_rows32(const float *__restrict__ feat, int64_t row0, int64_t rows, float (&v)[kRowLoads]) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n = min((int64_t)32, rows - row0) * F;  // floats that exist (<= 0 past the end)
 #pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __bfloat162float(__float2bfloat16_rn(fmaxf(v[j] + bias[c0 + j], 0.f)));
-    if (t) tc_store32(t, r, c0, v);
-    if (trace)
+  for (int u = 0; u < kRowLoads; ++u) {
+    const int e = lane + 32 * u;
+    v[u] = e < n ? __ldg(feat + row0 * F + e) : 0.f;
+  }
+}
+// ... to the [128][32] core tile x, rows r0 .. r0 + 31; columns 25 .. 31 zero
+__device__ __forceinline__ void store_rows32(unsigned char *x, int r0, const float (&v)[kRowLoads]) {
+  const int lane = threadIdx.x & 31;
+  *(uint4 *)(x + tc::core_off(r0 + lane, 24, FPAD)) = make_uint4(0u, 0u, 0u, 0u);
+  __syncwarp();
+  int row = lane / F, c = lane % F;
 #pragma unroll
-      for (int j = 0; j < 32; ++j) trace[c0 + j] = v[j];
-    if (w4)
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        o0 = fmaf(v[j], w4[c0 + j], o0);
-        o1 = fmaf(v[j], w4[H + c0 + j], o1);
-      }
+  for (int u = 0; u < kRowLoads; ++u) {
+    *(bf16 *)(x + tc::core_off(r0 + row, c, FPAD)) = __float2bfloat16_rn(v[u]);
+    c += 32 - F;
+    row += 1;
+    if (c >= F) { c -= F; row += 1; }
   }
 }
 
-constexpr uint32_t kFwdW1 = 0, kFwdW2 = kFwdW1 + kW1B, kFwdW3 = kFwdW2 + kHB, kFwdX = kFwdW3 + kHB,
-                   kFwdH = kFwdX + kW1B, kFwdF = kFwdH + kHB, kFwdBar = kFwdF + (5 * H + 2) * 4 + 8;
-constexpr size_t kFwdSmem = (size_t)kFwdBar + 16 + 1024;  // + the barrier, TMEM address, flag; + alignment slack
-
-// Forward: out[rows][2] for rows of feat[rows][25]; trace (may be null): float[rows][3][128], the
-// bf16 activations of the three hidden layers.  Persistent over tiles of 128 rows.
-__global__ void __launch_bounds__(128, 1) forward_tc_kernel(const bf16 *__restrict__ wb, const float *__restrict__ params,
-                                                             const float *__restrict__ feat, int64_t rows, float *out,
-                                                             float *trace) {
+__global__ void __launch_bounds__(128 * kFwdGroups, 1)
+forward_tc_kernel(const bf16 *__restrict__ wb, const float *__restrict__ params, const float *__restrict__ feat,
+                  int64_t rows, float *out, float *trace) {
   extern __shared__ unsigned char sm_raw[];
-  unsigned char *sm = (unsigned char *)(((uintptr_t)sm_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char *w1 = sm + kFwdW1, *w2 = sm + kFwdW2, *w3 = sm + kFwdW3, *x = sm + kFwdX, *h = sm + kFwdH;
+  unsigned char *sm = (unsigned char *)(((uintptr_t)sm_raw + 127) & ~(uintptr_t)127);
+  unsigned char *w1 = sm + kFwdW1, *w2 = sm + kFwdW2, *w3 = sm + kFwdW3;
   float *fb = (float *)(sm + kFwdF);
-  uint64_t *mbar = (uint64_t *)(sm + kFwdBar);
-  uint32_t *tslot = (uint32_t *)(mbar + 1);
-  int *flag = (int *)(tslot + 1);
-  const int r = threadIdx.x;
+  const int g = threadIdx.x >> 7, r = threadIdx.x & 127, r0 = r & ~31;
+  uint64_t *mbar = (uint64_t *)(sm + kFwdBar) + g;
+  uint32_t *tslot = (uint32_t *)(sm + kFwdBar + 8 * kFwdGroups);
+  unsigned char *h = sm + kFwdT + g * kHB;
+  const bool issuer = r == 0;
   tc_load_weights(wb, params, w1, w2, w3, fb);
-  if (r == 0) { tc::mbar_init(mbar); *flag = 0; }
-  if (r < 32) tc::tmem_alloc<128>(tslot);
+  if (issuer) tc::mbar_init(mbar);
+  if (threadIdx.x < 32) tc::tmem_alloc<128 * kFwdGroups>(tslot);
   tc_sync();
-  const uint32_t tacc = *tslot;
-  const uint32_t sw1 = tc::smem_u32(w1), sw2 = tc::smem_u32(w2), sw3 = tc::smem_u32(w3), sx = tc::smem_u32(x),
-                 sh = tc::smem_u32(h);
+  const uint32_t tacc = *tslot + 128 * g, lanes = (uint32_t)r0 << 16;
+  const uint32_t sw1 = tc::smem_u32(w1), sw2 = tc::smem_u32(w2), sw3 = tc::smem_u32(w3), sh = tc::smem_u32(h);
   uint32_t phase = 0;
   bool ok = true;
-  const int64_t tiles = (rows + TM - 1) / TM;
-  for (int64_t tl = blockIdx.x; tl < tiles && ok; tl += gridDim.x) {
+  const int64_t tiles = (rows + TM - 1) / TM, stride = (int64_t)gridDim.x * kFwdGroups;
+  int64_t tl = (int64_t)g * gridDim.x + blockIdx.x;  // the first tiles go to different SMs
+  float v[kRowLoads];
+  if (tl < tiles) load_rows32(feat, tl * TM + r0, rows, v);
+  for (; tl < tiles; tl += stride) {
     const int64_t gr = tl * TM + r;
     float *tr = (trace && gr < rows) ? trace + gr * 3 * H : nullptr;
-    tc_load_row(feat, gr, rows, r, x);
-    tc_sync();
-    if (r == 0) tc_gemm(tacc, sx, false, FPAD, kColStep, sw1, false, FPAD, kColStep, H, FPAD, false);
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
+    store_rows32(h, r0, v);
+    if (!(ok = tc_sync(ok, g))) break;
+    if (issuer) { tc_gemm(tacc, sh, false, FPAD, kColStep, sw1, false, FPAD, kColStep, H, FPAD, false); tc::commit(mbar); }
+    ok = tc_wait(mbar, phase);
     float o0 = 0.f, o1 = 0.f;
-    tc_hidden_epilogue(tacc, fb, h, tr, nullptr, o0, o1);
-    tc_sync();
-    if (r == 0) tc_gemm(tacc, sh, false, H, kColStep, sw2, false, H, kColStep, H, H, false);
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
-    tc_hidden_epilogue(tacc, fb + H, h, tr ? tr + H : nullptr, nullptr, o0, o1);
-    tc_sync();
-    if (r == 0) tc_gemm(tacc, sh, false, H, kColStep, sw3, false, H, kColStep, H, H, false);
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
-    tc_hidden_epilogue(tacc, fb + 2 * H, nullptr, tr ? tr + 2 * H : nullptr, fb + 3 * H, o0, o1);
+    for (int layer = 0; layer < 2; ++layer) {
+      for (int c0 = 0; c0 < H; c0 += 32) {
+        uint32_t w[16];
+        tc_hidden32(tacc + lanes + (uint32_t)c0, fb + layer * H + c0, w);
+        tc_store32(h, r, c0, H, w);
+        if (tr) trace32(tr + layer * H + c0, w);
+      }
+      if (!(ok = tc_sync(ok, g))) break;
+      if (issuer) {
+        tc_gemm(tacc, sh, false, H, kColStep, layer == 0 ? sw2 : sw3, false, H, kColStep, H, H, false);
+        tc::commit(mbar);
+      }
+      if (layer == 1 && tl + stride < tiles) load_rows32(feat, (tl + stride) * TM + r0, rows, v);
+      ok = tc_wait(mbar, phase);
+    }
+    for (int c0 = 0; ok && c0 < H; c0 += 32) {
+      uint32_t w[16];
+      tc_hidden32(tacc + lanes + (uint32_t)c0, fb + 2 * H + c0, w);
+      if (tr) trace32(tr + 2 * H + c0, w);
+      tc_out32(w, fb + 3 * H + 2 * c0, o0, o1);
+    }
     if (gr < rows) {
       out[gr * 2] = o0 + fb[5 * H];
       out[gr * 2 + 1] = o1 + fb[5 * H + 1];
     }
-    tc::fence_before();
-    __syncthreads();  // every row's TMEM reads precede the next tile's MMAs
-    tc::fence_after();
   }
+  ok = !group_any(!ok, g);  // the last tile's wait
   if (!ok)  // the tensor cores did not answer in time: NaN outputs, nothing left waiting
-    for (int64_t gr = (int64_t)blockIdx.x * TM + r; gr < rows; gr += (int64_t)gridDim.x * TM) {
-      out[gr * 2] = out[gr * 2 + 1] = __int_as_float(0x7fc00000);
-    }
+    for (tl = (int64_t)g * gridDim.x + blockIdx.x; tl < tiles; tl += stride)
+      if (tl * TM + r < rows) out[(tl * TM + r) * 2] = out[(tl * TM + r) * 2 + 1] = __int_as_float(0x7fc00000);
   tc::fence_before();
   __syncthreads();
-  if (r < 32) {
+  if (threadIdx.x < 32) {
     tc::fence_after();
-    tc::tmem_free<128>(tacc);
+    tc::tmem_free<128 * kFwdGroups>(*tslot);
   }
 }
 
 // ------------------------------------------------------------------------------- training ----
-// One block per SM, persistent over tiles of 128 rows: forward (keeping X, H1, H2, H3), then
-//   dO = 2 (out - target) / rows (rounded to bf16);  dW4 += dO' H3, db4 += sum dO   (CUDA cores)
-//   dZ3 = (dO W4) o [H3 > 0]                                                         (CUDA cores)
-//   dW3 += dZ3' H2 (TMEM, across tiles);  dH2 = dZ3 W3;  dZ2 = dH2 o [H2 > 0]        (tensor cores)
-//   dW2 += dZ2' H1;  dH1 = dZ2 W2;  dZ1 = dH1 o [H1 > 0];  dW1 += dZ1' X             (tensor cores)
-//   db_l += column sums of dZ_l.  Every GEMM input is bf16 (dZ rounded like the activations).
-// The gradient accumulators dW3, dW2, dW1 stay in TMEM until the block's last tile; the block then
-// writes its partial gradient to part[block][NPAR] and its loss to loss_part[block].
+// One block of 512 threads per SM, persistent over tiles of 128 rows; in every epilogue four threads
+// share a row, 32 columns each, so that an epilogue is one TMEM load deep.  Per tile: forward (keeping X,
+// H1, H2, H3), then
+//   dO = 2 (out - target) / rows (rounded to bf16)                          (CUDA cores)
+//   dZ3 = (dO W4) o [H3 > 0]                                                (CUDA cores)
+//   dH2 = dZ3 W3, dW4 += dO' H3, dW3 += dZ3' [H2 1];  dZ2 = dH2 o [H2 > 0]  (tensor cores)
+//   dH1 = dZ2 W2, dW2 += dZ2' [H1 1];                 dZ1 = dH1 o [H1 > 0]  (tensor cores)
+//   dW1 += dZ1' [X 1]                                                       (tensor cores)
+// Every GEMM input is bf16 (dZ rounded like the activations).  The bias gradients are the columns of
+// ones: column 128 of the 144-wide H1 and H2 tiles, column 25 of X (W1 is zero there).  The ReLU masks
+// stay in registers, a word per layer.  dH2 and dH1 are issued before the weight gradients of their
+// stage, which then run behind the next epilogue; dZ2 takes H3's room for that.  The accumulators dW1 to
+// dW4 stay in TMEM until the block's last tile; the block then writes its partial gradient to
+// part[block][NPAR] and its loss to loss_part[block].
+// 333 000 rows: 159 us, bound by the chain of six MMA and epilogue stages per tile; 484 us with one
+// 128-thread group, the column sums as scalar reads of shared memory and every MMA waited for.
 // bwd_trace (may be null): float[rows][4][128], the bf16 dZ3, dZ2, dZ1 of every row, then its bf16
 // dO (2 values) and its outputs (2 values).
+constexpr int kTrT = 512;                      // threads
+constexpr int HX = H + 16;                     // columns of the H1, H2 tiles: the activations, ones, zeros
+constexpr uint32_t kHXB = TM * HX * 2, kDOB = TM * 16 * 2;
 constexpr uint32_t kTrW1 = 0, kTrW2 = kTrW1 + kW1B, kTrW3 = kTrW2 + kHB, kTrX = kTrW3 + kHB, kTrH1 = kTrX + kW1B,
-                   kTrH2 = kTrH1 + kHB, kTrH3 = kTrH2 + kHB, kTrZ = kTrH3 + kHB, kTrF = kTrZ + kHB;
-// floats after kTrF: biases and W4 (5 H + 2), dO [128][2], dW4 accumulator [2][128], bias gradient
-// accumulators db1 db2 db3 [128] and db4 [2], the loss of each warp [4]
-constexpr int kTrFdO = 5 * H + 2, kTrFdW4 = kTrFdO + 2 * TM, kTrFdb = kTrFdW4 + 2 * H, kTrFls = kTrFdb + 3 * H + 2,
-              kTrFn = kTrFls + 4;
-constexpr uint32_t kTrBar = kTrF + ((kTrFn * 4 + 15) & ~15);
-constexpr size_t kTrainSmem = (size_t)kTrBar + 16 + 1024;
+                   kTrH2 = kTrH1 + kHXB, kTrH3 = kTrH2 + kHXB, kTrZ = kTrH3 + kHB, kTrO = kTrZ + kHB,
+                   kTrF = kTrO + kDOB;
+// floats after kTrF: biases and W4 (5 H + 4), the partial outputs of the row quarters [4][128][2]
+constexpr int kTrFo = 5 * H + 4, kTrFn = kTrFo + 8 * TM;
+constexpr uint32_t kTrBar = kTrF + kTrFn * 4;  // two barriers, TMEM address
+constexpr size_t kTrainSmem = (size_t)kTrBar + 32;
+static_assert(kTrainSmem <= 227 * 1024, "one block per SM");
+constexpr int kTrLoads = (TM * F + kTrT - 1) / kTrT;
+// TMEM columns: [0, 128) the layer accumulator, then dW3 [144], dW2 [144], dW1 [32], dW4 [16]
+constexpr uint32_t kTcW3 = 128, kTcW2 = 288, kTcW1 = 448, kTcW4 = 480;
 
-__global__ void __launch_bounds__(128, 1) train_tc_kernel(const bf16 *__restrict__ wb, const float *__restrict__ params,
+__global__ void __launch_bounds__(kTrT, 1) train_tc_kernel(const bf16 *__restrict__ wb, const float *__restrict__ params,
                                                            const float *__restrict__ feat, const float *__restrict__ target,
                                                            int64_t rows, float *part, float *loss_part,
                                                            float *fwd_trace, float *bwd_trace) {
-  extern __shared__ unsigned char sm_raw[];
-  unsigned char *sm = (unsigned char *)(((uintptr_t)sm_raw + 1023) & ~(uintptr_t)1023);
+  extern __shared__ __align__(128) unsigned char sm[];
   unsigned char *w1 = sm + kTrW1, *w2 = sm + kTrW2, *w3 = sm + kTrW3, *x = sm + kTrX;
-  unsigned char *h1 = sm + kTrH1, *h2 = sm + kTrH2, *h3 = sm + kTrH3, *z = sm + kTrZ;
-  float *fb = (float *)(sm + kTrF);
-  float *dO = fb + kTrFdO, *adW4 = fb + kTrFdW4, *adb = fb + kTrFdb, *lsw = fb + kTrFls;
-  uint64_t *mbar = (uint64_t *)(sm + kTrBar);
-  uint32_t *tslot = (uint32_t *)(mbar + 1);
-  int *flag = (int *)(tslot + 1);
-  const int r = threadIdx.x, lane = r & 31, w = r >> 5;
+  unsigned char *h1 = sm + kTrH1, *h2 = sm + kTrH2, *h3 = sm + kTrH3, *z = sm + kTrZ, *dot = sm + kTrO;
+  float *fb = (float *)(sm + kTrF), *opart = fb + kTrFo;
+  uint64_t *mbar = (uint64_t *)(sm + kTrBar), *mbar2 = mbar + 1;
+  uint32_t *tslot = (uint32_t *)(mbar + 2);
+  const int tid = threadIdx.x, r = tid & 127, cq = tid >> 7, c0 = 32 * cq;
+  const bool issuer = tid == 0;
   tc_load_weights(wb, params, w1, w2, w3, fb);
-  for (int u = r; u < 2 * H + 3 * H + 2; u += blockDim.x) adW4[u] = 0.f;  // adW4 and adb are adjacent
-  if (r == 0) { tc::mbar_init(mbar); *flag = 0; }
-  if (r < 32) tc::tmem_alloc<512>(tslot);
+  const bf16 one = __float2bfloat16_rn(1.f);
+  for (int u = tid; u < 2 * TM; u += kTrT) {  // the columns past the activations: a one, zeros
+    unsigned char *t = u < TM ? h1 : h2;
+    *(uint4 *)(t + tc::core_off(u % TM, H, HX)) = make_uint4(pack2(one, __float2bfloat16_rn(0.f)), 0u, 0u, 0u);
+    *(uint4 *)(t + tc::core_off(u % TM, H + 8, HX)) = make_uint4(0u, 0u, 0u, 0u);
+  }
+  if (tid < TM) {
+    *(uint4 *)(x + tc::core_off(tid, 24, FPAD)) = make_uint4(pack2(__float2bfloat16_rn(0.f), one), 0u, 0u, 0u);
+    *(uint4 *)(dot + tc::core_off(tid, 0, 16)) = make_uint4(0u, 0u, 0u, 0u);
+    *(uint4 *)(dot + tc::core_off(tid, 8, 16)) = make_uint4(0u, 0u, 0u, 0u);
+  }
+  if (issuer) { tc::mbar_init(mbar); tc::mbar_init(mbar2); }
+  if (tid < 32) tc::tmem_alloc<512>(tslot);
   tc_sync();
-  // TMEM columns: [0, 128) the layer accumulator, [128, 256) dW3, [256, 384) dW2, [384, 416) dW1
-  const uint32_t tacc = *tslot, tdw3 = tacc + 128, tdw2 = tacc + 256, tdw1 = tacc + 384;
-  const uint32_t lanes = (uint32_t)(r & ~31) << 16;
+  const uint32_t tacc = *tslot, lanes = (uint32_t)(r & ~31) << 16;
   const uint32_t sw1 = tc::smem_u32(w1), sw2 = tc::smem_u32(w2), sw3 = tc::smem_u32(w3), sx = tc::smem_u32(x);
-  const uint32_t sh1 = tc::smem_u32(h1), sh2 = tc::smem_u32(h2), sz = tc::smem_u32(z);
-  const uint32_t kRowStep = 2 * (H / 8) * 128;     // two 8-row core groups of a [128][128] tile
-  const uint32_t kRowStepX = 2 * (FPAD / 8) * 128;  // of a [128][32] tile
+  const uint32_t sh1 = tc::smem_u32(h1), sh2 = tc::smem_u32(h2), sh3 = tc::smem_u32(h3), sz = tc::smem_u32(z),
+                 sdo = tc::smem_u32(dot);
+  // bytes of two 8-row core groups (a K step of 16 along the rows) by width
+  constexpr uint32_t kStepH = 2 * (H / 8) * 128, kStepHX = 2 * (HX / 8) * 128, kStepX = 2 * (FPAD / 8) * 128,
+                     kStepO = 2 * 2 * 128;
   const float scale = 2.f / (float)rows;
-  float lsum = 0.f;
-  uint32_t phase = 0;
+  float lsum = 0.f, sg0 = 0.f, sg1 = 0.f;
+  uint32_t phase = 0, phase2 = 0;
   bool ok = true, first = true;
   const int64_t tiles = (rows + TM - 1) / TM;
-  for (int64_t tl = blockIdx.x; tl < tiles && ok; tl += gridDim.x) {
-    const int64_t gr = tl * TM + r;
-    float *ft = (fwd_trace && gr < rows) ? fwd_trace + gr * 3 * H : nullptr;
-    float *bt = (bwd_trace && gr < rows) ? bwd_trace + gr * 4 * H : nullptr;
-    // ---- forward
-    tc_load_row(feat, gr, rows, r, x);
-    tc_sync();
-    if (r == 0) tc_gemm(tacc, sx, false, FPAD, kColStep, sw1, false, FPAD, kColStep, H, FPAD, false);
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
-    float o0 = 0.f, o1 = 0.f;
-    tc_hidden_epilogue(tacc, fb, h1, ft, nullptr, o0, o1);
-    tc_sync();
-    if (r == 0) tc_gemm(tacc, sh1, false, H, kColStep, sw2, false, H, kColStep, H, H, false);
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
-    tc_hidden_epilogue(tacc, fb + H, h2, ft ? ft + H : nullptr, nullptr, o0, o1);
-    tc_sync();
-    if (r == 0) tc_gemm(tacc, sh2, false, H, kColStep, sw3, false, H, kColStep, H, H, false);
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
-    tc_hidden_epilogue(tacc, fb + 2 * H, h3, ft ? ft + 2 * H : nullptr, fb + 3 * H, o0, o1);
-    // ---- output layer: dO of this row, rounded to bf16
-    float d0 = 0.f, d1 = 0.f;
-    if (gr < rows) {
-      d0 = (o0 + fb[5 * H]) - target[gr * 2];
-      d1 = (o1 + fb[5 * H + 1]) - target[gr * 2 + 1];
+  float v25[kTrLoads];
+  auto load_tile = [&](int64_t t) {  // 128 rows of F floats, coalesced (zero past rows)
+    const int64_t n = min((int64_t)TM, rows - t * TM) * F;
+#pragma unroll
+    for (int u = 0; u < kTrLoads; ++u) {
+      const int e = tid + kTrT * u;
+      v25[u] = e < n ? __ldg(feat + t * TM * F + e) : 0.f;
     }
-    lsum += d0 * d0 + d1 * d1;
-    const float g0 = __bfloat162float(__float2bfloat16_rn(d0 * scale));
-    const float g1 = __bfloat162float(__float2bfloat16_rn(d1 * scale));
-    dO[2 * r] = g0;
-    dO[2 * r + 1] = g1;
-    if (bt) {
-      bt[3 * H] = g0;
-      bt[3 * H + 1] = g1;
-      bt[3 * H + 2] = o0 + fb[5 * H];
-      bt[3 * H + 3] = o1 + fb[5 * H + 1];
+  };
+  int64_t tl = blockIdx.x;
+  if (tl < tiles) load_tile(tl);
+  for (; tl < tiles; tl += gridDim.x) {
+    const int64_t gr = tl * TM + r;
+    const bool live = gr < rows;
+    float *ft = (fwd_trace && live) ? fwd_trace + gr * 3 * H + c0 : nullptr;
+    float *bt = (bwd_trace && live) ? bwd_trace + gr * 4 * H + c0 : nullptr;
+    // ---- forward
+#pragma unroll
+    for (int u = 0; u < kTrLoads; ++u) {
+      const int e = tid + kTrT * u;
+      if (e < TM * F) *(bf16 *)(x + tc::core_off(e / F, e % F, FPAD)) = __float2bfloat16_rn(v25[u]);
+    }
+    const float2 tg = live ? make_float2(__ldg(target + 2 * gr), __ldg(target + 2 * gr + 1)) : make_float2(0.f, 0.f);
+    if (!(ok = tc_sync(ok))) break;
+    if (issuer) { tc_gemm(tacc, sx, false, FPAD, kColStep, sw1, false, FPAD, kColStep, H, FPAD, false); tc::commit(mbar); }
+    ok = ok && tc_wait(mbar, phase);
+    uint32_t w[16], mask[3];
+    auto positive = [&]() {  // bit j: column c0 + j of the rounded activation is positive
+      uint32_t m = 0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        m |= ((w[j] & 0x7fffu) ? 1u << (2 * j) : 0u) | ((w[j] & 0x7fff0000u) ? 2u << (2 * j) : 0u);
+      return m;
+    };
+    tc_hidden32(tacc + lanes + c0, fb + c0, w);
+    tc_store32(h1, r, c0, HX, w);
+    if (ft) trace32(ft, w);
+    mask[0] = positive();
+    if (!(ok = tc_sync(ok))) break;
+    if (issuer) { tc_gemm(tacc, sh1, false, HX, kColStep, sw2, false, H, kColStep, H, H, false); tc::commit(mbar); }
+    ok = ok && tc_wait(mbar, phase);
+    tc_hidden32(tacc + lanes + c0, fb + H + c0, w);
+    tc_store32(h2, r, c0, HX, w);
+    if (ft) trace32(ft + H, w);
+    mask[1] = positive();
+    if (!(ok = tc_sync(ok))) break;
+    if (issuer) { tc_gemm(tacc, sh2, false, HX, kColStep, sw3, false, H, kColStep, H, H, false); tc::commit(mbar); }
+    ok = ok && tc_wait(mbar, phase);
+    tc_hidden32(tacc + lanes + c0, fb + 2 * H + c0, w);
+    tc_store32(h3, r, c0, H, w);
+    if (ft) trace32(ft + 2 * H, w);
+    mask[2] = positive();
+    {
+      float p0 = 0.f, p1 = 0.f;
+      tc_out32(w, fb + 3 * H + 2 * c0, p0, p1);
+      *(float2 *)(opart + 2 * (cq * TM + r)) = make_float2(p0, p1);
+    }
+    __syncthreads();
+    // ---- output layer: dO of this row, rounded to bf16 (the same in the row's four threads)
+    float o0 = fb[5 * H], o1 = fb[5 * H + 1];
+    {
+      const float2 a = *(float2 *)(opart + 2 * r), b = *(float2 *)(opart + 2 * (TM + r)),
+                   c = *(float2 *)(opart + 2 * (2 * TM + r)), d = *(float2 *)(opart + 2 * (3 * TM + r));
+      o0 += (a.x + b.x) + (c.x + d.x);
+      o1 += (a.y + b.y) + (c.y + d.y);
+    }
+    const float d0 = live ? o0 - tg.x : 0.f, d1 = live ? o1 - tg.y : 0.f;
+    const uint32_t gw = pack2f(d0 * scale, d1 * scale);
+    const float g0 = lo2f(gw), g1 = hi2f(gw);
+    if (cq == 0) {
+      lsum += d0 * d0 + d1 * d1;
+      sg0 += g0;
+      sg1 += g1;
+      *(uint32_t *)(dot + tc::core_off(r, 0, 16)) = gw;
+      if (bt) {
+        bt[3 * H] = g0;
+        bt[3 * H + 1] = g1;
+        bt[3 * H + 2] = o0;
+        bt[3 * H + 3] = o1;
+      }
     }
     // dZ3 of this row from dO and W4, masked by H3
-    for (int c0 = 0; c0 < H; c0 += 32) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const float4 a = *(const float4 *)(fb + 3 * H + 2 * (c0 + 2 * j));
+      const float za = (mask[2] >> (2 * j)) & 1u ? fmaf(g1, a.y, g0 * a.x) : 0.f;
+      const float zb = (mask[2] >> (2 * j)) & 2u ? fmaf(g1, a.w, g0 * a.z) : 0.f;
+      w[j] = pack2f(za, zb);
+    }
+    tc_store32(z, r, c0, H, w);
+    if (bt) trace32(bt, w);
+    if (!(ok = tc_sync(ok))) break;
+    if (issuer) {
+      tc_gemm(tacc, sz, false, H, kColStep, sw3, true, H, kStepH, H, H, false);
+      tc_gemm(tacc + kTcW4, sh3, true, H, kStepH, sdo, true, 16, kStepO, 16, TM, !first);
+      tc::commit(mbar);
+      tc_gemm(tacc + kTcW3, sz, true, H, kStepH, sh2, true, HX, kStepHX, HX, TM, !first);
+      tc::commit(mbar2);
+    }
+    ok = ok && tc_wait(mbar, phase);
+    // dZ = dH o [layer > 0], 32 columns of this row
+    auto back = [&](uint32_t m, unsigned char *t, float *tr) {
       float v[32];
+      tc::ld32(tacc + lanes + c0, v);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const int c = c0 + j;
-        const float dz = fmaf(g1, fb[4 * H + c], g0 * fb[3 * H + c]);
-        v[j] = tc_get(h3, r, c, H) > 0.f ? __bfloat162float(__float2bfloat16_rn(dz)) : 0.f;
-      }
-      tc_store32(z, r, c0, v);
-      if (bt)
-#pragma unroll
-        for (int j = 0; j < 32; ++j) bt[c0 + j] = v[j];
+      for (int j = 0; j < 16; ++j)
+        w[j] = pack2f((m >> (2 * j)) & 1u ? v[2 * j] : 0.f, (m >> (2 * j)) & 2u ? v[2 * j + 1] : 0.f);
+      tc_store32(t, r, c0, H, w);
+      if (tr) trace32(tr, w);
+    };
+    back(mask[1], h3, bt ? bt + H : nullptr);  // dZ2 to H3's room: dW4 is done with it
+    if (!(ok = tc_sync(ok))) break;
+    if (issuer) {
+      tc_gemm(tacc, sh3, false, H, kColStep, sw2, true, H, kStepH, H, H, false);
+      tc::commit(mbar);
     }
-    tc_sync();
-    // dW3 += dZ3' H2 and dH2 = dZ3 W3 on the tensor cores; meanwhile dW4, db4 and db3 on the CUDA cores
-    if (r == 0) {
-      tc_gemm(tdw3, sz, true, H, kRowStep, sh2, true, H, kRowStep, H, TM, !first);
-      tc_gemm(tacc, sz, false, H, kColStep, sw3, true, H, kRowStep, H, H, false);
+    ok = ok && tc_wait(mbar2, phase2);  // dW3 is done with dZ3's room
+    if (issuer) {
+      tc_gemm(tacc + kTcW2, sh3, true, H, kStepH, sh1, true, HX, kStepHX, HX, TM, !first);
+      tc::commit(mbar2);
     }
-    {
-      float s0 = 0.f, s1 = 0.f, sb3 = 0.f;
-      for (int q = 0; q < TM; ++q) {
-        const float hq = tc_get(h3, q, r, H);
-        s0 = fmaf(dO[2 * q], hq, s0);
-        s1 = fmaf(dO[2 * q + 1], hq, s1);
-        sb3 += tc_get(z, q, r, H);
-      }
-      adW4[r] += s0;
-      adW4[H + r] += s1;
-      adb[2 * H + r] += sb3;
-      if (r < 2) {
-        float sb4 = 0.f;
-        for (int q = 0; q < TM; ++q) sb4 += dO[2 * q + r];
-        adb[3 * H + r] += sb4;
-      }
+    if (tl + gridDim.x < tiles) load_tile(tl + gridDim.x);
+    ok = ok && tc_wait(mbar, phase);
+    back(mask[0], z, bt ? bt + 2 * H : nullptr);
+    if (!(ok = tc_sync(ok))) break;
+    if (issuer) {
+      tc_gemm(tacc + kTcW1, sz, true, H, kStepH, sx, true, FPAD, kStepX, FPAD, TM, !first);
+      tc::commit(mbar);
     }
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
-    // dZ2 = dH2 o [H2 > 0]
-    for (int c0 = 0; c0 < H; c0 += 32) {
-      float v[32];
-      tc::ld32(tacc + lanes + (uint32_t)c0, v);
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        v[j] = tc_get(h2, r, c0 + j, H) > 0.f ? __bfloat162float(__float2bfloat16_rn(v[j])) : 0.f;
-      tc_store32(z, r, c0, v);
-      if (bt)
-#pragma unroll
-        for (int j = 0; j < 32; ++j) bt[H + c0 + j] = v[j];
-    }
-    tc_sync();
-    if (r == 0) {
-      tc_gemm(tdw2, sz, true, H, kRowStep, sh1, true, H, kRowStep, H, TM, !first);
-      tc_gemm(tacc, sz, false, H, kColStep, sw2, true, H, kRowStep, H, H, false);
-    }
-    {
-      float sb2 = 0.f;
-      for (int q = 0; q < TM; ++q) sb2 += tc_get(z, q, r, H);
-      adb[H + r] += sb2;
-    }
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
-    // dZ1 = dH1 o [H1 > 0]
-    for (int c0 = 0; c0 < H; c0 += 32) {
-      float v[32];
-      tc::ld32(tacc + lanes + (uint32_t)c0, v);
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        v[j] = tc_get(h1, r, c0 + j, H) > 0.f ? __bfloat162float(__float2bfloat16_rn(v[j])) : 0.f;
-      tc_store32(z, r, c0, v);
-      if (bt)
-#pragma unroll
-        for (int j = 0; j < 32; ++j) bt[2 * H + c0 + j] = v[j];
-    }
-    tc_sync();
-    if (r == 0) tc_gemm(tdw1, sz, true, H, kRowStep, sx, true, FPAD, kRowStepX, FPAD, TM, !first);
-    {
-      float sb1 = 0.f;
-      for (int q = 0; q < TM; ++q) sb1 += tc_get(z, q, r, H);
-      adb[r] += sb1;
-    }
-    if (!(ok = tc_commit_wait(mbar, phase, flag))) break;
     first = false;
+    ok = ok && tc_wait(mbar2, phase2) && tc_wait(mbar, phase);
   }
-  // ---- the block's partial gradient
+  ok = !group_any(!ok, -1);  // the last tile's waits
+  // ---- the block's partial gradient: row r of each, a quarter of the columns
   float *gp = part + (size_t)blockIdx.x * NPAR;
   const float nanv = __int_as_float(0x7fc00000);
   if (ok && !first) {
-    for (int c0 = 0; c0 < H; c0 += 32) {
-      float v[32];
-      tc::ld32(tdw3 + lanes + (uint32_t)c0, v);
-      for (int j = 0; j < 32; ++j) gp[OW3 + r * H + c0 + j] = v[j];
-      tc::ld32(tdw2 + lanes + (uint32_t)c0, v);
-      for (int j = 0; j < 32; ++j) gp[OW2 + r * H + c0 + j] = v[j];
-    }
     float v[32];
-    tc::ld32(tdw1 + lanes, v);
-    for (int j = 0; j < F; ++j) gp[OW1 + r * F + j] = v[j];
+    tc::ld32(tacc + kTcW3 + lanes + c0, v);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) gp[OW3 + r * H + c0 + j] = v[j];
+    tc::ld32(tacc + kTcW2 + lanes + c0, v);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) gp[OW2 + r * H + c0 + j] = v[j];
+    if (cq == 0) {
+      tc::ld32(tacc + kTcW1 + lanes, v);
+#pragma unroll
+      for (int j = 0; j < F; ++j) gp[OW1 + r * F + j] = v[j];
+      gp[OB1 + r] = v[F];
+    } else if (cq == 1) {
+      tc::ld32(tacc + kTcW3 + H + lanes, v);  // the ones column (the columns past 144 are not read further)
+      gp[OB3 + r] = v[0];
+    } else if (cq == 2) {
+      tc::ld32(tacc + kTcW2 + H + lanes, v);
+      gp[OB2 + r] = v[0];
+    } else {
+      tc::ld32(tacc + kTcW4 + lanes, v);
+      gp[OW4 + r] = v[0];
+      gp[OW4 + H + r] = v[1];
+    }
   } else {
     const float fill = ok ? 0.f : nanv;  // a block without tiles adds nothing
-    for (int u = r; u < H * H; u += blockDim.x) { gp[OW3 + u] = fill; gp[OW2 + u] = fill; }
-    for (int u = r; u < H * F; u += blockDim.x) gp[OW1 + u] = fill;
+    for (int u = tid; u < OB4; u += kTrT) gp[u] = fill;
   }
+  // loss and output bias: the sums of the first 128 threads' rows
   __syncthreads();
-  for (int u = r; u < H; u += blockDim.x) {
-    gp[OB1 + u] = ok ? adb[u] : nanv;
-    gp[OB2 + u] = ok ? adb[H + u] : nanv;
-    gp[OB3 + u] = ok ? adb[2 * H + u] : nanv;
-    gp[OW4 + u] = ok ? adW4[u] : nanv;
-    gp[OW4 + H + u] = ok ? adW4[H + u] : nanv;
+  if (tid < TM) {
+    lsum = warp_sum(lsum);
+    sg0 = warp_sum(sg0);
+    sg1 = warp_sum(sg1);
+    if ((tid & 31) == 0) {
+      opart[tid >> 5] = lsum;
+      opart[4 + (tid >> 5)] = sg0;
+      opart[8 + (tid >> 5)] = sg1;
+    }
   }
-  if (r < 2) gp[OB4 + r] = ok ? adb[3 * H + r] : nanv;
-  lsum = warp_sum(lsum);
-  if (lane == 0) lsw[w] = lsum;
   tc::fence_before();
   __syncthreads();
-  if (r == 0) loss_part[blockIdx.x] = ok ? lsw[0] + lsw[1] + lsw[2] + lsw[3] : nanv;
-  if (r < 32) {
+  if (tid < 3) {
+    const float t = (opart[4 * tid] + opart[4 * tid + 1]) + (opart[4 * tid + 2] + opart[4 * tid + 3]);
+    if (tid == 0) loss_part[blockIdx.x] = ok ? t : nanv;
+    else gp[OB4 + tid - 1] = ok ? t : nanv;
+  }
+  if (tid < 32) {
     tc::fence_after();
     tc::tmem_free<512>(tacc);
   }
@@ -732,7 +833,7 @@ cudaError_t mlp_forward(const bf16 *wb, const float *params, const float *feat, 
   if (rows <= 0) return cudaSuccess;
   const int64_t tiles = (rows + TM - 1) / TM;
   const int grid = (int)std::min<int64_t>(tiles, (int64_t)sms);
-  forward_tc_kernel<<<grid, TM, kFwdSmem, s>>>(wb, params, feat, rows, out, trace);
+  forward_tc_kernel<<<grid, TM * kFwdGroups, kFwdSmem, s>>>(wb, params, feat, rows, out, trace);
   return cudaGetLastError();
 }
 
@@ -747,8 +848,8 @@ cudaError_t mlp_grad(const bf16 *wb, const float *params, const float *feat, con
     if (e) return e;
     attr = true;
   }
-  const int nb = mlp_train_blocks(sms);
-  train_tc_kernel<<<nb, TM, kTrainSmem, s>>>(wb, params, feat, target, rows, part, lpart, fwd_trace, bwd_trace);
+  const int nb = (int)std::min<int64_t>((rows + TM - 1) / TM, (int64_t)mlp_train_blocks(sms));
+  train_tc_kernel<<<nb, kTrT, kTrainSmem, s>>>(wb, params, feat, target, rows, part, lpart, fwd_trace, bwd_trace);
   grad_reduce_kernel<<<nblk(NPAR, 256), 256, 0, s>>>(part, nb, grad, lpart, rows, loss);
   return cudaGetLastError();
 }
