@@ -43,8 +43,9 @@ template <> struct Coords<double> {
 // operations, each relative 2^-24 of at most 2 R, and R inv <= nc / 2 up to a rounding), a quarter of
 // the slack; a value further than the slack from an integer lies in the same cell.
 template <typename V>
-__device__ __forceinline__ int cell_coord_fast(V v, double R, double inv, int nc, float Rf, float invf, float slack) {
-  const float f = ((float)v + Rf) * invf;
+__device__ __forceinline__ int cell_coord_fast(V v, float vf, double R, double inv, int nc, float Rf, float invf,
+                                               float slack) {
+  const float f = (vf + Rf) * invf;
   const float fl = floorf(f), fr = f - fl;
   if (f < -slack) return 0;
   if (f > (float)nc + slack) return nc - 1;
@@ -52,65 +53,74 @@ __device__ __forceinline__ int cell_coord_fast(V v, double R, double inv, int nc
   return cell_coord((double)v, R, inv, nc);
 }
 template <typename P>
-__device__ __forceinline__ int cell_key_fast(P p, double R, double inv, int nc) {
+__device__ __forceinline__ int cell_key_fast(P p, float2 f, double R, double inv, int nc) {
   const float Rf = (float)R, invf = (float)inv, slack = (float)nc * (1.f / 1048576.f);
-  const int cx = cell_coord_fast(p.x, R, inv, nc, Rf, invf, slack);
-  return cell_coord_fast(p.y, R, inv, nc, Rf, invf, slack) * nc + cx;
+  const int cx = cell_coord_fast(p.x, f.x, R, inv, nc, Rf, invf, slack);
+  return cell_coord_fast(p.y, f.y, R, inv, nc, Rf, invf, slack) * nc + cx;
 }
 
 // Distance slack around a circle whose coordinates are at most M in absolute value, for pairs near a
 // distance l: the binary32 distance of the rounded coordinates is off by less than 2^-22 (M + l).
 __device__ __forceinline__ float dist_slack(float M, float l) { return (M + l + 8.f) * (1.f / 1048576.f); }
 
-// The neighbor predicate of Sec. 4.3 for circle i against the circle at sorted position q.
+// The neighbor predicate of Sec. 4.3 for circle i (binary32 coordinates xf, given to set()) against the
+// circle at sorted position q.
 template <typename T> struct Near;
 template <> struct Near<float> {
   float lc2;
-  __device__ __forceinline__ void init(float2, double l_cut) { lc2 = (float)(l_cut * l_cut); }
+  float2 xf;
+  __device__ __forceinline__ explicit Near(double l_cut) : lc2((float)(l_cut * l_cut)) {}
+  __device__ __forceinline__ void set(float2 x) { xf = x; }
   template <typename I>
-  __device__ __forceinline__ bool operator()(float2 xi, float2 xq, const Coords<float> &, const I *, int) const {
-    return nbr_pred(xi, xq, lc2);
+  __device__ __forceinline__ bool operator()(int, float2 xq, const Coords<float> &, const I *, int) const {
+    return nbr_pred(xf, xq, lc2);
   }
 };
 template <> struct Near<double> {
   double lc2;
+  float lc;
   float2 xf;
   float lo, hi;  // binary32 squared distances below lo are inside, above hi outside
-  __device__ __forceinline__ void init(double2 xi, double l_cut) {
-    lc2 = l_cut * l_cut;
-    xf = make_float2((float)xi.x, (float)xi.y);
-    const float lc = (float)l_cut, m = dist_slack(fabsf(xf.x) + fabsf(xf.y), lc);
+  __device__ __forceinline__ explicit Near(double l_cut) : lc2(l_cut * l_cut), lc((float)l_cut) {}
+  __device__ __forceinline__ void set(float2 x) {
+    xf = x;
+    const float m = dist_slack(fabsf(x.x) + fabsf(x.y), lc);
     const bool ok = m <= 0.25f;  // else (far out, not finite): every distance in binary64
     lo = ok ? (lc - m) * (lc - m) : -1.f;
     hi = ok ? (lc + m) * (lc + m) : __int_as_float(0x7f800000);
   }
   template <typename I>
-  __device__ __forceinline__ bool operator()(double2 xi, float2 xq, const Coords<double> &X, const I *ord, int q) const {
+  __device__ __forceinline__ bool operator()(int i, float2 xq, const Coords<double> &X, const I *ord, int q) const {
     const float dx = xf.x - xq.x, dy = xf.y - xq.y, s = dx * dx + dy * dy;
     if (s > hi) return false;
     if (s < lo) return true;
-    return nbr_pred(xi, X.at(ord[q]), lc2);
+    return nbr_pred(X.at(i), X.at(ord[q]), lc2);
   }
 };
 
+// A coordinate that is not finite, without a binary64 operation.
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+__device__ __forceinline__ bool not_finite(float v) { return (__float_as_uint(v) & 0x7f800000u) == 0x7f800000u; }
+
 // ---- one block per instance ----
-// Shared-memory layout for an instance of n circles: coordinates in cell order, then three 16-bit
-// arrays, then `extra` bytes of the kernel's own, then the cell table when it fits its share (1.25 cells
+// Shared-memory layout for an instance of n circles: coordinates in cell order (binary64 searches: and
+// in index order, so that each is converted once), then three 16-bit arrays, then `extra` bytes of the kernel's own, then the cell table when it fits its share (1.25 cells
 // per circle: the layouts of this library have about 0.8), else the table in global memory.
 __host__ __device__ inline int cell_share(int n) { return n + n / 4 + 64 < 256 ? 256 : n + n / 4 + 64; }
 __host__ __device__ inline size_t cells_r16(size_t b) { return (b + 15) & ~size_t(15); }
-__host__ __device__ inline size_t cells_smem(int n, size_t extra) {
-  return cells_r16(8 * (size_t)n) + 3 * cells_r16(2 * (size_t)n) + extra + 4 * (size_t)(cell_share(n) + 1);
+__host__ __device__ inline size_t cells_smem(int n, size_t extra, bool wide) {
+  return (wide ? 2 : 1) * cells_r16(8 * (size_t)n) + 3 * cells_r16(2 * (size_t)n) + extra + 4 * (size_t)(cell_share(n) + 1);
 }
 struct BlockCells {
   float2 *xs;            // coordinates in cell order (rounded to binary32)
+  const float2 *xi;      // ... in index order (binary32 searches: the caller's)
   uint16_t *key, *ord;   // cell of circle i; circle at sorted position p
   int32_t *start;        // cell starts, ncell + 1
   unsigned char *extra;
 };
 
 // Sort the n circles by (cell, index).  ckey / corder (may be null): the cells and the order for export.
-// visit(i, point): called once per circle by its thread while its coordinates are at hand.
+// visit(point, binary32 point, i): called once per circle by its thread while its coordinates are at hand.
 template <typename T, typename Visit>
 __device__ __forceinline__ BlockCells block_cells(const Coords<T> &X, int n, double R, double inv, int nc,
                                                   unsigned char *sm, size_t extra, int32_t *cells_g, uint32_t *ckey,
@@ -119,7 +129,15 @@ __device__ __forceinline__ BlockCells block_cells(const Coords<T> &X, int n, dou
   BlockCells C;
   const size_t nb = cells_r16(2 * (size_t)n);
   C.xs = (float2 *)sm;
-  C.key = (uint16_t *)(sm + cells_r16(8 * (size_t)n));
+  sm += cells_r16(8 * (size_t)n);
+  float2 *xi = nullptr;
+  if constexpr (sizeof(T) == 8) {
+    C.xi = xi = (float2 *)sm;
+    sm += cells_r16(8 * (size_t)n);
+  } else {
+    C.xi = X.x;
+  }
+  C.key = (uint16_t *)sm;
   uint16_t *tmp = (uint16_t *)((unsigned char *)C.key + nb);
   C.ord = (uint16_t *)((unsigned char *)tmp + nb);  // until the last step: arrival rank within the cell
   C.extra = (unsigned char *)C.ord + nb;
@@ -129,11 +147,13 @@ __device__ __forceinline__ BlockCells block_cells(const Coords<T> &X, int n, dou
   __syncthreads();
   for (int i = tid; i < n; i += B) {
     const typename Coords<T>::point p = X.at(i);
-    const int key = cell_key_fast(p, R, inv, nc);
+    const float2 f = make_float2((float)p.x, (float)p.y);
+    if constexpr (sizeof(T) == 8) xi[i] = f;
+    const int key = cell_key_fast(p, f, R, inv, nc);
     C.key[i] = (uint16_t)key;
     if (ckey) ckey[i] = (uint32_t)key;
     C.ord[i] = (uint16_t)atomicAdd(&C.start[key + 1], 1);
-    visit(i, p);
+    visit(p, f, i);
   }
   __syncthreads();
   block_scan_inplace(C.start + 1, ncell, sh);
@@ -145,7 +165,7 @@ __device__ __forceinline__ BlockCells block_cells(const Coords<T> &X, int n, dou
     int r = C.start[c];
     for (int q = C.start[c], hi = C.start[c + 1]; q < hi; ++q) r += tmp[q] < i;
     C.ord[r] = (uint16_t)i;
-    C.xs[r] = X.low(i);
+    C.xs[r] = C.xi[i];
     if (corder) corder[r] = i;
   }
   __syncthreads();

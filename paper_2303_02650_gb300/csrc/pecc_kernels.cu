@@ -111,9 +111,9 @@ __global__ void set_radius_kernel(InstDesc *desc, const double *__restrict__ R, 
 // entries straight to global memory, insertion sort).
 constexpr int kRowHits = 16;
 
-// Hits of the circle at xi (index i, cell key) over the 3x3 cells, in scan order: f(q) for each.
+// Hits of circle i (cell key; near.set() done) over the 3x3 cells, in scan order: f(q) for each.
 template <typename T, typename I, typename F>
-__device__ __forceinline__ void for_neighbors(const Coords<T> &X, typename Coords<T>::point xi, int i, int key, int nc,
+__device__ __forceinline__ void for_neighbors(const Coords<T> &X, int i, int key, int nc,
                                               const int32_t *start, const float2 *xs, const I *ord,
                                               const Near<T> &near, F f) {
   const int cy = key / nc, cx = key - cy * nc;
@@ -121,7 +121,7 @@ __device__ __forceinline__ void for_neighbors(const Coords<T> &X, typename Coord
   for (int by = max(cy - 1, 0); by <= min(cy + 1, nc - 1); ++by) {
     const int lo = start[by * nc + bx0], hi = start[by * nc + bx1 + 1];
     for (int q = lo; q < hi; ++q)
-      if (near(xi, xs[q], X, ord, q) && (int)ord[q] != i) f(q);
+      if (near(i, xs[q], X, ord, q) && (int)ord[q] != i) f(q);
   }
 }
 
@@ -135,11 +135,10 @@ __device__ __forceinline__ void write_rows(const Coords<T> &X, bool act, int i, 
   const int lane = threadIdx.x & 31;
   if (__any_sync(0xffffffffu, cnt > kRowHits)) {
     if (act) {
-      const typename Coords<T>::point xi = X.at(i);
-      Near<T> near;
-      near.init(xi, X.l_cut);
+      Near<T> near(X.l_cut);
+      near.set(X.low(i));
       int w = row0;
-      for_neighbors<T, I>(X, xi, i, key, nc, start, xs, ord, near, [&](int q) {
+      for_neighbors<T, I>(X, i, key, nc, start, xs, ord, near, [&](int q) {
         const int v = (int)ord[q];
         if (w < cap) {  // insert in ascending order
           int t = w - 1;
@@ -253,22 +252,21 @@ __global__ void __launch_bounds__(512) build_block_kernel(StandaloneParams P, in
   const int nc = D.ncx, cap = D.cap;
   const size_t extra = (size_t)(blockDim.x >> 5) * kBuildWarpBytes;
   const BlockCells C = block_cells<T>(X, n, D.R, D.inv_cs, nc, sm, extra, P.cells + D.cell_off, P.ckey + off,
-                                      P.corder + off, sh, [&](int i, PP p) { xb[i] = p; });
+                                      P.corder + off, sh, [&](PP p, float2, int i) { xb[i] = p; });
   int32_t *rp = P.rp + off + q, *col = P.col + D.col_s_off;
   uint16_t *buf = (uint16_t *)(C.extra + (threadIdx.x >> 5) * kBuildWarpBytes);
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) rp[0] = 0;
   int run = 0;
+  Near<T> near(P.l_cut);
   for (int i0 = 0; i0 < n; i0 += blockDim.x) {
     const int i = i0 + threadIdx.x;
     const bool act = i < n;
     int cnt = 0, key = 0;
     if (act) {
-      const PP xi = X.at(i);
       key = C.key[i];
-      Near<T> near;
-      near.init(xi, P.l_cut);
-      for_neighbors<T, uint16_t>(X, xi, i, key, nc, C.start, C.xs, C.ord, near, [&](int qq) {
+      near.set(C.xi[i]);
+      for_neighbors<T, uint16_t>(X, i, key, nc, C.start, C.xs, C.ord, near, [&](int qq) {
         if (cnt < kRowHits) buf[32 * cnt + lane] = C.ord[qq];
         ++cnt;
       });
@@ -325,14 +323,14 @@ __global__ void __launch_bounds__(kTileRows) large_key_kernel(StandaloneParams P
   int bad = 0;
   if (i < D.n) {
     const typename Coords<T>::point p = coords_of<T>(P, D.off, from32).at(i);
-    const int key = cell_key_fast(p, D.R, D.inv_cs, D.ncx);
+    const float2 f = make_float2((float)p.x, (float)p.y);
+    const int key = cell_key_fast(p, f, D.R, D.inv_cs, D.ncx);
     O.ckey[D.off + i] = (uint32_t)key;
     L.rank[D.off + i] = atomicAdd(P.cells + D.cell_off + key + 1, 1);
     if (xbuild) xbuild[D.off + i] = p;
     if (CHECK) {
-      const float fx = (float)p.x, fy = (float)p.y;
-      r2 = fx * fx + fy * fy;
-      bad = !(isfinite(p.x) && isfinite(p.y));
+      r2 = f.x * f.x + f.y * f.y;
+      bad = not_finite(p.x) || not_finite(p.y);
     }
   }
   if (CHECK) {
@@ -430,11 +428,10 @@ __global__ void __launch_bounds__(kTileRows) large_rows_kernel(StandaloneParams 
   const bool act = i < n;
   int cnt = 0, key = 0;
   if (act) {
-    const typename Coords<T>::point xi = X.at(i);
     key = (int)O.ckey[D.off + i];
-    Near<T> near;
-    near.init(xi, P.l_cut);
-    for_neighbors<T, int32_t>(X, xi, i, key, nc, start, xs, ord, near, [&](int q) {
+    Near<T> near(P.l_cut);
+    near.set(X.low(i));
+    for_neighbors<T, int32_t>(X, i, key, nc, start, xs, ord, near, [&](int q) {
       if (FILL && cnt < kRowHits) buf[32 * cnt + lane] = ord[q];
       ++cnt;
     });
@@ -732,19 +729,17 @@ __global__ void __launch_bounds__(512) feasible_block_kernel(StandaloneParams P,
   int bad = 0;
   const BlockCells C =
       block_cells<double>(X, n, D.R, D.inv_cs, nc, sm, 0, P.cells + D.cell_off, nullptr, nullptr, sh,
-                          [&](int, double2 p) {
-                            const float fx = (float)p.x, fy = (float)p.y;
-                            rmax = fmaxf(rmax, fx * fx + fy * fy);
-                            bad |= !(isfinite(p.x) && isfinite(p.y));
+                          [&](double2 p, float2 f, int) {
+                            rmax = fmaxf(rmax, f.x * f.x + f.y * f.y);
+                            bad |= not_finite(p.x) || not_finite(p.y);
                           });
   const float inf = __int_as_float(0x7f800000);
   float smin = inf;
   int hits = 0;
+  Near<double> near(P.l_cut);
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
     const int i = C.ord[p];
-    Near<double> near;
-    const float2 a = C.xs[p];
-    near.init(make_double2((double)a.x, (double)a.y), P.l_cut);  // lo and hi allow for the rounding
+    near.set(C.xs[p]);
     for_candidates(p, (int)C.key[i], nc, C.start, C.xs, C.ord, [&](int qq, float s) {
       smin = fminf(smin, s);
       if (s > near.hi) return;
@@ -805,9 +800,8 @@ __global__ void __launch_bounds__(kTileRows) large_check_kernel(StandaloneParams
     int hits = 0;
     if (p < n) {
       const int i = ord[p];
-      Near<double> near;
-      const float2 a = xs[p];
-      near.init(make_double2((double)a.x, (double)a.y), P.l_cut);
+      Near<double> near(P.l_cut);
+      near.set(xs[p]);
       for_candidates(p, (int)O.ckey[D.off + i], nc, start, xs, ord, [&](int q, float s) {
         smin = fminf(smin, s);
         if (s > near.hi) return;
@@ -946,7 +940,7 @@ static cudaError_t build_t(const StandaloneParams &p, const LargeTiles &L, int n
                            int32_t *rebuilt, cudaStream_t s) {
   if (n_small >= 0) {
     const int block = cells_threads(n_small, p.num, sms);
-    const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kBuildWarpBytes);
+    const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kBuildWarpBytes, sizeof(T) == 8);
     cudaError_t e = cudaFuncSetAttribute(build_block_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     build_block_kernel<T><<<p.num, block, smem, s>>>(p, force, rebuilt);
@@ -1011,7 +1005,7 @@ cudaError_t launch_feasible(const StandaloneParams &p, const LargeTiles &L, int 
                             double tol, uint8_t *feasible, double *max_overlap, cudaStream_t s) {
   if (p.num <= 0) return cudaSuccess;
   if (n_small >= 0) {
-    const size_t smem = cells_smem(n_small, 0);
+    const size_t smem = cells_smem(n_small, 0, true);
     cudaError_t e = cudaFuncSetAttribute(feasible_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     feasible_block_kernel<<<p.num, cells_threads(n_small, p.num, sms), smem, s>>>(p, from32, tol, feasible, max_overlap);
