@@ -221,11 +221,11 @@ template <> __device__ __forceinline__ Coords<double> coords_of<double>(const St
 // Instances of at most kCellsBlockN circles, one block each, everything on chip: the coordinates come
 // in once, the rows, cells and order go out once.  What bounds it is the latency of the block's chain
 // (cell counts, two scans, candidate walks).  The 4096-instance batch's new positions, lists, energy and
-// gradient take 216 us with it, about 160 us of them here; 966 us with the kernel it replaced (lists
+// gradient take 215 us with it, about 158 us of them here; 966 us with the kernel it replaced (lists
 // built and sorted in global memory, 901 us).
 constexpr int kBuildWarpBytes = 32 * kRowHits * (int)sizeof(uint16_t);
 template <typename T>
-__global__ void __launch_bounds__(512) build_block_kernel(StandaloneParams P, int force, int32_t *rebuilt) {
+__global__ void __launch_bounds__(512, 3) build_block_kernel(StandaloneParams P, int force, int32_t *rebuilt) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int32_t sh[40];
   using PP = v2<T>;
@@ -660,8 +660,9 @@ __global__ void __launch_bounds__(1024) energy_reduce_kernel(StandaloneParams P,
 // search runs in binary32; the binary64 values are formed for the pairs and circles whose binary32 ones
 // lie within the slack of the extreme.  The entries a list with cutoff l_cut > 2 would hold (it holds
 // every overlapping pair) are counted: past twice the capacity the instance is not checkable.
-// The 4096-instance batch: 187 us, against 2212 us for a binary64 list build and a walk over it, which
-// the two binary64 lanes of an SM bound.
+// The 4096-instance batch: 150 us, against 2212 us for a binary64 list build and a walk over it, which
+// the two binary64 lanes of an SM bound.  40 registers let six 256-thread blocks share an SM (170 us with
+// 64 registers and four).
 __device__ __forceinline__ double dist2_exact(double2 a, double2 b) {
   const double dx = __dsub_rn(a.x, b.x), dy = __dsub_rn(a.y, b.y);
   return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
@@ -712,7 +713,7 @@ __device__ __forceinline__ void for_candidates(int p, int key, int nc, const int
   }
 }
 
-__global__ void __launch_bounds__(512) feasible_block_kernel(StandaloneParams P, int from32, double tol,
+__global__ void __launch_bounds__(512, 3) feasible_block_kernel(StandaloneParams P, int from32, double tol,
                                                              uint8_t *feasible, double *max_overlap) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int32_t sh[40];
