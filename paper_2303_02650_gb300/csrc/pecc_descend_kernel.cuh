@@ -39,25 +39,6 @@ namespace pecc {
 
 namespace {
 
-constexpr int KS = kMaxSlots;     // basis index of Y slot a is KS + a
-constexpr int GI = 2 * kMaxSlots; // basis index of g
-// The dots of the first reduction of a batch step come in chunks of 32 values, one chunk per six
-// physical slots a: in chunk a / 6, from 4 (a % 6): g's_a, g'y_a, y's_a, y'y_a, where (s, y) is the
-// pending pair; chunk 0 also carries g'g, s's, s'y and y'y at 24..27.  The two-loop on the Gram
-// matrix reads an s only against the y's of its own or a newer pair, and no s against another s, so
-// s's_a and s'y_a are not taken: four values per slot instead of six put the six slots of m = 5 in
-// one chunk (one pass over the slots and one reduce-scatter instead of two), the eleven of m = 10
-// in two instead of three.
-constexpr int kSlotsPerChunk = 6;
-constexpr int kChunks = (kMaxSlots + kSlotsPerChunk - 1) / kSlotsPerChunk;
-constexpr int kPA = 32 * kChunks;  // per-warp partial values of the first reduction
-constexpr int PA_GG = 24, PA_SS = 25, PA_SY = 26, PA_YY = 27;
-__device__ __forceinline__ int pa_idx(int a, int kind) {
-  return 32 * (a / kSlotsPerChunk) + 4 * (a % kSlotsPerChunk) + kind;
-}
-// Gram matrix of a batch: s_a'y_b at a KS + b (a not newer than b), then y_a'y_b at KS KS + a KS + b.
-constexpr int kGram = 2 * KS * KS;
-constexpr int kYY = KS * KS;
 constexpr int kRingInts = kMaxSlots + 3;  // count, stage, ring[kMaxSlots], pending
 
 __device__ __forceinline__ uint64_t sortable(double v) {
@@ -155,31 +136,6 @@ __host__ __device__ inline size_t batch_room(int n, int k, size_t vec, size_t po
   const size_t nbm = (size_t)(n + k - 1) / k;
   const size_t step = 3 * round16(nbm * vec) + nbm * pos, build = round16(8 * (size_t)n) + (size_t)n * pos;
   return step > build ? step : build;
-}
-
-// One secant pair of one circle: s and y side by side, one 16-byte access in binary32 (two in
-// binary64) where separate arrays took two.
-template <typename T> struct alignas(16) SecantPair { v2<T> s, y; };
-__device__ __forceinline__ SecantPair<float> ld_pair(const SecantPair<float> *p) {
-  const float4 v = *(const float4 *)p;
-  return SecantPair<float>{make_float2(v.x, v.y), make_float2(v.z, v.w)};
-}
-__device__ __forceinline__ SecantPair<double> ld_pair(const SecantPair<double> *p) { return *p; }
-__device__ __forceinline__ void st_pair(SecantPair<float> *p, float2 s, float2 y) {
-  *(float4 *)p = make_float4(s.x, s.y, y.x, y.y);
-}
-__device__ __forceinline__ void st_pair(SecantPair<double> *p, double2 s, double2 y) { p->s = s; p->y = y; }
-
-// The pairs of circle pos in the physical slots [A0, A0 + N), of mm in all.  Every load is issued
-// whether its slot is in use or not (its value is then ignored; a slot past the last is read as slot
-// 0), so that all of them are in flight together: behind a test of its own each slot waited for its
-// own L2 round trip (the 4096-instance batch at m = 5: 210.5 ms, with the groups 191.2).  Six slots
-// per group, those of m = 5, and one circle per thread at a time: seven slots, or two circles, take
-// registers the kernel does not have (196.0 and 192.6 ms, and a single instance gets slower).
-template <int A0, int N, typename T>
-__device__ __forceinline__ void load_slots(const SecantPair<T> *SY, int mm, int n, int pos, SecantPair<T> *pr) {
-#pragma unroll
-  for (int j = 0; j < N; ++j) pr[j] = ld_pair(SY + (A0 + j < mm ? A0 + j : 0) * n + pos);
 }
 
 // Bump allocator over dynamic shared memory; returns the fallback when the request does not fit.

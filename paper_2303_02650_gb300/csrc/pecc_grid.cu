@@ -2,9 +2,9 @@
 // ANM (Sec. 4.3), the steps of descend_kernel with every block-wide step made grid-wide.
 //
 // One cooperative launch (every block resident) runs the whole descent.  Blocks meet at a grid
-// barrier built here (an arrival counter and a generation word in global memory); every wait is
-// bounded by %globaltimer and raises an error flag instead of spinning on.  Reductions: each block
-// reduces its part, block 0 adds the parts, every block reads the totals.  All control decisions,
+// barrier built here (an arrival counter in global memory that only grows); every wait is bounded by
+// %globaltimer and raises an error flag instead of spinning on.  Reductions: each block reduces its
+// part and, after one barrier, every block combines all parts itself in the same order.  All control decisions,
 // the secant-pair ring, the Gram matrices and the two-loop recursion are computed redundantly and
 // identically by every block from those totals, so they need no further synchronisation.
 //   partition   pseudo-angle (annulus: radius, fence: x) keys; buckets by key value (monotone),
@@ -18,62 +18,67 @@
 namespace pecc {
 namespace {
 
-constexpr int KS = kMaxSlots;
-constexpr int GI = 2 * kMaxSlots;
-constexpr int OP = 1 + 2 * kMaxSlots;
-constexpr int NV1 = OP + 4 * kMaxSlots + 3;  // values of the first reduction of a batch step
-constexpr int kPart = 72;                    // stride of a block's partials (>= NV1 + 2)
-constexpr int kRing = kMaxSlots + 4;         // count, stage, ring[kMaxSlots], pending, used
+constexpr int PA_E = 28;                  // first reduction of a batch step: the batch energy (chunk 0)
+constexpr int kPart = 72;                 // stride of a block's partials (>= 32 kChunks)
+constexpr int kRing = kMaxSlots + 4;      // count, stage, ring[kMaxSlots], pending, used
+constexpr int kGramOnChip = 8;            // batches whose Gram matrices a block keeps in shared memory
 constexpr long long kBarrierTimeoutNs = 2000000000ll;
 
-__device__ __forceinline__ unsigned ldv(const unsigned *p) { return *(volatile const unsigned *)p; }
-__device__ __forceinline__ int ldv(const int *p) { return *(volatile const int *)p; }
-
-// Grid barrier for `expected` arriving blocks; false (for the whole block) once any block's wait
-// has run past timeout_ns (measured on %globaltimer) and raised the shared error flag.
-__device__ bool grid_sync_n(GridCtl *c, unsigned expected, long long timeout_ns) {
+// Grid barrier for `expected` arriving blocks: the arrival counter only grows, *done is the number of
+// barriers this block has passed (in its shared memory), so a barrier is one reduction and one polled
+// word (a separate generation word, read before every arrival and written after the last one, took two
+// more round trips to L2; polling with a sleep and the clock in the loop, another).  False (for the
+// whole block) once any block's wait has run past timeout_ns (measured on %globaltimer) and raised the
+// shared error flag.
+__device__ bool grid_sync_n(GridCtl *c, unsigned expected, unsigned *done, long long timeout_ns) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned g = ldv(&c->gen);
-    __threadfence();
-    const unsigned arrived = atomicAdd(&c->count, 1u) + 1u;
+    const unsigned target = (*done + 1u) * expected;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&c->count) : "memory");
+    auto arrived = [&]() {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&c->count) : "memory");
+      return (int)(v - target) >= 0;
+    };
+    auto failed = [&]() { return *(volatile const int *)&c->err != 0; };
     int good = 1;
-    if (arrived == expected) {
-      atomicExch(&c->count, 0u);
-      __threadfence();
-      atomicAdd(&c->gen, 1u);
-    } else {
+    bool there = arrived();
+    for (int it = 0; it < 4096 && !there; ++it) there = arrived();
+    if (!there) {
       const long long t0 = globaltimer_ns();
-      while (ldv(&c->gen) == g) {
-        if (ldv(&c->err)) { good = 0; break; }
+      while (!arrived()) {
+        if (failed()) { good = 0; break; }
         if (globaltimer_ns() - t0 > timeout_ns) { atomicExch(&c->err, 1); good = 0; break; }
         __nanosleep(64);
       }
     }
-    __threadfence();
-    ok = good && !ldv(&c->err);
+    ++*done;
+    ok = good && !failed();
   }
   __syncthreads();
   return ok;
 }
 
-__device__ __forceinline__ bool grid_sync(GridCtl *c) { return grid_sync_n(c, gridDim.x, kBarrierTimeoutNs); }
-
 template <class A> struct GSmem {
   using vec_t = typename A::vec_t;
   double wb[16 * kPart];       // per-warp partials
   double tot[kPart];           // reduction totals
-  vec_t gram[kBasis * kBasis]; // Gram matrix of the current batch (identical in every block)
+  vec_t gram[kGramOnChip * kGram];  // Gram matrices of the first batches (identical in every block)
   vec_t coef[kBasis];
   int ring[kMaxK][kRing];
   int32_t sh[40];
   long long iv[2];
   int flag;
   int rbuf;  // partial buffer of the next grid_reduce (same in every block)
+  unsigned barriers;  // grid barriers passed
 };
 
-// Grid-wide reduction of NV values (kind 0: sum, 1: max) with one grid barrier: every block writes
+template <class A> __device__ __forceinline__ bool grid_sync(GSmem<A> &S, GridCtl *c) {
+  return grid_sync_n(c, gridDim.x, &S.barriers, kBarrierTimeoutNs);
+}
+
+// Grid-wide reduction of NV <= 8 values (kind 0: sum, 1: max) with one grid barrier: every block writes
 // its partials to buffer S.rbuf of G.part, and after the barrier every block combines all blocks'
 // partials itself (warp q takes value q, its lanes stride over the blocks, then a fixed butterfly),
 // so every block holds bit-identical totals in S.tot[].  Consecutive reductions alternate the two
@@ -81,6 +86,7 @@ template <class A> struct GSmem {
 // block passes after its reads of this one.
 template <class A, int NV, typename T>
 __device__ bool grid_reduce(GSmem<A> &S, const GridBufs &G, GridCtl *c, T (&v)[NV], const int (&kind)[NV]) {
+  static_assert(NV <= 8, "one warp per value");
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int buf = S.rbuf;
   double *part = G.part + (size_t)buf * gridDim.x * kPart;
@@ -95,40 +101,64 @@ __device__ bool grid_reduce(GSmem<A> &S, const GridBufs &G, GridCtl *c, T (&v)[N
     for (int u = 1; u < nw; ++u) s = kind[q] ? fmax(s, S.wb[u * kPart + q]) : s + S.wb[u * kPart + q];
     part[(size_t)blockIdx.x * kPart + q] = s;
   }
-  if (!grid_sync(c)) return false;
-  if (NV <= 8) {
-    for (int q = w; q < NV; q += nw) {
-      double s = kind[q] ? -INFINITY : 0.0;
-      for (int b = lane; b < (int)gridDim.x; b += 32) {
-        const double x = __ldcg(part + (size_t)b * kPart + q);  // L2: another block wrote it
-        s = kind[q] ? fmax(s, x) : s + x;
-      }
-      s = kind[q] ? warp_max(s) : warp_sum(s);
-      if (lane == 0) S.tot[q] = s;
+  if (!grid_sync(S, c)) return false;
+  for (int q = w; q < NV; q += nw) {
+    double s = kind[q] ? -INFINITY : 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) {
+      const double x = __ldcg(part + (size_t)b * kPart + q);  // L2: another block wrote it
+      s = kind[q] ? fmax(s, x) : s + x;
     }
-  } else {
-    // many values: block q combines value q over all blocks and publishes it, then a second
-    // barrier, and every block reads the NV totals (instead of every block reading NV x grid
-    // partials)
-    double *res = G.res + (size_t)buf * kPart;
-    for (int q = blockIdx.x; q < NV; q += gridDim.x) {
-      double s = kind[q] ? -INFINITY : 0.0;
-      for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-        const double x = __ldcg(part + (size_t)b * kPart + q);
-        s = kind[q] ? fmax(s, x) : s + x;
+    s = kind[q] ? warp_max(s) : warp_sum(s);
+    if (lane == 0) S.tot[q] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) S.rbuf = buf ^ 1;
+  __syncthreads();
+  return true;
+}
+
+// The same for the nch chunks of 32 sums of a batch step's first reduction.  The lanes of a warp
+// reduce-scatter a chunk (31 additions per lane where 32 butterflies took 160: the binary64 additions,
+// two lanes per SM and clock, were most of this reduction's time); after the barrier warp u does the
+// same with the partials of blocks 32 u .. 32 u + 31, and one thread per value adds the warps' totals.
+template <class A>
+__device__ bool grid_reduce_chunks(GSmem<A> &S, const GridBufs &G, GridCtl *c, double (&v0)[32], double (&v1)[32], int nch) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int buf = S.rbuf;
+  double *part = G.part + (size_t)buf * gridDim.x * kPart;
+  warp_reduce_scatter<double, 32>(v0);
+  S.wb[w * kPart + lane] = v0[0];
+  if (nch > 1) {
+    warp_reduce_scatter<double, 32>(v1);
+    S.wb[w * kPart + 32 + lane] = v1[0];
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < 32 * nch; q += blockDim.x) {
+    double s = S.wb[q];
+    for (int u = 1; u < nw; ++u) s = s + S.wb[u * kPart + q];
+    part[(size_t)blockIdx.x * kPart + q] = s;
+  }
+  if (!grid_sync(S, c)) return false;
+  for (int h = 0; h < nch; ++h) {
+#pragma unroll
+    for (int q = 0; q < 32; ++q) v0[q] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+      const double2 *x = (const double2 *)(part + (size_t)b * kPart + 32 * h);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const double2 t = __ldcg(x + q);
+        v0[2 * q] += t.x;
+        v0[2 * q + 1] += t.y;
       }
-      s = kind[q] ? warp_max(s) : warp_sum(s);
-      if (lane == 0) S.wb[w] = s;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double t = S.wb[0];
-        for (int u = 1; u < nw; ++u) t = kind[q] ? fmax(t, S.wb[u]) : t + S.wb[u];
-        res[q] = t;
-      }
-      __syncthreads();
     }
-    if (!grid_sync(c)) return false;
-    for (int q = threadIdx.x; q < NV; q += blockDim.x) S.tot[q] = __ldcg(res + q);
+    if (32 * w < (int)gridDim.x) warp_reduce_scatter<double, 32>(v0);  // else all zeros
+    S.wb[w * kPart + 32 * h + lane] = v0[0];
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < 32 * nch; q += blockDim.x) {
+    double t = S.wb[q];
+    for (int u = 1; u < nw; ++u) t = t + S.wb[u * kPart + q];
+    S.tot[q] = t;
   }
   __syncthreads();
   if (threadIdx.x == 0) S.rbuf = buf ^ 1;
@@ -145,23 +175,45 @@ __device__ bool grid_scan(GSmem<A> &S, const GridBufs &G, GridCtl *c, int32_t *a
   const int lo = min(len, b * chunk), hi = min(len, lo + chunk);
   block_scan_inplace(a + lo, hi - lo, S.sh);
   if (threadIdx.x == 0) G.ipart[b] = (hi > lo) ? a[hi - 1] : 0;
-  if (!grid_sync(c)) return false;
-  if (threadIdx.x == 0) {
+  if (!grid_sync(S, c)) return false;
+  if (threadIdx.x < 32) {  // the blocks before this one, and all of them
     long long off = 0, tot = 0;
-    for (int u = 0; u < nb; ++u) {
-      const int v = *(volatile const int *)&G.ipart[u];
-      if (u < b) off += v;
+    for (int u = threadIdx.x; u < nb; u += 32) {
+      const int v = __ldcg(&G.ipart[u]);
+      off += u < b ? v : 0;
       tot += v;
     }
-    S.iv[0] = off;
-    S.iv[1] = tot;
+    off = warp_sum(off);
+    tot = warp_sum(tot);
+    if (threadIdx.x == 0) { S.iv[0] = off; S.iv[1] = tot; }
   }
   __syncthreads();
   const int off = (int)S.iv[0];
   for (int i = lo + threadIdx.x; i < hi; i += blockDim.x) a[i] += off;
-  return grid_sync(c);
+  return grid_sync(S, c);
 }
 
+// Forces on circle pos from the entries col[t0 .. t1) of its row, and its share of the batch energy (the
+// pairs with a circle outside the batch [b, e) or inside it with a smaller index), one entry at a time:
+// two per step are no faster here.
+template <class A, typename PP>
+__device__ __forceinline__ void grid_row(const PP xi, const int32_t *col, int t0, int t1, const PP *xw, int b, int e,
+                                         int pos, typename A::vec_t &gx, typename A::vec_t &gy,
+                                         typename A::acc_t &ei) {
+  using vec_t = typename A::vec_t;
+  using acc_t = typename A::acc_t;
+  for (int t = t0; t < t1; ++t) {
+    const int j = col[t];
+    vec_t fx, fy;
+    const acc_t d = A::pair(xi, xw[j], fx, fy);
+    gx += fx; gy += fy;
+    if (j < b || j >= e || j < pos) ei += d * d;
+  }
+}
+
+// One block per SM: the blocks' sums are grouped by it.  100000 circles at the benchmark's settings: 75 ms
+// per descent, 137 ms with 72 binary64 butterflies per step, six barriers per step, twelve per list build
+// and the scans' block totals added one by one.
 template <class A>
 __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, int q, GridBufs G, GridCtl *ctl) {
   using pos_t = typename A::pos_t;
@@ -182,7 +234,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
   const sc_t c1 = (sc_t)P.c1, step_max = (sc_t)P.step_max, two_skin = (sc_t)(2.0 * P.rebuild_disp);
   const sc_t gsum_tol = (sc_t)P.gsum_tol, curv_eps = (sc_t)P.curv_eps;
 
-  if (tid == 0) S.rbuf = 0;
+  if (tid == 0) { S.rbuf = 0; S.barriers = 0; }
   __syncthreads();
   if (A::kId == 2) {  // the polish runs only on instances the FP32 descent left near zero energy
     if (!(O->E32 <= P.polish_gate) || O->status32 >= 4) {
@@ -197,7 +249,8 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
   const int k = (P.k_override > 0) ? min(P.k_override, D.k) : D.k;
   PP *xw = (PP *)((double2 *)P.xw + D.off), *xb = (PP *)((double2 *)P.xb + D.off), *xo = (PP *)((double2 *)P.xo + D.off);
   VV *g = (VV *)((double2 *)P.g + D.off), *gt = (VV *)((double2 *)P.gt + D.off), *dv = (VV *)((double2 *)P.d + D.off);
-  VV *Sv = (VV *)P.S + 2 * (int64_t)mm * D.off, *Yv = Sv + (int64_t)mm * n;
+  using SP = SecantPair<vec_t>;
+  SP *SY = (SP *)P.S + (int64_t)mm * D.off;
   int32_t *perm = P.perm + D.off;
   uint64_t *skey = P.skey + D.off;
   int32_t *rp = P.rp + D.rp_off;
@@ -209,6 +262,10 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
   const CellGrid Gc = (A::kId == 1) ? CellGrid{D.R, D.inv_cs, (float)D.R, D.inv_f, D.ncx_f, true}
                                     : CellGrid{D.R, D.inv_cs, 0.f, 0.f, D.ncx, false};
   const pos_t lc2 = (pos_t)(P.l_cut * P.l_cut);
+  // the cell counters for the next build: cleared where nothing reads them before the next barrier
+  auto clear_cells = [&]() {
+    for (int c = gid; c <= Gc.nc * Gc.nc; c += gstride) cells[c] = 0;
+  };
   int status = 3;
   bool ok = true;
 
@@ -243,15 +300,15 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
   };
   if (ok) {
     for (int i = gid; i < n; i += gstride) atomicAdd(&G.bucket[bucket_of(skey[i]) + 1], 1);
-    ok = grid_sync(ctl) && grid_scan(S, G, ctl, G.bucket + 1, nbk);
+    ok = grid_sync(S, ctl) && grid_scan(S, G, ctl, G.bucket + 1, nbk);
   }
   if (ok) {
     int32_t *bfill = G.bucket + nbk + 1;
     for (int c = gid; c < nbk; c += gstride) bfill[c] = G.bucket[c];
-    ok = grid_sync(ctl);
+    ok = grid_sync(S, ctl);
     if (ok) {
       for (int i = gid; i < n; i += gstride) perm[atomicAdd(&bfill[bucket_of(skey[i])], 1)] = i;
-      ok = grid_sync(ctl);
+      ok = grid_sync(S, ctl);
     }
   }
   if (ok) {
@@ -271,7 +328,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
         perm[b + 1] = v;
       }
     }
-    ok = grid_sync(ctl);
+    ok = grid_sync(S, ctl);
   }
   // ---- 2. renumber in partition order
   int bad = 0;
@@ -285,6 +342,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
       xw[p] = v;
       xb[p] = v;
     }
+    clear_cells();
     double vb[1] = {(double)bad};
     const int kind[1] = {1};
     ok = grid_reduce<A, 1, double>(S, G, ctl, vb, kind);
@@ -300,32 +358,29 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
   // ---- neighbor lists over the grid; false on overflow or a barrier failure (status set)
   auto build = [&]() -> bool {
     const int ncell = Gc.nc * Gc.nc;
-    int32_t *cstart = cells, *cfill = cells + ncell + 1;
-    for (int c = gid; c <= ncell; c += gstride) cstart[c] = 0;
+    int32_t *cstart = cells;
+    // scratch in the direction, which no batch step needs across a build: arrival rank of a circle in
+    // its cell, circles by (cell, arrival)
+    int32_t *rank = (int32_t *)dv, *tmp = rank + n;
     if (gid == 0) { *G.hash = 0ull; rp[0] = 0; }
-    if (!grid_sync(ctl)) return false;
-    for (int i = gid; i < n; i += gstride) {
+    for (int i = gid; i < n; i += gstride) {  // the counters are zero: cleared after the last build
       const uint32_t key = grid_key<pos_t>(xw[i], Gc);
       ckey[i] = key;
-      atomicAdd(&cstart[key + 1], 1);
+      rank[i] = atomicAdd(&cstart[key + 1], 1);
     }
-    if (!grid_sync(ctl) || !grid_scan(S, G, ctl, cstart + 1, ncell)) return false;
-    for (int c = gid; c < ncell; c += gstride) cfill[c] = cstart[c];
-    if (!grid_sync(ctl)) return false;
-    for (int i = gid; i < n; i += gstride) corder[atomicAdd(&cfill[ckey[i]], 1)] = i;
-    if (!grid_sync(ctl)) return false;
-    for (int c = gid; c < ncell; c += gstride) {
-      const int lo = cstart[c], hi = cstart[c + 1];
-      for (int a = lo + 1; a < hi; ++a) {
-        const int v = corder[a];
-        int b = a - 1;
-        while (b >= lo && corder[b] > v) { corder[b + 1] = corder[b]; --b; }
-        corder[b + 1] = v;
-      }
+    if (!grid_sync(S, ctl) || !grid_scan(S, G, ctl, cstart + 1, ncell)) return false;
+    for (int i = gid; i < n; i += gstride) tmp[cstart[ckey[i]] + rank[i]] = i;
+    if (!grid_sync(S, ctl)) return false;
+    // arrival order to index order (a circle's place in its cell is the number of smaller indices
+    // there), with the coordinates in cell order
+    for (int p = gid; p < n; p += gstride) {
+      const int i = tmp[p], c = (int)ckey[i];
+      int r = cstart[c];
+      for (int q0 = cstart[c], hi = cstart[c + 1]; q0 < hi; ++q0) r += tmp[q0] < i;
+      corder[r] = i;
+      xo[r] = xw[i];
     }
-    if (!grid_sync(ctl)) return false;
-    for (int p = gid; p < n; p += gstride) xo[p] = xw[corder[p]];  // coordinates in cell order
-    if (!grid_sync(ctl)) return false;
+    if (!grid_sync(S, ctl)) return false;
     const int nc = Gc.nc;
     for (int q0 = gid; q0 < n; q0 += gstride) {
       const int i = corder[q0];
@@ -340,7 +395,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
       }
       rp[i + 1] = cntn;
     }
-    if (!grid_sync(ctl) || !grid_scan(S, G, ctl, rp + 1, n)) return false;
+    if (!grid_sync(S, ctl) || !grid_scan(S, G, ctl, rp + 1, n)) return false;
     const long long total = S.iv[1];
     if (total > cap) { status = 4; return false; }
     unsigned long long h = 0ull;
@@ -365,7 +420,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
     if ((tid & 31) == 0) atomicAdd(G.hash, h);
-    if (!grid_sync(ctl)) return false;
+    if (!grid_sync(S, ctl)) return false;
     return true;
   };
   auto anm_rebuild = [&]() -> bool {
@@ -376,8 +431,9 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
     else if (len < (1 << 30)) len *= 2;
     cnt = 0;
     for (int p = gid; p < n; p += gstride) xb[p] = xw[p];
+    clear_cells();
     Dmax = 0;
-    return grid_sync(ctl);
+    return grid_sync(S, ctl);
   };
   auto full_energy = [&](bool &good) -> acc_t {
     double e = 0.0;
@@ -407,6 +463,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
   else {
     builds = 1;
     hcur = *(volatile unsigned long long *)G.hash;
+    clear_cells();  // the energy's reduction holds the barrier
     bool good = true;
     E = full_energy(good);
     if (!good) status = 6;
@@ -416,7 +473,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
   for (int u = tid; u < k * kRing; u += blockDim.x) S.ring[u / kRing][u % kRing] = 0;
   // every block keeps identical Gram matrices (built from identical totals) in its own slice
   vec_t *gram_mine = (vec_t *)G.gram + (size_t)blockIdx.x * G.kmax * kBasis * kBasis;
-  for (int u = tid; u < k * kBasis * kBasis; u += blockDim.x) gram_mine[u] = vec_t(0);
+  for (int u = tid; u < k * kGram; u += blockDim.x) (k <= kGramOnChip ? S.gram : gram_mine)[u] = vec_t(0);
   __syncthreads();
 
   const int q_ = n / k, r_ = n % k;
@@ -435,82 +492,78 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
         fresh = false;
       }
       int *ring = S.ring[p];
-      vec_t *Gm = gram_mine + (size_t)p * kBasis * kBasis;
+      vec_t *Gm = (k <= kGramOnChip ? S.gram : gram_mine) + (size_t)p * kGram;
       const int count0 = ring[0], st = ring[1], pending = ring[2 + KS];
       // ---- pass A
-      double vA[NV1 + 1];  // the dots, and the batch energy last
-      int kindA[NV1 + 1];
+      const int nch = mm > kSlotsPerChunk ? 2 : 1;
+      double vA[32], vB2[32];  // the dots in chunks of six slots; chunk 0 with g'g, s's, s'y, y'y, E_p
 #pragma unroll
-      for (int u = 0; u <= NV1; ++u) { vA[u] = 0.0; kindA[u] = 0; }
+      for (int u = 0; u < 32; ++u) vA[u] = vB2[u] = 0.0;
       if (fresh) { VV *t_ = g; g = gt; gt = t_; }
       for (int pos = b + gid; pos < e; pos += gstride) {
+        SP pr[kSlotsPerChunk];
+        load_slots<0, kSlotsPerChunk>(SY, mm, (int64_t)n, pos, pr);
+        SP pp{};
+        if (pending) pp = ld_pair(SY + (int64_t)st * n + pos);
         const PP xi = xw[pos];
         xo[pos] = xi;
         VV gi;
         if (!fresh) {
           vec_t gx = 0, gy = 0;
           acc_t ei = 0;
-          for (int t = rp[pos]; t < rp[pos + 1]; ++t) {
-            const int j = col[t];
-            vec_t fx, fy;
-            const acc_t d = A::pair(xi, xw[j], fx, fy);
-            gx += fx; gy += fy;
-            if (j < b || j >= e || j < pos) ei += d * d;
-          }
+          grid_row<A, PP>(xi, col, rp[pos], rp[pos + 1], xw, b, e, pos, gx, gy, ei);
           vec_t fx, fy;
           const acc_t d0 = A::wall(xi, R, Rm1sq, fx, fy);
           gx += fx; gy += fy;
-          vA[NV1] += (double)(ei + d0 * d0);
+          vA[PA_E] += (double)(ei + d0 * d0);
           gi.x = gx; gi.y = gy;
           g[pos] = gi;
         } else {
           gi = g[pos];
         }
-        vA[0] += (double)(gi.x * gi.x + gi.y * gi.y);
-        VV sp, yp;
-        if (pending) { sp = Sv[(int64_t)st * n + pos]; yp = Yv[(int64_t)st * n + pos]; }
-#pragma unroll
-        for (int a = 0; a < kMaxSlots; ++a) {
-          if (a < mm) {
-            const VV s_ = Sv[(int64_t)a * n + pos], y_ = Yv[(int64_t)a * n + pos];
-            vA[1 + a] += (double)(gi.x * s_.x + gi.y * s_.y);
-            vA[1 + KS + a] += (double)(gi.x * y_.x + gi.y * y_.y);
-            if (pending) {
-              vA[OP + a] += (double)(sp.x * s_.x + sp.y * s_.y);
-              vA[OP + KS + a] += (double)(sp.x * y_.x + sp.y * y_.y);
-              vA[OP + 2 * KS + a] += (double)(yp.x * s_.x + yp.y * s_.y);
-              vA[OP + 3 * KS + a] += (double)(yp.x * y_.x + yp.y * y_.y);
-            }
-          }
-        }
+        const VV sp = pp.s, yp = pp.y;
+        vA[PA_GG] += (double)(gi.x * gi.x + gi.y * gi.y);
         if (pending) {
-          vA[OP + 4 * KS + 0] += (double)(sp.x * sp.x + sp.y * sp.y);
-          vA[OP + 4 * KS + 1] += (double)(sp.x * yp.x + sp.y * yp.y);
-          vA[OP + 4 * KS + 2] += (double)(yp.x * yp.x + yp.y * yp.y);
+          vA[PA_SS] += (double)(sp.x * sp.x + sp.y * sp.y);
+          vA[PA_SY] += (double)(sp.x * yp.x + sp.y * yp.y);
+          vA[PA_YY] += (double)(yp.x * yp.x + yp.y * yp.y);
+        }
+        auto dots = [&](double *v, const SP &q) {
+          v[0] += (double)(gi.x * q.s.x + gi.y * q.s.y);
+          v[1] += (double)(gi.x * q.y.x + gi.y * q.y.y);
+          if (pending) {
+            v[2] += (double)(yp.x * q.s.x + yp.y * q.s.y);
+            v[3] += (double)(yp.x * q.y.x + yp.y * q.y.y);
+          }
+        };
+#pragma unroll
+        for (int a = 0; a < kSlotsPerChunk; ++a)
+          if (a < mm) dots(vA + 4 * a, pr[a]);
+        if (nch > 1) {
+          load_slots<kSlotsPerChunk, kMaxSlots - kSlotsPerChunk>(SY, mm, (int64_t)n, pos, pr);
+#pragma unroll
+          for (int a = 0; a < kMaxSlots - kSlotsPerChunk; ++a)
+            if (kSlotsPerChunk + a < mm) dots(vB2 + 4 * a, pr[a]);
         }
       }
-      if (!grid_reduce<A, NV1 + 1, double>(S, G, ctl, vA, kindA)) { status = 6; break; }
-      const acc_t Ep = fresh ? E : (acc_t)S.tot[NV1];
-      const vec_t gg = (vec_t)S.tot[0];
+      if (!grid_reduce_chunks<A>(S, G, ctl, vA, vB2, nch)) { status = 6; break; }
+      const acc_t Ep = fresh ? E : (acc_t)S.tot[PA_E];
+      const vec_t gg = (vec_t)S.tot[PA_GG];
       const sc_t gnorm = sqrt((sc_t)gg);
       gsum += gnorm;
       fresh = false;
       if (pending) {  // curvature test and push (identical in every block)
-        const vec_t ss = (vec_t)S.tot[OP + 4 * KS], sy = (vec_t)S.tot[OP + 4 * KS + 1],
-                    yy = (vec_t)S.tot[OP + 4 * KS + 2];
+        const vec_t ss = (vec_t)S.tot[PA_SS], sy = (vec_t)S.tot[PA_SY], yy = (vec_t)S.tot[PA_YY];
         const bool push = (sc_t)sy > curv_eps * sqrt((sc_t)ss) * sqrt((sc_t)yy) && P.m > 0;
         if (push) {
           if (tid < count0) {
             const int sl = ring[2 + tid];
-            Gm[st * kBasis + sl] = Gm[sl * kBasis + st] = (vec_t)S.tot[OP + sl];
-            Gm[st * kBasis + KS + sl] = Gm[(KS + sl) * kBasis + st] = (vec_t)S.tot[OP + KS + sl];
-            Gm[(KS + st) * kBasis + sl] = Gm[sl * kBasis + KS + st] = (vec_t)S.tot[OP + 2 * KS + sl];
-            Gm[(KS + st) * kBasis + KS + sl] = Gm[(KS + sl) * kBasis + KS + st] = (vec_t)S.tot[OP + 3 * KS + sl];
+            Gm[sl * KS + st] = (vec_t)S.tot[pa_idx(sl, 2)];
+            Gm[kYY + st * KS + sl] = Gm[kYY + sl * KS + st] = (vec_t)S.tot[pa_idx(sl, 3)];
           }
           if (tid == 0) {
-            Gm[st * kBasis + st] = ss;
-            Gm[st * kBasis + KS + st] = Gm[(KS + st) * kBasis + st] = sy;
-            Gm[(KS + st) * kBasis + KS + st] = yy;
+            Gm[st * KS + st] = sy;
+            Gm[kYY + st * KS + st] = yy;
           }
         }
         __syncthreads();
@@ -548,24 +601,24 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
         const int lane = tid;
         const bool act = lane < count;
         const int sl = act ? ring[2 + lane] : 0;
-        const vec_t rho = act ? vec_t(1) / Gm[sl * kBasis + KS + sl] : vec_t(0);
-        vec_t acc = act ? (vec_t)S.tot[1 + sl] : vec_t(0);
+        const vec_t rho = act ? vec_t(1) / Gm[sl * KS + sl] : vec_t(0);
+        vec_t acc = act ? (vec_t)S.tot[pa_idx(sl, 0)] : vec_t(0);
         vec_t my_alpha = 0, my_w = 0, gam = 1;
         for (int cc = count - 1; cc >= 0; --cc) {
           const vec_t a = __shfl_sync(0xffffffffu, rho * acc, cc);
           if (lane == cc) my_alpha = a;
           const int slc = ring[2 + cc];
-          if (lane < cc) acc -= a * Gm[sl * kBasis + KS + slc];
+          if (lane < cc) acc -= a * Gm[sl * KS + slc];
         }
         if (count > 0) {
           const int nw_ = ring[2 + count - 1];
-          gam = Gm[nw_ * kBasis + KS + nw_] / Gm[(KS + nw_) * kBasis + KS + nw_];
+          gam = Gm[nw_ * KS + nw_] / Gm[kYY + nw_ * KS + nw_];
         }
-        vec_t t = act ? (vec_t)S.tot[1 + KS + sl] : vec_t(0);
+        vec_t t = act ? (vec_t)S.tot[pa_idx(sl, 1)] : vec_t(0);
         for (int dd = 0; dd < count; ++dd) {
           const vec_t ad = __shfl_sync(0xffffffffu, my_alpha, dd);
           const int sld = ring[2 + dd];
-          if (act) t -= ad * Gm[(KS + sl) * kBasis + KS + sld];
+          if (act) t -= ad * Gm[kYY + sl * KS + sld];
         }
         vec_t acc2 = gam * t;
         for (int cc = 0; cc < count; ++cc) {
@@ -573,7 +626,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
           const vec_t w = __shfl_sync(0xffffffffu, my_alpha, cc) - bcc;
           if (lane == cc) my_w = w;
           const int slc = ring[2 + cc];
-          if (act && lane > cc) acc2 += w * Gm[slc * kBasis + KS + sl];
+          if (act && lane > cc) acc2 += w * Gm[slc * KS + sl];
         }
         for (int u = lane; u < kBasis; u += 32) S.coef[u] = vec_t(0);
         __syncwarp();
@@ -602,12 +655,19 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
             const VV gi = g[pos];
             const vec_t cg = S.coef[GI];
             vec_t dx = cg * gi.x, dy = cg * gi.y;
-            for (int c = 0; c < cnt_now; ++c) {
-              const int sl = ring[2 + c];
-              const VV s_ = Sv[(int64_t)sl * n + pos], y_ = Yv[(int64_t)sl * n + pos];
-              const vec_t cs = S.coef[sl], cy = S.coef[KS + sl];
-              dx += cs * s_.x + cy * y_.x;
-              dy += cs * s_.y + cy * y_.y;
+            for (int c0 = 0; c0 < cnt_now; c0 += 5) {  // five pairs in flight at a time
+              SP pr[5];
+#pragma unroll
+              for (int u = 0; u < 5; ++u) pr[u] = ld_pair(SY + (int64_t)ring[2 + min(c0 + u, cnt_now - 1)] * n + pos);
+#pragma unroll
+              for (int u = 0; u < 5; ++u)
+                if (c0 + u < cnt_now) {
+                  const int sl = ring[2 + c0 + u];
+                  const VV s_ = pr[u].s, y_ = pr[u].y;
+                  const vec_t cs = S.coef[sl], cy = S.coef[KS + sl];
+                  dx += cs * s_.x + cy * y_.x;
+                  dy += cs * s_.y + cy * y_.y;
+                }
             }
             VV dd; dd.x = dx; dd.y = dy;
             dv[pos] = dd;
@@ -636,20 +696,14 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
             v.y = xo_.y + (pos_t)(al * (sc_t)dd.y);
             xw[pos] = v;
           }
-          if (!grid_sync(ctl)) { status = 6; break; }
+          if (!grid_sync(S, ctl)) { status = 6; break; }
           double vD[2] = {0.0, 0.0};
           const int kindD[2] = {0, 1};
           for (int pos = b + gid; pos < e; pos += gstride) {
             const PP xi = xw[pos];
             vec_t gx = 0, gy = 0;
             acc_t ei = 0;
-            for (int t = rp[pos]; t < rp[pos + 1]; ++t) {
-              const int j = col[t];
-              vec_t fx, fy;
-              const acc_t d = A::pair(xi, xw[j], fx, fy);
-              gx += fx; gy += fy;
-              if (j < b || j >= e || j < pos) ei += d * d;
-            }
+            grid_row<A, PP>(xi, col, rp[pos], rp[pos + 1], xw, b, e, pos, gx, gy, ei);
             vec_t fx, fy;
             const acc_t d0 = A::wall(xi, R, Rm1sq, fx, fy);
             gx += fx; gy += fy;
@@ -669,7 +723,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
         if (status != 3) break;
         if (!accepted) {
           for (int pos = b + gid; pos < e; pos += gstride) xw[pos] = xo[pos];
-          if (!grid_sync(ctl)) { status = 6; break; }
+          if (!grid_sync(S, ctl)) { status = 6; break; }
         }
       }
       if (status != 3) break;
@@ -684,8 +738,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
           VV s_; s_.x = (vec_t)(xn.x - x0.x); s_.y = (vec_t)(xn.y - x0.y);
           const VV gn = gt[pos], go = g[pos];
           VV y_; y_.x = gn.x - go.x; y_.y = gn.y - go.y;
-          Sv[(int64_t)stg * n + pos] = s_;
-          Yv[(int64_t)stg * n + pos] = y_;
+          st_pair(SY + (int64_t)stg * n + pos, s_, y_);
         }
         __syncthreads();
         if (tid == 0) ring[2 + KS] = 1;
@@ -719,10 +772,10 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
     }
     if (P.budget_ns > 0) {
       // every block must take the same decision: block 0 reads the clock, a barrier publishes it
-      if (gid == 0) G.res[2 * kPart] = (globaltimer_ns() - *P.t0 > P.budget_ns) ? 1.0 : 0.0;
-      if (!grid_sync(ctl)) { status = 6; break; }
-      const bool late = *(volatile double *)&G.res[2 * kPart] > 0.5;
-      if (!grid_sync(ctl)) { status = 6; break; }
+      if (gid == 0) G.res[0] = (globaltimer_ns() - *P.t0 > P.budget_ns) ? 1.0 : 0.0;
+      if (!grid_sync(S, ctl)) { status = 6; break; }
+      const bool late = *(volatile double *)&G.res[0] > 0.5;
+      if (!grid_sync(S, ctl)) { status = 6; break; }
       if (late) { status = 6; break; }
     }
   }
@@ -773,7 +826,9 @@ template <class A> cudaError_t coop_launch(const DescendParams &p, int q, const 
 // flag raised.  Block 0 reports whether it saw the barrier fail and how long it waited.
 __global__ void barrier_selftest_kernel(GridCtl *c, long long timeout_ns, int *failed, long long *waited) {
   const long long t0 = globaltimer_ns();
-  const bool ok = grid_sync_n(c, gridDim.x + 1u, timeout_ns);
+  __shared__ unsigned done;
+  if (threadIdx.x == 0) done = 0;
+  const bool ok = grid_sync_n(c, gridDim.x + 1u, &done, timeout_ns);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *failed = ok ? 0 : 1;
     *waited = globaltimer_ns() - t0;

@@ -97,12 +97,12 @@ cudaError_t launch_stamp(long long *t0, cudaStream_t s);
 
 // Whole-GPU descent of one large instance (pecc_grid.cu).
 struct GridCtl {
-  unsigned int count, gen;  // barrier arrivals, generation
-  int err, pad;             // a wait timed out
+  unsigned int count;  // barrier arrivals, over all barriers of a launch
+  int err;             // a wait timed out
 };
 struct GridBufs {
   double *part;             // [grid][72] block partials
-  double *res;              // [72] totals
+  double *res;              // [1] time-budget flag
   int32_t *ipart;           // [grid] block totals of integer scans
   int32_t *bucket;          // [2 (n / 4) + 2] partition buckets
   unsigned long long *hash; // [1] pair-set digest
