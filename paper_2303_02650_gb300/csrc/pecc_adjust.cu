@@ -27,7 +27,7 @@ constexpr int kAdjW = kAdjT / 32;
 constexpr int kAdjM = kMaxSlots - 1;  // memory pairs at most
 
 struct AdjSmem {
-  double red[kAdjW][4];
+  double val[4][kAdjT + 4 * kAdjW];  // one value per thread and reduction slot, four words between warps' rows
   double tot[4];
   double sR[kAdjM], yR[kAdjM], rho[kAdjM], yy[kAdjM], alpha[kAdjM];
   int32_t sh[40];
@@ -35,26 +35,40 @@ struct AdjSmem {
   int q;
 };
 
-// Block reduction of NV values (sum, or max where mx[q]); every thread gets the totals in v.
+// Block reduction of NV values (sum, or max where mx[q]); every thread gets the totals in v.  A thread
+// leaves its values in shared memory, and warp q adds up value q: the butterfly over each warp's 32
+// values (distances 16, 8, 4, 2, 1), then the warps in order.  A lane takes eight values of one warp, so
+// the first three stages are its own additions and the eight butterflies share the warp's instructions:
+// 16 binary64 additions per value instead of 47, with two binary64 lanes per SM and clock.
 template <int NV>
 __device__ __forceinline__ void bred(AdjSmem &S, double (&v)[NV], const bool (&mx)[NV]) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) S.val[q][tid + 4 * w] = v[q];
+  __syncthreads();
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
-    const double s = mx[q] ? warp_max(v[q]) : warp_sum(v[q]);
-    if (lane == 0) S.red[w][q] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x < NV) {
-    const int q = threadIdx.x;
-    double s = S.red[0][q];
-    for (int u = 1; u < nw; ++u) s = mx[q] ? fmax(s, S.red[u][q]) : s + S.red[u][q];
-    S.tot[q] = s;
+    if (w != q) continue;
+    auto op = [&](double a, double b) { return mx[q] ? fmax(a, b) : a + b; };
+    const double *x = S.val[q] + 36 * (lane >> 2) + (lane & 3);
+    double t[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) t[m] = x[4 * m];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+      for (int m = 0; m < o; ++m) t[m] = op(t[m], t[m + o]);
+    double a = t[0];
+    a = op(a, __shfl_xor_sync(0xffffffffu, a, 2));
+    a = op(a, __shfl_xor_sync(0xffffffffu, a, 1));
+    double s = __shfl_sync(0xffffffffu, a, 0);
+#pragma unroll
+    for (int u = 1; u < kAdjW; ++u) s = op(s, __shfl_sync(0xffffffffu, a, 4 * u));
+    if (lane == 0) S.tot[q] = s;
   }
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < NV; ++q) v[q] = S.tot[q];
-  __syncthreads();
 }
 
 template <class A, typename VT>
@@ -118,11 +132,12 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
       __syncthreads();
       return true;
     };
-    // U, its gradient over x into gout, and dU/dR, at the current x and radius Rz
-    auto eval = [&](GV2 *gout, double Rz, double lam, double &U, double &gR) {
+    // U, its gradient over x into gout with its squared norm g2, and dU/dR, at the current x and radius Rz
+    auto eval = [&](GV2 *gout, double Rz, double lam, double &U, double &gR, double &g2) {
       const double Rm1sq = (Rz >= 1.0) ? (Rz - 1.0) * (Rz - 1.0) : -1.0;
-      double v[2] = {0.0, 0.0};
-      const bool mx[2] = {false, false};
+      double v[3] = {0.0, 0.0, 0.0};
+      const bool mx[3] = {false, false, false};
+      GT p1 = 0;
       for (int i = tid; i < n; i += T) {
         const double2 xi = x[i];
         GT gx = 0, gy = 0;
@@ -150,8 +165,11 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
         v[0] += e + d0 * d0;
         v[1] += d0;
         gout[i] = mk2<GT>(gx, gy);
+        p1 += gx * gx + gy * gy;
       }
-      bred<2>(S, v, mx);
+      v[2] = (double)p1;
+      bred<3>(S, v, mx);
+      g2 = v[2];
       U = v[0] + lam * Rz * Rz;
       gR = -2.0 * v[1] + 2.0 * lam * Rz;
     };
@@ -161,8 +179,8 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
     double lam = P.lambda0;
     for (int round = 0; round < P.rounds && ok; ++round) {
       int head = 0, count = 0;
-      double U0, gR;
-      eval(g, R, lam, U0, gR);
+      double U0, gR, g2;
+      eval(g, R, lam, U0, gR, g2);
       status = 3;
       for (int it = 0; it < P.max_iter; ++it) {
         if (2.0 * Dmax + P.step_max > 2.0 * P.rebuild_disp) {
@@ -170,16 +188,12 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
         }
         ++iters;
         const bool mx1[1] = {false};
-        GT p1 = 0;
-        for (int i = tid; i < n; i += T) { const GV2 gi = g[i]; p1 += gi.x * gi.x + gi.y * gi.y; }
-        double v1[1] = {(double)p1};
-        bred<1>(S, v1, mx1);
-        const double gg = v1[0] + gR * gR, gnorm = sqrt(gg);
+        const double gg = g2 + gR * gR, gnorm = sqrt(gg);
         if (!(gnorm > P.gsum_tol)) { status = 1; break; }
         for (int i = tid; i < n; i += T) zo[i] = x[i];
         const double Ro = R;
         bool accepted = false;
-        double Ut = U0, gnR = gR;
+        double Ut = U0, gnR = gR, gn2 = g2;
         for (int attempt = 0; attempt < 2 && !accepted; ++attempt) {
           if (attempt == 1) {
             if (count == 0) break;
@@ -279,7 +293,7 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
             R = Ro + al * dR;
             __syncthreads();
             ++trials;
-            eval(gn, R, lam, Ut, gnR);
+            eval(gn, R, lam, Ut, gnR, gn2);
             if (Ut <= U0 + P.c1 * al * gd) { accepted = true; break; }
             al *= 0.5;
           }
@@ -323,6 +337,7 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
         { GV2 *t_ = g; g = gn; gn = t_; }  // the trial's gradient is the next iteration's
         U0 = Ut;
         gR = gnR;
+        g2 = gn2;
         __syncthreads();
         if (P.anm) {
           ++cnt;
