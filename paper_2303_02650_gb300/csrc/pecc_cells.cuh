@@ -38,31 +38,6 @@ template <> struct Coords<double> {
   }
 };
 
-// Cell coordinate of v (the value of cell_coord) decided in binary32 where that is certain.  In
-// binary32 (v + R) inv is off by less than nc 2^-22 (three roundings of the operands, two of the
-// operations, each relative 2^-24 of at most 2 R, and R inv <= nc / 2 up to a rounding), a quarter of
-// the slack; a value further than the slack from an integer lies in the same cell.
-template <typename V>
-__device__ __forceinline__ int cell_coord_fast(V v, float vf, double R, double inv, int nc, float Rf, float invf,
-                                               float slack) {
-  const float f = (vf + Rf) * invf;
-  const float fl = floorf(f), fr = f - fl;
-  if (f < -slack) return 0;
-  if (f > (float)nc + slack) return nc - 1;
-  if (fr > slack && fr < 1.f - slack && f > 0.f && f < (float)nc) return (int)fl;
-  return cell_coord((double)v, R, inv, nc);
-}
-template <typename P>
-__device__ __forceinline__ int cell_key_fast(P p, float2 f, double R, double inv, int nc) {
-  const float Rf = (float)R, invf = (float)inv, slack = (float)nc * (1.f / 1048576.f);
-  const int cx = cell_coord_fast(p.x, f.x, R, inv, nc, Rf, invf, slack);
-  return cell_coord_fast(p.y, f.y, R, inv, nc, Rf, invf, slack) * nc + cx;
-}
-
-// Distance slack around a circle whose coordinates are at most M in absolute value, for pairs near a
-// distance l: the binary32 distance of the rounded coordinates is off by less than 2^-22 (M + l).
-__device__ __forceinline__ float dist_slack(float M, float l) { return (M + l + 8.f) * (1.f / 1048576.f); }
-
 // The neighbor predicate of Sec. 4.3 for circle i (binary32 coordinates xf, given to set()) against the
 // circle at sorted position q.
 template <typename T> struct Near;

@@ -84,12 +84,30 @@ __device__ __forceinline__ int cell_coord(double v, double R, double inv, int nc
   return (int)f;
 }
 
-template <typename T>
-__device__ __forceinline__ uint32_t cell_key(v2<T> p, double R, double inv, int nc) {
-  int cx = cell_coord((double)p.x, R, inv, nc);
-  int cy = cell_coord((double)p.y, R, inv, nc);
-  return (uint32_t)cy * (uint32_t)nc + (uint32_t)cx;
+// Cell coordinate of v (the value of cell_coord) decided in binary32 where that is certain.  In
+// binary32 (v + R) inv is off by less than nc 2^-22 (three roundings of the operands, two of the
+// operations, each relative 2^-24 of at most 2 R, and R inv <= nc / 2 up to a rounding), a quarter of
+// the slack; a value further than the slack from an integer lies in the same cell.
+template <typename V>
+__device__ __forceinline__ int cell_coord_fast(V v, float vf, double R, double inv, int nc, float Rf, float invf,
+                                               float slack) {
+  const float f = (vf + Rf) * invf;
+  const float fl = floorf(f), fr = f - fl;
+  if (f < -slack) return 0;
+  if (f > (float)nc + slack) return nc - 1;
+  if (fr > slack && fr < 1.f - slack && f > 0.f && f < (float)nc) return (int)fl;
+  return cell_coord((double)v, R, inv, nc);
 }
+template <typename P>
+__device__ __forceinline__ int cell_key_fast(P p, float2 f, double R, double inv, int nc) {
+  const float Rf = (float)R, invf = (float)inv, slack = (float)nc * (1.f / 1048576.f);
+  const int cx = cell_coord_fast(p.x, f.x, R, inv, nc, Rf, invf, slack);
+  return cell_coord_fast(p.y, f.y, R, inv, nc, Rf, invf, slack) * nc + cx;
+}
+
+// Distance slack around a circle whose coordinates are at most M in absolute value, for pairs near a
+// distance l: the binary32 distance of the rounded coordinates is off by less than 2^-22 (M + l).
+__device__ __forceinline__ float dist_slack(float M, float l) { return (M + l + 8.f) * (1.f / 1048576.f); }
 
 // Neighbor predicate of Sec. 4.3: dx*dx + dy*dy < l_cut^2 with every operation
 // correctly rounded (no contraction), in the coordinates' own precision.
@@ -209,7 +227,7 @@ __device__ __forceinline__ uint32_t grid_key(v2<T> p, const CellGrid &G) {
     int cy = !(fy >= 0.f) ? 0 : (fy >= (float)G.nc ? G.nc - 1 : (int)fy);
     return (uint32_t)cy * (uint32_t)G.nc + (uint32_t)cx;
   }
-  return cell_key<T>(p, G.R, G.inv, G.nc);
+  return (uint32_t)cell_key_fast(p, make_float2((float)p.x, (float)p.y), G.R, G.inv, G.nc);
 }
 
 // 32-bit integer finaliser (xor-shift-multiply); a pair's digest term.  The digest only
@@ -231,10 +249,10 @@ __device__ __forceinline__ unsigned long long mix32(uint32_t x) {
 // order-independent 64-bit digest of the pair set, used to tell Gamma' from Gamma.
 // Cell binning and stable key sort of one instance (the first half of a list build): ckey[i]
 // = cell of circle i, corder = circles sorted by (cell, index), cells[0..ncell] = cell starts
-// (cells[ncell + 1 ..] is scratch), xs[q] = coordinates of corder[q].
+// (cells[ncell + 1 ..] is scratch), xs[q] = coordinates of corder[q] rounded to binary32.
 template <typename T>
 __device__ void cta_cell_sort(const v2<T> *__restrict__ x, int n, const CellGrid &G, uint32_t *ckey,
-                              int32_t *corder, int32_t *cells, v2<T> *xs, int32_t *sh) {
+                              int32_t *corder, int32_t *cells, float2 *xs, int32_t *sh) {
   const int T_ = blockDim.x, t = threadIdx.x;
   const int ncell = G.nc * G.nc;
   int32_t *cstart = cells;              // ncell + 1
@@ -264,33 +282,78 @@ __device__ void cta_cell_sort(const v2<T> *__restrict__ x, int n, const CellGrid
       while (b >= lo && corder[b] > v) { corder[b + 1] = corder[b]; --b; }
       corder[b + 1] = v;
     }
-    for (int a = lo; a < hi; ++a) xs[a] = x[corder[a]];
+    for (int a = lo; a < hi; ++a) {
+      const v2<T> v = x[corder[a]];
+      xs[a] = make_float2((float)v.x, (float)v.y);
+    }
   }
   __syncthreads();
 }
 
+// The predicate for the circle at sorted position q0 against the one at qq.  Binary64: decided by the
+// binary32 copies except within the slack of the cutoff (about one pair in a million), so that a build
+// leaves the two binary64 lanes of the SM alone: they took most of a polish's and an adjustment's builds.
+template <typename T> struct SortedNear;
+template <> struct SortedNear<float> {
+  const float2 *xs;
+  float lc2;
+  float2 a;
+  __device__ __forceinline__ SortedNear(const float2 *, const int32_t *, const float2 *xs_, float lc2_)
+      : xs(xs_), lc2(lc2_) {}
+  __device__ __forceinline__ void set(int q0) { a = xs[q0]; }
+  __device__ __forceinline__ bool operator()(int qq) const { return nbr_pred(a, xs[qq], lc2); }
+};
+template <> struct SortedNear<double> {
+  const double2 *x;
+  const int32_t *order;
+  const float2 *xs;
+  double lc2;
+  float lc, lo, hi;
+  float2 a;
+  int i;
+  __device__ __forceinline__ SortedNear(const double2 *x_, const int32_t *o, const float2 *xs_, double lc2_)
+      : x(x_), order(o), xs(xs_), lc2(lc2_), lc(sqrtf((float)lc2_)) {}
+  __device__ __forceinline__ void set(int q0) {
+    a = xs[q0];
+    i = order[q0];
+    const float m = dist_slack(fabsf(a.x) + fabsf(a.y), lc);
+    const bool ok = m <= 0.25f;  // else (far out, not finite): every distance in binary64
+    lo = ok ? (lc - m) * (lc - m) : -1.f;
+    hi = ok ? (lc + m) * (lc + m) : __int_as_float(0x7f800000);
+  }
+  __device__ __forceinline__ bool operator()(int qq) const {
+    const float2 b = xs[qq];
+    const float dx = a.x - b.x, dy = a.y - b.y, s = dx * dx + dy * dy;
+    if (s > hi) return false;
+    if (s < lo) return true;
+    return nbr_pred(x[i], x[order[qq]], lc2);
+  }
+};
+
 template <typename T, typename IdxT>
 __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const CellGrid &G, T lc2,
-                                   uint32_t *ckey, int32_t *corder, int32_t *cells, v2<T> *xs, int32_t *rp,
+                                   uint32_t *ckey, int32_t *corder, int32_t *cells, v2<T> *xs_, int32_t *rp,
                                    IdxT *col, int cap, int32_t *sh, unsigned long long *hash) {
   const int T_ = blockDim.x, t = threadIdx.x;
   const int nc = G.nc;
   int32_t *cstart = cells;
+  float2 *const xs = (float2 *)xs_;
   if (t == 0 && hash) *hash = 0ull;
   cta_cell_sort<T>(x, n, G, ckey, corder, cells, xs, sh);
   if (t == 0) rp[0] = 0;
   __syncthreads();
+  SortedNear<T> near(x, corder, xs, lc2);
   // count: circles visited in cell order, candidates as three contiguous row ranges
   for (int q0 = t; q0 < n; q0 += T_) {
     const int i = corder[q0];
-    const v2<T> xi = xs[q0];
+    near.set(q0);
     const uint32_t key = ckey[i];
     const int cx = (int)(key % (uint32_t)nc), cy = (int)(key / (uint32_t)nc);
     const int bx0 = max(cx - 1, 0), bx1 = min(cx + 1, nc - 1);
     int cntn = 0;
     for (int by = max(cy - 1, 0); by <= min(cy + 1, nc - 1); ++by) {
       const int lo = cstart[by * nc + bx0], hi = cstart[by * nc + bx1 + 1];
-      for (int qq = lo; qq < hi; ++qq) cntn += nbr_pred(xi, xs[qq], lc2) && qq != q0;
+      for (int qq = lo; qq < hi; ++qq) cntn += near(qq) && qq != q0;
     }
     rp[i + 1] = cntn;
   }
@@ -301,7 +364,7 @@ __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const Cel
     unsigned long long h = 0ull;
     for (int q0 = t; q0 < n; q0 += T_) {
       const int i = corder[q0];
-      const v2<T> xi = xs[q0];
+      near.set(q0);
       const uint32_t key = ckey[i];
       const int cx = (int)(key % (uint32_t)nc), cy = (int)(key / (uint32_t)nc);
       const int bx0 = max(cx - 1, 0), bx1 = min(cx + 1, nc - 1);
@@ -310,7 +373,7 @@ __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const Cel
       for (int by = max(cy - 1, 0); by <= min(cy + 1, nc - 1); ++by) {
         const int lo = cstart[by * nc + bx0], hi = cstart[by * nc + bx1 + 1];
         for (int qq = lo; qq < hi; ++qq) {
-          if (nbr_pred(xi, xs[qq], lc2) && qq != q0) {
+          if (near(qq) && qq != q0) {
             const int j = corder[qq];
             col[w++] = (IdxT)j;
             if (hash) h += mix32((uint32_t)i * 0x9E3779B1u ^ (uint32_t)j);
