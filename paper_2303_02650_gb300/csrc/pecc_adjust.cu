@@ -29,17 +29,40 @@ constexpr int kAdjM = kMaxSlots - 1;  // memory pairs at most
 struct AdjSmem {
   double val[4][kAdjT + 4 * kAdjW];  // one value per thread and reduction slot, four words between warps' rows
   double tot[4];
+  double qR;                                 // the radius's component of the two-loop's vector
+  double coef;                               // and the coefficient of its current step
   double sR[kAdjM], yR[kAdjM], rho[kAdjM], yy[kAdjM], alpha[kAdjM];
   int32_t sh[40];
   unsigned long long hash;
   int q;
 };
 
+// The butterfly over each warp's 32 values of S.val[q] (distances 16, 8, 4, 2, 1), then the warps in
+// order; the result in every lane of the calling warp.  A lane takes eight values of one warp, so the
+// first three stages are its own additions and the eight butterflies share the warp's instructions: 16
+// binary64 additions per value instead of 47, with two binary64 lanes per SM and clock.
+template <bool MAX> __device__ __forceinline__ double block_combine(const AdjSmem &S, int q) {
+  const int lane = threadIdx.x & 31;
+  auto op = [](double a, double b) { return MAX ? fmax(a, b) : a + b; };
+  const double *x = S.val[q] + 36 * (lane >> 2) + (lane & 3);
+  double t[8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) t[m] = x[4 * m];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+    for (int m = 0; m < o; ++m) t[m] = op(t[m], t[m + o]);
+  double a = t[0];
+  a = op(a, __shfl_xor_sync(0xffffffffu, a, 2));
+  a = op(a, __shfl_xor_sync(0xffffffffu, a, 1));
+  double s = __shfl_sync(0xffffffffu, a, 0);
+#pragma unroll
+  for (int u = 1; u < kAdjW; ++u) s = op(s, __shfl_sync(0xffffffffu, a, 4 * u));
+  return s;
+}
+
 // Block reduction of NV values (sum, or max where mx[q]); every thread gets the totals in v.  A thread
-// leaves its values in shared memory, and warp q adds up value q: the butterfly over each warp's 32
-// values (distances 16, 8, 4, 2, 1), then the warps in order.  A lane takes eight values of one warp, so
-// the first three stages are its own additions and the eight butterflies share the warp's instructions:
-// 16 binary64 additions per value instead of 47, with two binary64 lanes per SM and clock.
+// leaves its values in shared memory, and warp q combines value q.
 template <int NV>
 __device__ __forceinline__ void bred(AdjSmem &S, double (&v)[NV], const bool (&mx)[NV]) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -49,21 +72,7 @@ __device__ __forceinline__ void bred(AdjSmem &S, double (&v)[NV], const bool (&m
 #pragma unroll
   for (int q = 0; q < NV; ++q) {
     if (w != q) continue;
-    auto op = [&](double a, double b) { return mx[q] ? fmax(a, b) : a + b; };
-    const double *x = S.val[q] + 36 * (lane >> 2) + (lane & 3);
-    double t[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) t[m] = x[4 * m];
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1)
-#pragma unroll
-      for (int m = 0; m < o; ++m) t[m] = op(t[m], t[m + o]);
-    double a = t[0];
-    a = op(a, __shfl_xor_sync(0xffffffffu, a, 2));
-    a = op(a, __shfl_xor_sync(0xffffffffu, a, 1));
-    double s = __shfl_sync(0xffffffffu, a, 0);
-#pragma unroll
-    for (int u = 1; u < kAdjW; ++u) s = op(s, __shfl_sync(0xffffffffu, a, 4 * u));
+    const double s = mx[q] ? block_combine<true>(S, q) : block_combine<false>(S, q);
     if (lane == 0) S.tot[q] = s;
   }
   __syncthreads();
@@ -71,8 +80,153 @@ __device__ __forceinline__ void bred(AdjSmem &S, double (&v)[NV], const bool (&m
   for (int q = 0; q < NV; ++q) v[q] = S.tot[q];
 }
 
+// Block sum of v, with which one thread forms the scalars of a two-loop step (fin): formed by every
+// thread they were eight times the binary64 instructions.
+template <class F> __device__ __forceinline__ void sum_then(AdjSmem &S, double v, F fin) {
+  const int tid = threadIdx.x, w = tid >> 5;
+  S.val[0][tid + 4 * w] = v;
+  __syncthreads();
+  if (w == 0) {
+    const double s = block_combine<false>(S, 0);
+    if (tid == 0) fin(s);
+  }
+  __syncthreads();
+}
+
+constexpr int kAdjOwn = 4;  // circles of a thread that the two-loop keeps in registers (n <= 1024)
+
+// Two-loop recursion (Nocedal & Wright, Alg. 7.4) over the stored pairs from q = (g, gR): d = -q into dv,
+// and this thread's parts of g'd and of the largest move.  S.qR: q's radius component in and out.
+// OWN: the vector stays in the threads' registers, and each pair's vectors are loaded a step ahead, behind
+// the reduction of the step before; else (n > 1024) everything goes through memory.
+template <bool OWN, typename VT, typename GT>
+__device__ __forceinline__ void two_loop(AdjSmem &S, int n, int m, int head, int count, const v2<GT> *g, v2<VT> *dv,
+                                         const v2<VT> *Sv, const v2<VT> *Yv, GT &gd, VT &dm) {
+  using V2 = v2<VT>;
+  const int tid = threadIdx.x, T = kAdjT;
+  V2 d[kAdjOwn], a0[kAdjOwn], a1[kAdjOwn], a2[kAdjOwn];
+  auto slot = [&](const V2 *B, int c) { return B + (int64_t)((head + c) % m) * n; };
+  auto load = [&](V2 (&a)[kAdjOwn], const V2 *p) {
+#pragma unroll
+    for (int u = 0; u < kAdjOwn; ++u) {
+      const int i = tid + u * T;
+      if (i < n) a[u] = p[i];
+    }
+  };
+  // f(vector element, circle) for this thread's circles in order
+  auto each = [&](auto f) {
+    if constexpr (OWN) {
+#pragma unroll
+      for (int u = 0; u < kAdjOwn; ++u) {
+        const int i = tid + u * T;
+        if (i < n) f(d[u], i, u);
+      }
+    } else {
+      for (int i = tid; i < n; i += T) {
+        V2 b = dv[i];
+        f(b, i, 0);
+        dv[i] = b;
+      }
+    }
+  };
+  // the same without a change of the vector
+  auto look = [&](auto f) {
+    if constexpr (OWN) {
+#pragma unroll
+      for (int u = 0; u < kAdjOwn; ++u) {
+        const int i = tid + u * T;
+        if (i < n) f(d[u], i, u);
+      }
+    } else {
+      for (int i = tid; i < n; i += T) f(dv[i], i, 0);
+    }
+  };
+  each([&](V2 &b, int i, int) { const v2<GT> gi = g[i]; b = mk2<VT>((VT)gi.x, (VT)gi.y); });
+  if (OWN && count > 0) load(a0, slot(Sv, count - 1));
+  for (int c = count - 1; c >= 0; --c) {
+    const int sl = (head + c) % m;
+    const V2 *s_ = Sv + (int64_t)sl * n, *y_ = Yv + (int64_t)sl * n;
+    if (OWN) {
+      load(a1, y_);
+      if (c > 0) load(a2, slot(Sv, c - 1));
+    }
+    VT pv = 0;
+    look([&](const V2 &b, int i, int u) {
+      const V2 a = OWN ? a0[u] : s_[i];
+      pv += a.x * b.x + a.y * b.y;
+    });
+    sum_then(S, (double)pv, [&](double t) {
+      const double a = S.rho[sl] * (t + S.sR[sl] * S.qR);
+      S.alpha[c] = a;
+      S.coef = a;
+      S.qR -= a * S.yR[sl];
+    });
+    const VT av = (VT)S.coef;
+    each([&](V2 &b, int i, int u) {
+      const V2 yv = OWN ? a1[u] : y_[i];
+      b.x -= av * yv.x;
+      b.y -= av * yv.y;
+    });
+    if (OWN) {
+#pragma unroll
+      for (int u = 0; u < kAdjOwn; ++u) a0[u] = a2[u];
+    }
+  }
+  if (count > 0) {
+    const int nw_ = (head + count - 1) % m;
+    if (OWN) load(a0, slot(Yv, 0));
+    __syncthreads();  // the last coefficient has been read
+    if (tid == 0) {
+      const double gam = 1.0 / (S.rho[nw_] * S.yy[nw_]);  // s'y / y'y of the newest pair
+      S.coef = gam;
+      S.qR *= gam;
+    }
+    __syncthreads();
+    const VT gv = (VT)S.coef;
+    each([&](V2 &b, int, int) { b.x *= gv; b.y *= gv; });
+  }
+  for (int c = 0; c < count; ++c) {
+    const int sl = (head + c) % m;
+    const V2 *s_ = Sv + (int64_t)sl * n, *y_ = Yv + (int64_t)sl * n;
+    if (OWN) {
+      load(a1, s_);
+      if (c + 1 < count) load(a2, slot(Yv, c + 1));
+    }
+    VT pv = 0;
+    look([&](const V2 &b, int i, int u) {
+      const V2 a = OWN ? a0[u] : y_[i];
+      pv += a.x * b.x + a.y * b.y;
+    });
+    sum_then(S, (double)pv, [&](double t) {
+      const double bta = S.rho[sl] * (t + S.yR[sl] * S.qR);
+      const double w = S.alpha[c] - bta;
+      S.coef = w;
+      S.qR += w * S.sR[sl];
+    });
+    const VT wv = (VT)S.coef;
+    each([&](V2 &b, int i, int u) {
+      const V2 sa = OWN ? a1[u] : s_[i];
+      b.x += wv * sa.x;
+      b.y += wv * sa.y;
+    });
+    if (OWN) {
+#pragma unroll
+      for (int u = 0; u < kAdjOwn; ++u) a0[u] = a2[u];
+    }
+  }
+  // d = -q; g'd and the largest move
+  each([&](V2 &b, int i, int) {
+    b.x = -b.x;
+    b.y = -b.y;
+    if (OWN) dv[i] = b;
+    const v2<GT> gi = g[i];
+    gd += gi.x * (GT)b.x + gi.y * (GT)b.y;
+    dm = max(dm, b.x * b.x + b.y * b.y);
+  });
+}
+
 template <class A, typename VT>
-__global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
+__global__ void __launch_bounds__(kAdjT, 2) adjust_kernel(AdjustParams P) {
   using V2 = v2<VT>;
   using GT = typename A::vec_t;  // the forces' and the stored gradient's type
   using GV2 = v2<GT>;
@@ -187,7 +341,6 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
           if (!rebuild(true)) { ok = false; status = 4; break; }
         }
         ++iters;
-        const bool mx1[1] = {false};
         const double gg = g2 + gR * gR, gnorm = sqrt(gg);
         if (!(gnorm > P.gsum_tol)) { status = 1; break; }
         for (int i = tid; i < n; i += T) zo[i] = x[i];
@@ -200,71 +353,17 @@ __global__ void __launch_bounds__(kAdjT) adjust_kernel(AdjustParams P) {
             count = 0;
             head = 0;
           }
-          // ---- two-loop recursion (Nocedal & Wright, Alg. 7.4) over the stored pairs; q in dv
           visits += count;
-          for (int i = tid; i < n; i += T) { const GV2 gi = g[i]; dv[i] = mk2<VT>((VT)gi.x, (VT)gi.y); }
-          double qR = gR;
-          for (int c = count - 1; c >= 0; --c) {
-            const int sl = (head + c) % P.m;
-            const V2 *s_ = Sv + (int64_t)sl * n;
-            VT pv = 0;
-            for (int i = tid; i < n; i += T) { const V2 a = s_[i], b = dv[i]; pv += a.x * b.x + a.y * b.y; }
-            double v[1] = {(double)pv};
-            bred<1>(S, v, mx1);
-            const double a = S.rho[sl] * (v[0] + S.sR[sl] * qR);
-            if (tid == 0) S.alpha[c] = a;
-            const V2 *y_ = Yv + (int64_t)sl * n;
-            const VT av = (VT)a;
-            for (int i = tid; i < n; i += T) {
-              const V2 yv = y_[i];
-              V2 b = dv[i];
-              b.x -= av * yv.x; b.y -= av * yv.y;
-              dv[i] = b;
-            }
-            qR -= a * S.yR[sl];
-          }
-          if (count > 0) {
-            const int nw_ = (head + count - 1) % P.m;
-            const double gam = 1.0 / (S.rho[nw_] * S.yy[nw_]);  // s'y / y'y of the newest pair
-            const VT gv = (VT)gam;
-            for (int i = tid; i < n; i += T) { V2 b = dv[i]; b.x *= gv; b.y *= gv; dv[i] = b; }
-            qR *= gam;
-          }
-          __syncthreads();  // alpha[] written by thread 0
-          for (int c = 0; c < count; ++c) {
-            const int sl = (head + c) % P.m;
-            const V2 *y_ = Yv + (int64_t)sl * n;
-            VT pv = 0;
-            for (int i = tid; i < n; i += T) { const V2 a = y_[i], b = dv[i]; pv += a.x * b.x + a.y * b.y; }
-            double v[1] = {(double)pv};
-            bred<1>(S, v, mx1);
-            const double bta = S.rho[sl] * (v[0] + S.yR[sl] * qR);
-            const double w = S.alpha[c] - bta;
-            const V2 *s_ = Sv + (int64_t)sl * n;
-            const VT wv = (VT)w;
-            for (int i = tid; i < n; i += T) {
-              const V2 sa = s_[i];
-              V2 b = dv[i];
-              b.x += wv * sa.x; b.y += wv * sa.y;
-              dv[i] = b;
-            }
-            qR += w * S.sR[sl];
-          }
-          // d = -q; g'd and the largest move (circles and the radius)
+          if (tid == 0) S.qR = gR;  // read by thread 0 alone until the steps below are done
           const bool mx2[2] = {false, true};
           GT p2 = 0;
           VT m2 = 0;
-          for (int i = tid; i < n; i += T) {
-            V2 b = dv[i];
-            b.x = -b.x; b.y = -b.y;
-            dv[i] = b;
-            const GV2 gi = g[i];
-            p2 += gi.x * (GT)b.x + gi.y * (GT)b.y;
-            m2 = max(m2, b.x * b.x + b.y * b.y);
-          }
+          // binary64 vectors would take the registers of a block per SM
+          if (sizeof(VT) == 4 && n <= kAdjOwn * kAdjT) two_loop<sizeof(VT) == 4, VT, GT>(S, n, P.m, head, count, g, dv, Sv, Yv, p2, m2);
+          else two_loop<false, VT, GT>(S, n, P.m, head, count, g, dv, Sv, Yv, p2, m2);
           double v2[2] = {(double)p2, (double)m2};
           bred<2>(S, v2, mx2);
-          double dR = -qR;
+          double dR = -S.qR;
           double gd = v2[0] + gR * dR;
           double dmax = sqrt(fmax(v2[1], dR * dR));
           if (!(gd < 0.0)) {  // not a descent direction: drop the memory, take -g

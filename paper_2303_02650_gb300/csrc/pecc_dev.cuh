@@ -369,7 +369,6 @@ __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const Cel
       const int cx = (int)(key % (uint32_t)nc), cy = (int)(key / (uint32_t)nc);
       const int bx0 = max(cx - 1, 0), bx1 = min(cx + 1, nc - 1);
       int w = rp[i];
-      const int first = w;
       for (int by = max(cy - 1, 0); by <= min(cy + 1, nc - 1); ++by) {
         const int lo = cstart[by * nc + bx0], hi = cstart[by * nc + bx1 + 1];
         for (int qq = lo; qq < hi; ++qq) {

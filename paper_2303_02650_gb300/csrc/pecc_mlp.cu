@@ -457,7 +457,8 @@ __global__ void __launch_bounds__(kTrT, 1) train_tc_kernel(const bf16 *__restric
                                                            const float *__restrict__ feat, const float *__restrict__ target,
                                                            int64_t rows, float *part, float *loss_part,
                                                            float *fwd_trace, float *bwd_trace) {
-  extern __shared__ __align__(128) unsigned char sm[];
+  extern __shared__ __align__(128) unsigned char sm_train[];
+  unsigned char *const sm = sm_train;
   unsigned char *w1 = sm + kTrW1, *w2 = sm + kTrW2, *w3 = sm + kTrW3, *x = sm + kTrX;
   unsigned char *h1 = sm + kTrH1, *h2 = sm + kTrH2, *h3 = sm + kTrH3, *z = sm + kTrZ, *dot = sm + kTrO;
   float *fb = (float *)(sm + kTrF), *opart = fb + kTrFo;
