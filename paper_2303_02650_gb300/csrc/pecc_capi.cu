@@ -589,6 +589,10 @@ static pecc_status plan_launch(pecc_ctx *ctx, int arith, int block = 0, int bps_
     int want = (nmax + 1) / 2;
     blk = std::min(descend_max_block(arith), std::max(64, (want + 31) / 32 * 32));
     if (many) blk = std::min(blk, 256);
+    // a small binary64 instance alone on its SM: each of the SM's four partitions issues binary64
+    // instructions by itself, so its work goes to four warps (the sums' grouping stays that of 64
+    // threads: a thread past the circles adds zeros)
+    else if (arith == 0 && nmax <= 64) blk = 128;
   }
   blk = std::min(blk, descend_max_block(arith));
   L.block = blk;

@@ -54,6 +54,9 @@ size_t descend_smem_need(int arith, int n, int k, int ncx, int block, int m, boo
              al(4 * (size_t)(n + 1)) + al(2 * (size_t)n) + al(2 * (size_t)(8 * n + 64)) + step + al(pos * n) +
              (cells <= pos * (size_t)n ? 0 : al(cells)) + al(2 * vec * (size_t)(m + 1) * n) +
              (outer ? al(2 * (size_t)(kOuterPerCircle * n + 64)) : 0);
+  if (arith == 0)  // the energy entries of a line search
+    b += al(8 * (size_t)(kEntriesPerCircle * n + 32)) + al(4 * (size_t)(kEntriesPerCircle * n + 32)) +
+         al(4 * (size_t)((n + k - 1) / k + 1));
   return b;
 }
 

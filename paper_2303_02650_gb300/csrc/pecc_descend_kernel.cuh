@@ -138,6 +138,10 @@ __host__ __device__ inline size_t batch_room(int n, int k, size_t vec, size_t po
   return step > build ? step : build;
 }
 
+// Energy entries per circle that the binary64 form lists for a line search: half of its neighbors in a
+// one-batch step, more in a batch's border rows.
+constexpr int kEntriesPerCircle = 5;
+
 // Bump allocator over dynamic shared memory; returns the fallback when the request does not fit.
 struct Carve {
   unsigned char *base;
@@ -312,6 +316,23 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
     }
     lc2L = (pos_t)(lb * lb);
     if (GL.nc > G.nc) two = false;  // its cell table must fit the scratch
+  }
+  // Binary64: room for the energy's entries of a batch, one per lane, when the block's share has any left
+  // (single small instances).  A failed first trial is followed by up to max_trials more that need the
+  // energy alone: each entry once, packed over the lanes, instead of whole rows with their forces.
+  // Binary64 instructions issue slowly and the rows' chains are long: one instance of 50 circles, 22
+  // trials per sweep, took 372 ms per 2000 sweeps with whole rows; entry by entry 200 ms on two warps and
+  // 178 ms on four.  (Three entries per thread side by side, without branches: 235 ms; listing only pairs
+  // near contact: 182 ms.)
+  const int cap_e = kEntriesPerCircle * n + 32;
+  acc_t *ed = nullptr;
+  uint32_t *ep = nullptr;
+  int32_t *es = nullptr;
+  if (A::kId == 0) {
+    ed = cv.take<acc_t>(cap_e, (acc_t *)nullptr);
+    ep = cv.take<uint32_t>(cap_e, (uint32_t *)nullptr);
+    es = cv.take<int32_t>(nbm + 1, (int32_t *)nullptr);
+    if (ed == nullptr || ep == nullptr) es = nullptr;
   }
   int32_t *perm = P.perm + D.off;
   // the partition keys borrow the list storage (8 n bytes) before the first build
@@ -777,6 +798,8 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
         const sc_t dmax = sqrt((sc_t)dmB);
         if (!(gd < sc_t(0))) break;
         sc_t al = (dmax > step_max) ? step_max / dmax : sc_t(1);
+        int ne = -1;  // energy entries of the batch (-1: not listed yet, -2: no room)
+        if (A::kId != 0 || es == nullptr) ne = -2;
         for (int tr = 0; tr < P.max_trials; ++tr) {
           // ---- pass C: trial coordinates
           for (int i = tid; i < nb; i += T) {
@@ -788,6 +811,54 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
             xw[b + i] = v;
           }
           __syncthreads();
+          if constexpr (A::kId == 0) if (tr > 0 && ne != -2) {
+            // ---- the energy alone, entry by entry; the sums take a row's entries in row order, as pass D
+            if (ne == -1) {
+              if (tid == 0) es[0] = 0;
+              for (int i = tid; i < nb; i += T) {
+                const int pos = b + i, t0 = rp[pos];
+                int c = 0;
+                for (int t = t0; t < t0 + rl[pos]; ++t) { const int j = col[t]; c += j < b || j >= e || j < pos; }
+                es[i + 1] = c;
+              }
+              __syncthreads();
+              block_scan_inplace(es + 1, nb, S.sh);
+              ne = es[nb] <= cap_e ? es[nb] : -2;
+              if (ne >= 0)
+                for (int i = tid; i < nb; i += T) {
+                  const int pos = b + i, t0 = rp[pos];
+                  int w = es[i];
+                  for (int t = t0; t < t0 + rl[pos]; ++t) {
+                    const int j = col[t];
+                    if (j < b || j >= e || j < pos) ep[w++] = ((uint32_t)pos << 16) | (uint32_t)j;
+                  }
+                }
+              __syncthreads();
+            }
+            if (ne >= 0) {
+              vec_t ux, uy;  // unused
+              for (int t = tid; t < ne; t += T) {
+                const uint32_t pj = ep[t];
+                ed[t] = A::pair(xw[pj >> 16], xw[pj & 0xffffu], ux, uy);
+              }
+              __syncthreads();
+              acc_t aE = 0;
+              vec_t none = 0;
+              for (int i = tid; i < nb; i += T) {
+                acc_t ei = 0;
+                for (int t = es[i]; t < es[i + 1]; ++t) ei += ed[t] * ed[t];
+                const acc_t d0 = A::wall(xw[b + i], R, Rm1sq, ux, uy);
+                aE += ei + d0 * d0;
+              }
+              reduce_sm<A, W>(S, rbuf, aE, none);
+              if (!(aE <= Ep + c1 * al * gd)) {  // the gradient of an accepted trial: pass D
+                ++trials;
+                Et = aE;
+                al *= sc_t(0.5);
+                continue;
+              }
+            }
+          }
           // ---- pass D: trial batch energy and gradient, displacement since the build
           acc_t aD = 0;
           vec_t cD = 0;
