@@ -283,7 +283,7 @@ __device__ __forceinline__ void descend_instance(const DescendParams &P, Smem<A,
                                    : CellGrid{D.R, D.inv_cs, 0.f, 0.f, D.ncx, false};
   // the builds' cell table lives in the positions at the last build when it fits (they are
   // rewritten right after every build)
-  const size_t ncells = 2 * (size_t)G.nc * G.nc + 2;
+  const size_t ncells = (size_t)G.nc * G.nc + 1;
   int32_t *cells = (ncells * sizeof(int32_t) <= (size_t)n * sizeof(PP)) ? (int32_t *)xb
                                                                        : cv.take<int32_t>(ncells, P.cells + D.cell_off);
   if (tid == 0) { S.corder = corder; S.ckey = ckey; S.xs = xs; S.cells = cells; }

@@ -219,15 +219,25 @@ struct CellGrid {
   bool f32;
 };
 
+// Cell of a circle as cx | cy << 16 (a grid has at most 65535 cells per side).
+template <typename T>
+__device__ __forceinline__ uint32_t grid_cell(v2<T> p, const CellGrid &G) {
+  int cx, cy;
+  if (G.f32) {
+    const float fx = ((float)p.x + G.Rf) * G.invf, fy = ((float)p.y + G.Rf) * G.invf;
+    cx = !(fx >= 0.f) ? 0 : (fx >= (float)G.nc ? G.nc - 1 : (int)fx);
+    cy = !(fy >= 0.f) ? 0 : (fy >= (float)G.nc ? G.nc - 1 : (int)fy);
+  } else {
+    const float Rf = (float)G.R, invf = (float)G.inv, slack = (float)G.nc * (1.f / 1048576.f);
+    cx = cell_coord_fast(p.x, (float)p.x, G.R, G.inv, G.nc, Rf, invf, slack);
+    cy = cell_coord_fast(p.y, (float)p.y, G.R, G.inv, G.nc, Rf, invf, slack);
+  }
+  return (uint32_t)cx | ((uint32_t)cy << 16);
+}
 template <typename T>
 __device__ __forceinline__ uint32_t grid_key(v2<T> p, const CellGrid &G) {
-  if (G.f32) {
-    float fx = ((float)p.x + G.Rf) * G.invf, fy = ((float)p.y + G.Rf) * G.invf;
-    int cx = !(fx >= 0.f) ? 0 : (fx >= (float)G.nc ? G.nc - 1 : (int)fx);
-    int cy = !(fy >= 0.f) ? 0 : (fy >= (float)G.nc ? G.nc - 1 : (int)fy);
-    return (uint32_t)cy * (uint32_t)G.nc + (uint32_t)cx;
-  }
-  return (uint32_t)cell_key_fast(p, make_float2((float)p.x, (float)p.y), G.R, G.inv, G.nc);
+  const uint32_t c = grid_cell<T>(p, G);
+  return (c >> 16) * (uint32_t)G.nc + (c & 0xffffu);
 }
 
 // 32-bit integer finaliser (xor-shift-multiply); a pair's digest term.  The digest only
@@ -241,51 +251,48 @@ __device__ __forceinline__ unsigned long long mix32(uint32_t x) {
 }
 
 // Cell binning and stable key sort, then CSR rows over the 3x3 cells.  x: n positions of
-// one instance; lists go to rp[0..n], col[0..cap).  cells: 2 * nc^2 + 2 int32 of scratch;
+// one instance; lists go to rp[0..n], col[0..cap).  cells: nc^2 + 1 int32 of scratch;
 // ckey/corder: n each; xs: n positions of scratch (the coordinates in cell order, so that
 // the three cells of a row of the 3x3 block are one contiguous range).  All pointers may
 // be shared or global memory.  Rows come in cell-scan order (deterministic).  Returns the number of entries (block-uniform); > cap means
 // overflow and the rows are then not written.  hash (shared, may be null) receives an
 // order-independent 64-bit digest of the pair set, used to tell Gamma' from Gamma.
-// Cell binning and stable key sort of one instance (the first half of a list build): ckey[i]
-// = cell of circle i, corder = circles sorted by (cell, index), cells[0..ncell] = cell starts
-// (cells[ncell + 1 ..] is scratch), xs[q] = coordinates of corder[q] rounded to binary32.
+// Cell binning and stable key sort of one instance (the first half of a list build): ckey[i] = cell
+// of circle i (cx | cy << 16), corder = circles sorted by (cell, index), cells[0..ncell] = cell starts,
+// xs[q] = coordinates of corder[q] rounded to binary32.  tmp: n int32 of scratch.  A circle keeps its
+// arrival rank from the count, so the scatter needs no second cursor, and then finds its place in its
+// cell as the number of smaller indices there: every step one circle per thread (cells sorted one per
+// thread, circle after circle, left most threads waiting).
 template <typename T>
 __device__ void cta_cell_sort(const v2<T> *__restrict__ x, int n, const CellGrid &G, uint32_t *ckey,
-                              int32_t *corder, int32_t *cells, float2 *xs, int32_t *sh) {
+                              int32_t *corder, int32_t *cells, float2 *xs, int32_t *tmp, int32_t *sh) {
   const int T_ = blockDim.x, t = threadIdx.x;
-  const int ncell = G.nc * G.nc;
-  int32_t *cstart = cells;              // ncell + 1
-  int32_t *cfill = cells + ncell + 1;   // ncell
+  const int nc = G.nc, ncell = nc * nc;
+  int32_t *cstart = cells;  // ncell + 1
   for (int c = t; c <= ncell; c += T_) cstart[c] = 0;
   __syncthreads();
   for (int i = t; i < n; i += T_) {
-    uint32_t key = grid_key<T>(x[i], G);
-    ckey[i] = key;
-    atomicAdd(&cstart[key + 1], 1);
+    const uint32_t c = grid_cell<T>(x[i], G);
+    ckey[i] = c;
+    corder[i] = atomicAdd(&cstart[(int)(c >> 16) * nc + (int)(c & 0xffffu) + 1], 1);
   }
   __syncthreads();
-  // the scan leaves the cell starts in cstart[1..] and, shifted by one, the fill cursors in cfill
-  // (cfill[c] = cstart[c]: cell 0 starts at 0)
-  if (t == 0) cfill[0] = 0;
-  block_scan_inplace(cstart + 1, ncell, sh, cfill + 1);
+  block_scan_inplace(cstart + 1, ncell, sh);
   for (int i = t; i < n; i += T_) {
-    int p = atomicAdd(&cfill[ckey[i]], 1);
-    corder[p] = i;
+    const uint32_t c = ckey[i];
+    tmp[cstart[(int)(c >> 16) * nc + (int)(c & 0xffffu)] + corder[i]] = i;
   }
   __syncthreads();
-  // stable order: sort every cell's members by index, then their coordinates in that order
-  for (int c = t; c < ncell; c += T_) {
-    int lo = cstart[c], hi = cstart[c + 1];
-    for (int a = lo + 1; a < hi; ++a) {
-      int v = corder[a], b = a - 1;
-      while (b >= lo && corder[b] > v) { corder[b + 1] = corder[b]; --b; }
-      corder[b + 1] = v;
-    }
-    for (int a = lo; a < hi; ++a) {
-      const v2<T> v = x[corder[a]];
-      xs[a] = make_float2((float)v.x, (float)v.y);
-    }
+  for (int p = t; p < n; p += T_) {
+    const int i = tmp[p];
+    const uint32_t c = ckey[i];
+    const int key = (int)(c >> 16) * nc + (int)(c & 0xffffu);
+    const int lo = cstart[key], hi = cstart[key + 1];
+    int r = lo;
+    for (int q = lo; q < hi; ++q) r += tmp[q] < i;
+    const v2<T> v = x[i];
+    corder[r] = i;
+    xs[r] = make_float2((float)v.x, (float)v.y);
   }
   __syncthreads();
 }
@@ -339,7 +346,7 @@ __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const Cel
   int32_t *cstart = cells;
   float2 *const xs = (float2 *)xs_;
   if (t == 0 && hash) *hash = 0ull;
-  cta_cell_sort<T>(x, n, G, ckey, corder, cells, xs, sh);
+  cta_cell_sort<T>(x, n, G, ckey, corder, cells, xs, rp, sh);  // rp is free until the count
   if (t == 0) rp[0] = 0;
   __syncthreads();
   SortedNear<T> near(x, corder, xs, lc2);
@@ -347,8 +354,8 @@ __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const Cel
   for (int q0 = t; q0 < n; q0 += T_) {
     const int i = corder[q0];
     near.set(q0);
-    const uint32_t key = ckey[i];
-    const int cx = (int)(key % (uint32_t)nc), cy = (int)(key / (uint32_t)nc);
+    const uint32_t cell = ckey[i];
+    const int cx = (int)(cell & 0xffffu), cy = (int)(cell >> 16);
     const int bx0 = max(cx - 1, 0), bx1 = min(cx + 1, nc - 1);
     int cntn = 0;
     for (int by = max(cy - 1, 0); by <= min(cy + 1, nc - 1); ++by) {
@@ -365,8 +372,8 @@ __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const Cel
     for (int q0 = t; q0 < n; q0 += T_) {
       const int i = corder[q0];
       near.set(q0);
-      const uint32_t key = ckey[i];
-      const int cx = (int)(key % (uint32_t)nc), cy = (int)(key / (uint32_t)nc);
+      const uint32_t cell = ckey[i];
+      const int cx = (int)(cell & 0xffffu), cy = (int)(cell >> 16);
       const int bx0 = max(cx - 1, 0), bx1 = min(cx + 1, nc - 1);
       int w = rp[i];
       for (int by = max(cy - 1, 0); by <= min(cy + 1, nc - 1); ++by) {
