@@ -52,6 +52,8 @@ struct pecc_ctx {
   int block = 0, bps = 0, grid = 0;
   LargeTiles lt{};   // tiles of the instances past kCellsBlockN circles (standalone kernels)
   int n_small = -1;  // the largest instance that is not one of them
+  int eg_small[3] = {-1, -1, -1};  // energy + gradient kernels by arithmetic (energy_grad_split)
+  bool eg_large[3] = {false, false, false};
   // per arithmetic (0 FP64, 1 FP32, 2 polish) and 3 = FP32 descent + polish fused in one kernel
   struct Launch { int block = 0, bps = 0, grid = 0, var = 0; size_t smem = 0; } lc[4];
   bool lc_ready = false;
@@ -170,6 +172,7 @@ void pecc_config_default(pecc_config *c) {
   c->list_outer = 0.5;
 }
 
+static void energy_grad_split(pecc_ctx *ctx);
 static int default_k(int n) { return n < 300 ? 1 : (n < 500 ? 3 : 5); }
 
 pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
@@ -327,6 +330,7 @@ pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
     ctx->gb.kmax = kmax;
     ALC(ctx->gctl, GridCtl, 1);
   }
+  energy_grad_split(ctx);
   // tiles of the instances the standalone kernels give several blocks
   std::vector<int2> row_tiles, cell_tiles;
   for (int q = 0; q < ctx->num; ++q) {
@@ -532,23 +536,22 @@ pecc_status pecc_export_cells(pecc_ctx *ctx, uint32_t *key_dev, int32_t *order_d
   return PECC_OK;
 }
 
-// Which energy + gradient kernels a call needs: the largest instance the block kernel stages, and
-// whether any instance is too large for it.
-static void energy_grad_split(const pecc_ctx *ctx, int eval, int *max_small_n, bool *any_large) {
-  const int lim = energy_stage_n(eval);
-  *max_small_n = -1;  // no instance for the block kernel
-  *any_large = false;
-  for (int q = 0; q < ctx->num; ++q) {
-    if (ctx->n[q] <= lim) *max_small_n = std::max(*max_small_n, ctx->n[q]);
-    else *any_large = true;
+// Which energy + gradient kernels a call needs, per arithmetic: the largest instance the block kernel
+// stages, and whether any instance is too large for it (the instances are fixed: found at create).
+static void energy_grad_split(pecc_ctx *ctx) {
+  for (int eval = 0; eval < 3; ++eval) {
+    const int lim = energy_stage_n(eval);
+    ctx->eg_small[eval] = -1;  // no instance for the block kernel
+    ctx->eg_large[eval] = false;
+    for (int q = 0; q < ctx->num; ++q) {
+      if (ctx->n[q] <= lim) ctx->eg_small[eval] = std::max(ctx->eg_small[eval], ctx->n[q]);
+      else ctx->eg_large[eval] = true;
+    }
   }
 }
 
 static cudaError_t energy_grad_launch(pecc_ctx *ctx, const StandaloneParams &sp, int eval, double *E, void *grad) {
-  int ms = 0;
-  bool big = false;
-  energy_grad_split(ctx, eval, &ms, &big);
-  return launch_energy_grad(sp, eval, E, grad, ctx->ecirc, ms, big, ctx->stream);
+  return launch_energy_grad(sp, eval, E, grad, ctx->ecirc, ctx->eg_small[eval], ctx->eg_large[eval], ctx->stream);
 }
 
 pecc_status pecc_energy_grad_ex(pecc_ctx *ctx, int32_t eval, double *E_dev, void *grad_dev) {

@@ -213,6 +213,12 @@ cudaError_t launch_frame_record(const SedParams &p, const double *Rn, const doub
                                 double2 *xbest, cudaStream_t s);
 int adjust_max_m();
 
+// Dynamic shared memory past 48 KB has to be asked for; below, the call is only host time.
+inline cudaError_t allow_smem(const void *kernel, size_t bytes) {
+  return bytes <= 48 * 1024 ? cudaSuccess
+                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // Largest instance whose coordinates the block energy + gradient kernel stages in shared memory.
 inline int energy_stage_n(int eval) { return (int)(PECC_ENERGY_STAGE_BYTES / (eval == 1 ? 8 : 16)); }
 

@@ -296,8 +296,9 @@ __global__ void __launch_bounds__(kTileRows) large_go_kernel(StandaloneParams P,
   const int ncell = D.ncx * D.ncx, last = (n - 1) / kTileRows;
   const int c1 = t.y == last ? ncell + 1 : min(ncell + 1, (t.y + 1) * 4 * kTileRows);
   for (int c = t.y * 4 * kTileRows + threadIdx.x; c < c1; c += kTileRows) cells[c] = 0;
-  int go = force;
-  if (!go) {
+  if (force) {
+    if (threadIdx.x == 0 && t.y == 0) L.go[t.x] = 1;
+  } else {
     using PP = v2<T>;
     double m = 0.0;
     if (i < n) {
@@ -305,9 +306,9 @@ __global__ void __launch_bounds__(kTileRows) large_go_kernel(StandaloneParams P,
       const double dx = (double)a.x - (double)b.x, dy = (double)a.y - (double)b.y;
       m = dx * dx + dy * dy;
     }
-    go = __syncthreads_or(m > P.rebuild_disp * P.rebuild_disp);
+    const int go = __syncthreads_or(m > P.rebuild_disp * P.rebuild_disp);
+    if (threadIdx.x == 0 && go) atomicOr(&L.go[t.x], 1);  // cleared before this launch
   }
-  if (threadIdx.x == 0 && go) atomicOr(&L.go[t.x], 1);  // cleared before this launch
 }
 
 // cells of every circle and its arrival rank in its cell; for the list build also the reference
@@ -414,11 +415,14 @@ __global__ void __launch_bounds__(kTileRows) large_order_kernel(StandaloneParams
 
 // FILL = false: the entries of every tile of rows; true: the rows.
 template <typename T, bool FILL>
-__global__ void __launch_bounds__(kTileRows) large_rows_kernel(StandaloneParams P, LargeTiles L, LargeDest O) {
+__global__ void __launch_bounds__(kTileRows) large_rows_kernel(StandaloneParams P, LargeTiles L, LargeDest O,
+                                                               int32_t *rebuilt) {
   __shared__ int32_t sh[40];
   __shared__ int32_t bufs[FILL ? kTileRows * kRowHits : 1];
   const int2 t = L.rows[blockIdx.x];
-  if (!L.go[t.x]) return;
+  const int go = L.go[t.x];
+  if (FILL && rebuilt && t.y == 0 && threadIdx.x == 0) rebuilt[t.x] = go;
+  if (!go) return;
   const InstDesc &D = P.desc[t.x];
   const int n = D.n, i = t.y * kTileRows + threadIdx.x, lane = threadIdx.x & 31, nc = D.ncx;
   const Coords<T> X = coords_of<T>(P, D.off, 0);
@@ -451,19 +455,12 @@ __global__ void __launch_bounds__(kTileRows) large_rows_kernel(StandaloneParams 
   write_rows<T, int32_t>(X, act, i, key, nc, start, xs, ord, buf, cnt, row0, P.col + D.col_s_off, D.cap);
 }
 
-__global__ void large_rebuilt_kernel(StandaloneParams P, LargeTiles L, int32_t *rebuilt) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= L.nrows) return;
-  const int2 t = L.rows[b];
-  if (t.y == 0) rebuilt[t.x] = L.go[t.x];
-}
-
 // Cells, order and sorted coordinates of every large instance (flags in L.go, or all of them).
 template <typename T, bool CHECK>
 cudaError_t large_cells(const StandaloneParams &p, const LargeTiles &L, const LargeDest &O, int from32, int force,
                         v2<T> *xbuild, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(L.go, 0, sizeof(int32_t) * (size_t)p.num, s);
-  if (e != cudaSuccess) return e;
+  if (!force)
+    if (cudaError_t e = cudaMemsetAsync(L.go, 0, sizeof(int32_t) * (size_t)p.num, s)) return e;
   large_go_kernel<T><<<L.nrows, kTileRows, 0, s>>>(p, L, force);
   large_key_kernel<T, CHECK><<<L.nrows, kTileRows, 0, s>>>(p, L, O, from32, xbuild);
   large_cells_kernel<<<L.ncells, 256, 0, s>>>(p, L);
@@ -942,17 +939,15 @@ static cudaError_t build_t(const StandaloneParams &p, const LargeTiles &L, int n
   if (n_small >= 0) {
     const int block = cells_threads(n_small, p.num, sms);
     const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kBuildWarpBytes, sizeof(T) == 8);
-    cudaError_t e = cudaFuncSetAttribute(build_block_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (cudaError_t e = allow_smem((const void *)build_block_kernel<T>, smem)) return e;
     build_block_kernel<T><<<p.num, block, smem, s>>>(p, force, rebuilt);
   }
   if (L.nrows > 0) {
     const LargeDest O{p.ckey, p.corder, (float2 *)p.xtmp};
     cudaError_t e = large_cells<T, false>(p, L, O, 0, force, (v2<T> *)p.xbuild, s);
     if (e != cudaSuccess) return e;
-    large_rows_kernel<T, false><<<L.nrows, kTileRows, 0, s>>>(p, L, O);
-    large_rows_kernel<T, true><<<L.nrows, kTileRows, 0, s>>>(p, L, O);
-    if (rebuilt) large_rebuilt_kernel<<<blocks_for(L.nrows, 128), 128, 0, s>>>(p, L, rebuilt);
+    large_rows_kernel<T, false><<<L.nrows, kTileRows, 0, s>>>(p, L, O, nullptr);
+    large_rows_kernel<T, true><<<L.nrows, kTileRows, 0, s>>>(p, L, O, rebuilt);
   }
   return cudaGetLastError();
 }
@@ -970,9 +965,7 @@ cudaError_t launch_large_cells32(const StandaloneParams &p, const LargeTiles &L,
 
 template <class A> static cudaError_t launch_eg_block(const StandaloneParams &p, int stage_n, size_t smem,
                                                      void *grad, double *E, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(energy_grad_block_kernel<A>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
+  if (cudaError_t e = allow_smem((const void *)energy_grad_block_kernel<A>, smem)) return e;
   energy_grad_block_kernel<A><<<p.num, kEgBlock, smem, s>>>(p, stage_n, grad, E);
   return cudaGetLastError();
 }
@@ -1007,8 +1000,7 @@ cudaError_t launch_feasible(const StandaloneParams &p, const LargeTiles &L, int 
   if (p.num <= 0) return cudaSuccess;
   if (n_small >= 0) {
     const size_t smem = cells_smem(n_small, 0, true);
-    cudaError_t e = cudaFuncSetAttribute(feasible_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (cudaError_t e = allow_smem((const void *)feasible_block_kernel, smem)) return e;
     feasible_block_kernel<<<p.num, cells_threads(n_small, p.num, sms), smem, s>>>(p, from32, tol, feasible, max_overlap);
   }
   if (L.nrows > 0) {

@@ -814,8 +814,7 @@ cudaError_t mlp_features(const StandaloneParams &p, const LargeTiles &L, int n_s
   if (n_small >= 0) {
     const int block = n_small <= 64 ? 64 : (n_small <= 128 ? 128 : 256);
     const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kKnnWarpBytes, false);
-    cudaError_t e = cudaFuncSetAttribute(features_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (cudaError_t e = allow_smem((const void *)features_block_kernel, smem)) return e;
     features_block_kernel<<<p.num, block, smem, s>>>(p, feat);
   }
   if (L.nrows > 0) {

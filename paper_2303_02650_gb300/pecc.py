@@ -341,7 +341,7 @@ class Context:
         return out
 
     def rebuild_neighbors(self, force=True, eval=None):
-        rebuilt = torch.zeros(self.num, dtype=torch.int32, device=self.dev)
+        rebuilt = torch.empty(self.num, dtype=torch.int32, device=self.dev)  # written for every instance
         if eval is None:
             rc = self._L.pecc_rebuild_neighbors(self.h, int(force), _ptr(rebuilt))
         else:
