@@ -657,7 +657,8 @@ __global__ void __launch_bounds__(1024) energy_reduce_kernel(StandaloneParams P,
 // search runs in binary32; the binary64 values are formed for the pairs and circles whose binary32 ones
 // lie within the slack of the extreme.  The entries a list with cutoff l_cut > 2 would hold (it holds
 // every overlapping pair) are counted: past twice the capacity the instance is not checkable.
-// The 4096-instance batch: 150 us, against 2212 us for a binary64 list build and a walk over it, which
+// The 4096-instance batch: 150 us (447 us on its finished layouts, where every contact is near the extreme),
+// against 2212 us (2084) for a binary64 list build and a walk over it, which
 // the two binary64 lanes of an SM bound.  40 registers let six 256-thread blocks share an SM (170 us with
 // 64 registers and four).
 __device__ __forceinline__ double dist2_exact(double2 a, double2 b) {
@@ -757,7 +758,8 @@ __global__ void __launch_bounds__(512, 3) feasible_block_kernel(StandaloneParams
     tot += h_n[u];
   }
   bad |= tot > 2ll * D.cap;
-  double s2 = (double)inf, r2 = 0.0;
+  unsigned long long sb = 0x7ff0000000000000ull;  // squared distances compare as integers
+  double r2 = 0.0;
   if (!bad) {
     float s_hi, r_lo;
     exact_bounds(smin, rmax, &s_hi, &r_lo);
@@ -766,12 +768,16 @@ __global__ void __launch_bounds__(512, 3) feasible_block_kernel(StandaloneParams
       const float2 a = C.xs[p];
       const int i = C.ord[p];
       if (!(a.x * a.x + a.y * a.y < r_lo)) r2 = fmax(r2, norm2_exact(X.at(i)));
-      if (pairs)
+      if (pairs) {  // each pair once; in a finished layout every contact lies within the slack
+        const double2 xi = X.at(i);
         for_candidates(p, (int)C.key[i], nc, C.start, C.xs, C.ord, [&](int qq, float s) {
-          if (!(s > s_hi)) s2 = fmin(s2, dist2_exact(X.at(i), X.at(C.ord[qq])));
+          if (qq > p && !(s > s_hi))
+            sb = min(sb, (unsigned long long)__double_as_longlong(dist2_exact(xi, X.at(C.ord[qq]))));
         });
+      }
     }
   }
+  double s2 = __longlong_as_double((long long)sb);
   s2 = -warp_max(-s2);
   r2 = warp_max(r2);
   if (lane == 0) { d_s[w] = s2; d_r[w] = r2; }
@@ -821,10 +827,12 @@ __global__ void __launch_bounds__(kTileRows) large_check_kernel(StandaloneParams
     const float2 a = xs[p];
     if (!(a.x * a.x + a.y * a.y < r_lo))
       atomicMax(&L.rmax[t.x], (unsigned long long)__double_as_longlong(norm2_exact(X.at(i))));
+    unsigned long long sb = 0x7ff0000000000000ull;  // squared distances compare as integers
     for_candidates(p, (int)O.ckey[D.off + i], nc, start, xs, ord, [&](int q, float s) {
-      if (!(s > s_hi))
-        atomicMin(&L.smin[t.x], (unsigned long long)__double_as_longlong(dist2_exact(X.at(i), X.at(ord[q]))));
+      if (q > p && !(s > s_hi))  // each pair once; in a finished layout every contact lies within the slack
+        sb = min(sb, (unsigned long long)__double_as_longlong(dist2_exact(X.at(i), X.at(ord[q]))));
     });
+    if (sb < 0x7ff0000000000000ull) atomicMin(&L.smin[t.x], sb);
   }
 }
 __global__ void large_check_init_kernel(StandaloneParams P, LargeTiles L) {
