@@ -107,7 +107,8 @@ typedef struct {
     double nbr_capacity;    /* neighbor entries reserved per circle; 16 */
     int64_t time_budget_ns; /* per pecc_descend call, measured on the device; 0 = none */
     int32_t block_threads;  /* threads per instance block; 0 = about two circles per thread
-                               (at most 256 when instances outnumber SMs), or pecc_autotune's */
+                               (at most 256 when instances outnumber SMs; 128 for binary64
+                               instances of at most 64 circles that do not), or pecc_autotune's */
     int32_t blocks_per_sm;  /* target of resident instance blocks per SM, which also caps each
                                block's shared-memory share of the working set; 0 = 2 when
                                instances outnumber SMs, else 1, or pecc_autotune's */

@@ -125,8 +125,6 @@ static StandaloneParams sparams(pecc_ctx *c) {
   p.ckey = c->ckey_s;
   p.corder = c->corder_s;
   p.cells = c->cells;
-  p.rp_t = c->rp;
-  p.col_t = c->col;
   p.ckey_t = c->ckey;
   p.corder_t = c->corder;
   p.xtmp = c->xw;

@@ -253,8 +253,7 @@ struct StandaloneParams {
   int32_t *rp, *col;          // the standalone lists (one buffer per instance)
   uint32_t *ckey;
   int32_t *corder, *cells;
-  int32_t *rp_t, *col_t;      // scratch lists of the feasibility check (the descent's buffers)
-  uint32_t *ckey_t;
+  uint32_t *ckey_t;           // scratch cells of the feasibility check and the features (the descent's buffers)
   int32_t *corder_t;
   void *xtmp;                 // per-circle double2 scratch
   void *xtmp2;                // another per-circle double2 scratch
