@@ -496,8 +496,9 @@ pecc_status pecc_neighbor_count(pecc_ctx *ctx, int64_t *nnz_host) {
   CK(cudaStreamSynchronize(ctx->stream));
   int64_t t = 0;
   for (int q = 0; q < ctx->num; ++q) {
-    if (v[q] > ctx->desc_h[q].cap) return fail(ctx, PECC_ERR_NBR_OVERFLOW, "instance %d: %lld entries over capacity %d",
-                                              q, (long long)v[q], ctx->desc_h[q].cap);
+    if (v[q] > ctx->desc_h[q].cap)
+      return fail(ctx, PECC_ERR_NBR_OVERFLOW, "instance %d: %s%lld entries over capacity %d", q,
+                  v[q] >= kMaxEntries ? "at least " : "", (long long)v[q], ctx->desc_h[q].cap);
     t += v[q];
   }
   *nnz_host = t;

@@ -172,6 +172,12 @@ __device__ __forceinline__ void warp_reduce_scatter(T (&v)[NV]) {
   }
 }
 
+// Entry counts and row starts saturate here: above every list capacity (1e9 at most), and the sum of two
+// such counts still fits 32 bits.
+constexpr int32_t kMaxEntries = 0x3fffffff;
+
+__device__ __forceinline__ int32_t sat_add(int32_t a, int32_t b) { return min(a + b, kMaxEntries); }
+
 // Inclusive prefix sum of a[0..len) in place (int32), whole block; copy (may be null) receives the
 // same sums.
 __device__ inline void block_scan_inplace(int32_t *a, int len, int32_t *sh /*>=33 ints*/, int32_t *copy = nullptr) {

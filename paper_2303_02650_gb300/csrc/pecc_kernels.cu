@@ -188,13 +188,16 @@ __device__ __forceinline__ void write_rows(const Coords<T> &X, bool act, int i, 
 }
 
 // Exclusive prefix sum of one value per thread over the block; total: the block's sum.  sh: 33 ints.
+// SAT: the sums stop at kMaxEntries (entry counts of instances of any size).
+template <bool SAT = false>
 __device__ __forceinline__ int block_exclusive(int v, int32_t *sh, int &total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  auto add = [](int a, int b) { return SAT ? sat_add(a, b) : a + b; };
   int incl = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int u = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += u;
+    if (lane >= o) incl = add(incl, u);
   }
   __syncthreads();  // the previous call's reads of sh
   if (lane == 31) sh[w] = incl;
@@ -203,8 +206,12 @@ __device__ __forceinline__ int block_exclusive(int v, int32_t *sh, int &total) {
   total = 0;
   for (int u = 0; u < nw; ++u) {
     const int t = sh[u];
-    before += u < w ? t : 0;
-    total += t;
+    before = add(before, u < w ? t : 0);
+    total = add(total, t);
+  }
+  if constexpr (SAT) {  // a saturated sum cannot be taken back
+    const int prev = __shfl_up_sync(0xffffffffu, incl, 1);
+    return lane ? sat_add(before, prev) : before;
   }
   return before + incl - v;
 }
@@ -368,12 +375,12 @@ __global__ void __launch_bounds__(256) large_cells_kernel(StandaloneParams P, La
   if (threadIdx.x == 0) L.cell_total[blockIdx.x] = m > 0 ? total : 0;
 }
 
-// Sum of the totals of the earlier tiles of tile b's instance (its tile t.y of the instance).
+// Sum of the totals of the earlier tiles of tile b's instance (its tile t.y of the instance), saturated.
 __device__ __forceinline__ int tiles_before(const int32_t *total, int b, int ty, int32_t *sh) {
   int s = 0;
-  for (int u = threadIdx.x; u < ty; u += blockDim.x) s += total[b - ty + u];
+  for (int u = threadIdx.x; u < ty; u += blockDim.x) s = sat_add(s, total[b - ty + u]);
   int all;
-  block_exclusive(s, sh, all);
+  block_exclusive<true>(s, sh, all);
   return all;
 }
 
@@ -413,7 +420,9 @@ __global__ void __launch_bounds__(kTileRows) large_order_kernel(StandaloneParams
   O.xs[D.off + r] = coords_of<T>(P, D.off, from32).low(i);
 }
 
-// FILL = false: the entries of every tile of rows; true: the rows.
+// FILL = false: the entries of every tile of rows; true: the rows.  Counts and row starts saturate: 50000
+// circles in one place have 2.5e9 entries, and a start that wrapped to a negative one would pass every
+// test against the capacity.
 template <typename T, bool FILL>
 __global__ void __launch_bounds__(kTileRows) large_rows_kernel(StandaloneParams P, LargeTiles L, LargeDest O,
                                                                int32_t *rebuilt) {
@@ -442,15 +451,15 @@ __global__ void __launch_bounds__(kTileRows) large_rows_kernel(StandaloneParams 
   }
   if (!FILL) {
     int total;
-    block_exclusive(cnt, sh, total);
+    block_exclusive<true>(cnt, sh, total);
     if (threadIdx.x == 0) L.row_total[blockIdx.x] = total;
     return;
   }
   const int base = tiles_before(L.row_total, blockIdx.x, t.y, sh);
   int total;
-  const int row0 = base + block_exclusive(cnt, sh, total);
+  const int row0 = sat_add(base, block_exclusive<true>(cnt, sh, total));
   int32_t *rp = P.rp + D.off + t.x;
-  if (act) rp[i + 1] = row0 + cnt;
+  if (act) rp[i + 1] = sat_add(row0, cnt);
   if (i == 0) rp[0] = 0;
   write_rows<T, int32_t>(X, act, i, key, nc, start, xs, ord, buf, cnt, row0, P.col + D.col_s_off, D.cap);
 }
