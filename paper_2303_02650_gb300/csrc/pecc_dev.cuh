@@ -179,18 +179,20 @@ constexpr int32_t kMaxEntries = 0x3fffffff;
 __device__ __forceinline__ int32_t sat_add(int32_t a, int32_t b) { return min(a + b, kMaxEntries); }
 
 // Inclusive prefix sum of a[0..len) in place (int32), whole block; copy (may be null) receives the
-// same sums.
+// same sums.  SAT: the sums stop at kMaxEntries (entry counts of lists).
+template <bool SAT = false>
 __device__ inline void block_scan_inplace(int32_t *a, int len, int32_t *sh /*>=33 ints*/, int32_t *copy = nullptr) {
   const int T = blockDim.x, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = T >> 5;
+  auto add = [](int32_t x, int32_t y) { return SAT ? sat_add(x, y) : x + y; };
   int ch = (len + T - 1) / T;
   int lo = min(len, t * ch), hi = min(len, lo + ch);
   int32_t s = 0;
-  for (int i = lo; i < hi; ++i) s += a[i];
+  for (int i = lo; i < hi; ++i) s = add(s, a[i]);
   int32_t incl = s;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     int32_t u = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += u;
+    if (lane >= o) incl = add(incl, u);
   }
   if (lane == 31) sh[w] = incl;
   __syncthreads();
@@ -199,16 +201,22 @@ __device__ inline void block_scan_inplace(int32_t *a, int len, int32_t *sh /*>=3
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       int32_t u = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += u;
+      if (lane >= o) v = add(v, u);
     }
     if (lane < nw) sh[lane] = v;
   }
   __syncthreads();
-  int32_t run = incl - s + (w > 0 ? sh[w - 1] : 0);
+  int32_t run = w > 0 ? sh[w - 1] : 0;
+  if constexpr (SAT) {  // a saturated sum cannot be taken back
+    const int32_t prev = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (lane) run = sat_add(run, prev);
+  } else {
+    run += incl - s;
+  }
   if (copy)
-    for (int i = lo; i < hi; ++i) { run += a[i]; a[i] = run; copy[i] = run; }
+    for (int i = lo; i < hi; ++i) { run = add(run, a[i]); a[i] = run; copy[i] = run; }
   else
-    for (int i = lo; i < hi; ++i) { run += a[i]; a[i] = run; }
+    for (int i = lo; i < hi; ++i) { run = add(run, a[i]); a[i] = run; }
   __syncthreads();
 }
 

@@ -167,13 +167,14 @@ __device__ bool grid_reduce_chunks(GSmem<A> &S, const GridBufs &G, GridCtl *c, d
 }
 
 // Inclusive prefix sum of a[0..len) in place across the grid (each block one contiguous chunk);
-// the total goes to S.iv[1].  False on a barrier failure.
+// the total goes to S.iv[1].  A block's sums saturate (crowded rows of 600000 circles pass 32 bits within
+// a chunk); a total past every capacity leaves a[] unusable.  False on a barrier failure.
 template <class A>
 __device__ bool grid_scan(GSmem<A> &S, const GridBufs &G, GridCtl *c, int32_t *a, int len) {
   const int nb = gridDim.x, b = blockIdx.x;
   const int chunk = (len + nb - 1) / nb;
   const int lo = min(len, b * chunk), hi = min(len, lo + chunk);
-  block_scan_inplace(a + lo, hi - lo, S.sh);
+  block_scan_inplace<true>(a + lo, hi - lo, S.sh);
   if (threadIdx.x == 0) G.ipart[b] = (hi > lo) ? a[hi - 1] : 0;
   if (!grid_sync(S, c)) return false;
   if (threadIdx.x < 32) {  // the blocks before this one, and all of them

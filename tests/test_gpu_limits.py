@@ -27,3 +27,17 @@ def test_overflow_past_32_bit_counts(orc, prec):
     assert np.isnan(E[0]) and np.isnan(g[:50000]).all()
     assert np.isfinite(E[1]) and np.isfinite(g[50000:]).all()
     assert np.isnan(mo[0]) and mo[1] == orc.max_overlap(x, float(R[1]))[0] and feas[0] == 0
+
+
+def test_whole_gpu_overflow_past_32_bit_counts():
+    """600000 circles closer than the cutoff to one another: a block's share of the rows (3948 of them, each
+    with 599999 entries) passes 32 bits.  The descent ends with the overflow status."""
+    torch, pecc = need_gpu()
+    n = 600000
+    rng = np.random.default_rng(1)
+    r, a = 0.6 * np.sqrt(rng.uniform(size=n)), rng.uniform(0.0, 2.0 * np.pi, size=n)
+    with pecc.Context(np.array([n], dtype=np.int32), precision=1, max_iter=1) as c:
+        c.set_radius(np.array([synth.radius(n, 0.8)]))
+        c.set_positions(torch.from_numpy(np.stack([r * np.cos(a), r * np.sin(a)], 1)))
+        iters, status = c.descend()
+        assert int(status.cpu()[0]) == 4 and int(iters.cpu()[0]) == 0
