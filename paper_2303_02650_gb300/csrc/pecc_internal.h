@@ -213,10 +213,10 @@ cudaError_t launch_frame_record(const SedParams &p, const double *Rn, const doub
                                 double2 *xbest, cudaStream_t s);
 int adjust_max_m();
 
-// Dynamic shared memory past 48 KB has to be asked for; below, the call is only host time.
+// Sets the kernel's limit of dynamic shared memory.  Without it a launch gets 48 KB together with the
+// kernel's static shared memory, so no size close to that can do without.
 inline cudaError_t allow_smem(const void *kernel, size_t bytes) {
-  return bytes <= 48 * 1024 ? cudaSuccess
-                            : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // Largest instance whose coordinates the block energy + gradient kernel stages in shared memory.

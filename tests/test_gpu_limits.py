@@ -1,4 +1,9 @@
-"""Calls at the limits of what they take (marked gpu): list overflow of any length."""
+"""Calls at the limits of what they take (marked gpu): list overflow of any length, shared memory of any
+size."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -6,6 +11,8 @@ from paper_2303_02650_gb300 import synth
 from gpu_util import need_gpu
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.mark.parametrize("prec", [0, 1])
@@ -41,3 +48,48 @@ def test_whole_gpu_overflow_past_32_bit_counts():
         c.set_positions(torch.from_numpy(np.stack([r * np.cos(a), r * np.sin(a)], 1)))
         iters, status = c.descend()
         assert int(status.cpu()[0]) == 4 and int(iters.cpu()[0]) == 0
+
+
+# The first call of a process: nothing has raised a kernel's shared-memory limit before it.
+FIRST_CALL = """
+import sys
+import numpy as np, torch
+import oracle as orc
+from oracle import mlp as omlp
+from paper_2303_02650_gb300 import pecc, synth
+kind, n0, others, prec = sys.argv[1], int(sys.argv[2]), int(sys.argv[3]), int(sys.argv[4])
+orc.build()
+n = np.array([n0] + [1] * others, dtype=np.int32)
+R = np.array([synth.radius(int(v), 0.8) for v in n])
+x = synth.random_layout(n0, 0.9 * float(R[0]), 3).astype(np.float32).astype(np.float64)
+xy = np.concatenate([x, np.zeros((others, 2))])
+with pecc.Context(n, precision=prec) as c:
+    c.set_radius(R)
+    c.set_positions(torch.from_numpy(xy))
+    if kind == "check":
+        assert float(c.check_feasible()[1][0]) == orc.max_overlap(x, float(R[0]))[0]
+    elif kind == "features":
+        assert np.array_equal(c.features().cpu().numpy()[:n0], omlp.features(x.astype(np.float32), float(R[0])))
+    else:
+        c.rebuild_neighbors(force=True)
+        if kind == "lists":
+            rp, col = [t.cpu().numpy() for t in c.export_neighbors()]
+            rref, cref = orc.neighbors_brute(x, 2.5, prec32=(prec == 1))
+            assert np.array_equal(rp[:n0 + 1], rref) and np.array_equal(col[:rp[n0]], cref)
+        else:
+            E, g = c.energy_grad()
+            torch.cuda.synchronize()
+            assert np.isfinite(E.cpu().numpy()).all() and bool(torch.isfinite(g).all())
+print("first call ok")
+"""
+
+
+@pytest.mark.parametrize("kind,n,others,prec", [
+    ("check", 1790, 0, 0), ("check", 1790, 0, 2), ("lists", 1706, 0, 1), ("lists", 1200, 0, 0), ("lists", 1503, 200, 0),
+    ("features", 1218, 0, 1), ("energy", 6136, 0, 1), ("energy", 3064, 0, 0)])
+def test_first_call_of_a_process(orc, kind, n, others, prec):
+    """Sizes whose dynamic shared memory is just below 48 KB, and above it with the kernel's own."""
+    need_gpu()
+    r = subprocess.run([sys.executable, "-c", FIRST_CALL, kind, str(n), str(others), str(prec)], cwd=ROOT,
+                       env=dict(os.environ, PYTHONPATH=ROOT), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "first call ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
