@@ -227,6 +227,8 @@ pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
   };
   if (cudaGetDevice(&ctx->device) != cudaSuccess) return bail(fail(ctx, PECC_ERR_CUDA, "no CUDA device"));
   cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  if (standalone_smem_limits() != cudaSuccess || (cfg->precision != PECC_FP64 && features_smem_limit() != cudaSuccess))
+    return bail(fail(ctx, PECC_ERR_CUDA, "shared-memory limits"));
 
   const int m1 = cfg->lbfgs_m + 1;
   const bool fp64 = cfg->precision == PECC_FP64;
@@ -631,7 +633,7 @@ static pecc_status plan_launch(pecc_ctx *ctx, int arith, int block = 0, int bps_
     if (ctx->cfg.smem_per_block > 0) cap = std::min(cap, (size_t)ctx->cfg.smem_per_block);
     const size_t smem = std::max(mand, std::min(need, cap) & ~size_t(255));
     if (smem + stat > (size_t)optin) continue;
-    CK(cudaFuncSetAttribute(vs[v].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CK(raise_smem_limit(vs[v].fn));
     int occ = 0;
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, vs[v].fn, blk, smem));
     if (occ < 1) continue;
@@ -640,7 +642,6 @@ static pecc_status plan_launch(pecc_ctx *ctx, int arith, int block = 0, int bps_
   }
   if (best < 0)
     return fail(ctx, PECC_ERR_ARG, "descent kernel does not fit an SM (block %d, %zu bytes of shared memory needed)", blk, mand);
-  CK(cudaFuncSetAttribute(vs[best].fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)best_smem));
   L.var = best;
   L.smem = best_smem;
   L.bps = fixed ? std::min(bps_target, best_occ) : best_occ;

@@ -213,11 +213,13 @@ cudaError_t launch_frame_record(const SedParams &p, const double *Rn, const doub
                                 double2 *xbest, cudaStream_t s);
 int adjust_max_m();
 
-// Sets the kernel's limit of dynamic shared memory.  Without it a launch gets 48 KB together with the
-// kernel's static shared memory, so no size close to that can do without.
-inline cudaError_t allow_smem(const void *kernel, size_t bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
+// Raises a kernel's limit of dynamic shared memory to the most a block can have on the current device.  The
+// limit is the kernel's, for the whole process: set to one launch's size it could be lowered by another
+// thread's between that and the launch, so every setting is this same one, made when a context is created
+// (the standalone kernels) or plans its descent.  A launch takes what it asks for, whatever the limit.
+cudaError_t raise_smem_limit(const void *kernel);
+cudaError_t standalone_smem_limits();
+cudaError_t features_smem_limit();
 
 // Largest instance whose coordinates the block energy + gradient kernel stages in shared memory.
 inline int energy_stage_n(int eval) { return (int)(PECC_ENERGY_STAGE_BYTES / (eval == 1 ? 8 : 16)); }

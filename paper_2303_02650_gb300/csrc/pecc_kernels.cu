@@ -923,6 +923,24 @@ __global__ void stats_kernel(const InstOut *out, int num, int32_t *st) {
 
 }  // namespace
 
+cudaError_t raise_smem_limit(const void *kernel) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes a;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+}
+
+cudaError_t standalone_smem_limits() {
+  for (const void *k : {(const void *)build_block_kernel<float>, (const void *)build_block_kernel<double>,
+                        (const void *)feasible_block_kernel, (const void *)energy_grad_block_kernel<Arith64>,
+                        (const void *)energy_grad_block_kernel<Arith32>, (const void *)energy_grad_block_kernel<ArithMix>})
+    if (cudaError_t e = raise_smem_limit(k)) return e;
+  return cudaSuccess;
+}
+
 cudaError_t launch_init(const StandaloneParams &p, uint64_t seed, int mode, int prec, cudaStream_t s) {
   if (p.total > 0) init_kernel<<<blocks_for(p.total, 256), 256, 0, s>>>(p, seed, mode, prec);
   return cudaGetLastError();
@@ -956,7 +974,6 @@ static cudaError_t build_t(const StandaloneParams &p, const LargeTiles &L, int n
   if (n_small >= 0) {
     const int block = cells_threads(n_small, p.num, sms);
     const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kBuildWarpBytes, sizeof(T) == 8);
-    if (cudaError_t e = allow_smem((const void *)build_block_kernel<T>, smem)) return e;
     build_block_kernel<T><<<p.num, block, smem, s>>>(p, force, rebuilt);
   }
   if (L.nrows > 0) {
@@ -982,7 +999,6 @@ cudaError_t launch_large_cells32(const StandaloneParams &p, const LargeTiles &L,
 
 template <class A> static cudaError_t launch_eg_block(const StandaloneParams &p, int stage_n, size_t smem,
                                                      void *grad, double *E, cudaStream_t s) {
-  if (cudaError_t e = allow_smem((const void *)energy_grad_block_kernel<A>, smem)) return e;
   energy_grad_block_kernel<A><<<p.num, kEgBlock, smem, s>>>(p, stage_n, grad, E);
   return cudaGetLastError();
 }
@@ -1017,7 +1033,6 @@ cudaError_t launch_feasible(const StandaloneParams &p, const LargeTiles &L, int 
   if (p.num <= 0) return cudaSuccess;
   if (n_small >= 0) {
     const size_t smem = cells_smem(n_small, 0, true);
-    if (cudaError_t e = allow_smem((const void *)feasible_block_kernel, smem)) return e;
     feasible_block_kernel<<<p.num, cells_threads(n_small, p.num, sms), smem, s>>>(p, from32, tol, feasible, max_overlap);
   }
   if (L.nrows > 0) {

@@ -809,12 +809,13 @@ cudaError_t mlp_sync_bf16(const float *params, bf16 *wb, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+cudaError_t features_smem_limit() { return raise_smem_limit((const void *)features_block_kernel); }
+
 cudaError_t mlp_features(const StandaloneParams &p, const LargeTiles &L, int n_small, float *feat, cudaStream_t s) {
   if (p.num <= 0) return cudaSuccess;
   if (n_small >= 0) {
     const int block = n_small <= 64 ? 64 : (n_small <= 128 ? 128 : 256);
     const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kKnnWarpBytes, false);
-    if (cudaError_t e = allow_smem((const void *)features_block_kernel, smem)) return e;
     features_block_kernel<<<p.num, block, smem, s>>>(p, feat);
   }
   if (L.nrows > 0) {

@@ -1,8 +1,9 @@
 """Calls at the limits of what they take (marked gpu): list overflow of any length, shared memory of any
-size."""
+size, contexts of several host threads."""
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -93,3 +94,47 @@ def test_first_call_of_a_process(orc, kind, n, others, prec):
     r = subprocess.run([sys.executable, "-c", FIRST_CALL, kind, str(n), str(others), str(prec)], cwd=ROOT,
                        env=dict(os.environ, PYTHONPATH=ROOT), capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "first call ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
+
+
+def test_contexts_of_two_host_threads():
+    """Two threads whose contexts need different amounts of shared memory, each on its own stream, launching
+    without pause: every call of both succeeds with the results it has alone."""
+    torch, pecc = need_gpu()
+    sizes, rounds = [1900, 2048], 1500
+    errors, got = [], {}
+
+    def work(n0, gate=None, out=got):
+        try:
+            s = torch.cuda.Stream()
+            R = np.array([synth.radius(n0, 0.8)])
+            x = torch.from_numpy(synth.random_layout(n0, 0.9 * float(R[0]), 3))
+            with torch.cuda.stream(s), pecc.Context(np.array([n0], dtype=np.int32), precision=1, stream=s) as c:
+                m = pecc.MLP(7, stream=s)
+                c.set_radius(R)
+                c.set_positions(x)
+                s.synchronize()
+                if gate:
+                    gate.wait()
+                c.warm_start(m, rounds)  # list builds, energies and features, enqueued by one call
+                mo = c.check_feasible()[1]
+                xy = c.get_positions()
+                s.synchronize()
+                out[n0] = np.concatenate([xy.cpu().numpy().ravel(), mo.cpu().numpy()])
+                m.close()
+        except Exception as e:  # noqa: BLE001 -- reported by the test's own thread
+            errors.append((n0, repr(e)))
+            if gate:
+                gate.abort()
+
+    alone = {}
+    for v in sizes:
+        work(v, out=alone)
+    gate = threading.Barrier(len(sizes))
+    threads = [threading.Thread(target=work, args=(v, gate)) for v in sizes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for v in sizes:
+        assert np.array_equal(got[v], alone[v])
