@@ -437,6 +437,17 @@ pecc_status pecc_adjust_container(pecc_ctx *ctx, double *R_dev, double lambda0, 
  * the launch or a copy failed. */
 pecc_status pecc_selftest_grid_barrier(int64_t timeout_ns, int32_t *failed_host, int64_t *waited_ns_host);
 
+/* Self-test of the bounded wait of the network's kernels for their tensor-core instructions.  One warp
+ * waits for a barrier that a second one opens after open_after_ns; the lanes in short_lanes give up at
+ * once, the others a second after that time.  A warp has one answer: all lanes yes when no lane gave up,
+ * else none.  Runs on the current device and the legacy default stream; synchronises.
+ *   open_after_ns   > 0, at most 1 s
+ *   short_lanes     bit mask of the lanes that give up
+ *   yes_host        host int32[1]: how many lanes answered yes
+ * Returns PECC_ERR_ARG for a bad argument, PECC_ERR_CUDA (message in pecc_last_error(NULL)) if
+ * the launch or a copy failed. */
+pecc_status pecc_selftest_mma_wait(int64_t open_after_ns, uint32_t short_lanes, int32_t *yes_host);
+
 /* Text of the last error on this context (or of the last failed pecc_create when ctx is NULL). */
 const char *pecc_last_error(pecc_ctx *ctx);
 

@@ -430,6 +430,16 @@ pecc_status pecc_selftest_grid_barrier(int64_t timeout_ns, int32_t *failed_host,
   return PECC_OK;
 }
 
+pecc_status pecc_selftest_mma_wait(int64_t open_after_ns, uint32_t short_lanes, int32_t *yes_host) {
+  if (!yes_host || open_after_ns <= 0 || open_after_ns > 1000000000ll)
+    return fail(nullptr, PECC_ERR_ARG, "pecc_selftest_mma_wait: bad argument");
+  int yes = 0;
+  cudaError_t e = selftest_mma_wait((long long)open_after_ns, short_lanes, &yes);
+  if (e != cudaSuccess) return fail(nullptr, PECC_ERR_CUDA, "pecc_selftest_mma_wait: %s", cudaGetErrorString(e));
+  *yes_host = yes;
+  return PECC_OK;
+}
+
 const char *pecc_last_error(pecc_ctx *ctx) { return ctx ? ctx->err.c_str() : g_create_err.c_str(); }
 
 pecc_status pecc_set_radius(pecc_ctx *ctx, const double *R_dev) {

@@ -288,6 +288,7 @@ cudaError_t launch_outputs(const InstOut *out, int num, int32_t *iters, int32_t 
                            int32_t *builds, int32_t *changes, int32_t *trials, cudaStream_t s);
 
 // Learned warm start (pecc_mlp.cu).
+cudaError_t selftest_mma_wait(long long open_after_ns, uint32_t short_lanes, int *yes_host);
 int mlp_num_params();
 int mlp_num_bf16();
 int mlp_train_blocks(int sms);

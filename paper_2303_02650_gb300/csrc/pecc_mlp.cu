@@ -300,12 +300,12 @@ __device__ __forceinline__ bool tc_sync(bool ok = true, int g = -1) {
   return !any;
 }
 
-// Every thread waits for the barrier's current phase itself (a wait that runs out is reported to the
-// group at its next barrier, so that all of them leave together).
+// Every warp waits for the barrier's current phase itself (a wait that runs out is reported to the
+// group at its next barrier, so that all of them leave together).  The answer is the warp's: a lane that
+// left out the next wait or a TMEM load, both warp-wide, would leave the others standing there.
 __device__ __forceinline__ bool tc_wait(uint64_t *mbar, uint32_t &phase) {
-  const bool ok = tc::mbar_wait(mbar, phase, kWaitNs);
+  const bool ok = tc::mbar_wait_warp(mbar, phase, kWaitNs);
   phase ^= 1u;
-  __syncwarp();  // the TMEM loads that follow are warp-wide instructions
   tc::fence_after();
   return ok;
 }
@@ -792,6 +792,36 @@ __global__ void revert_kernel(StandaloneParams P, const float2 *__restrict__ bac
 inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
+
+// Self-test of that wait: a warp waits for a barrier that another opens after open_after_ns; the lanes of
+// short_lanes give up at once, the others a second later than that.  *yes: the lanes whose answer was yes.
+__global__ void wait_selftest_kernel(long long open_after_ns, uint32_t short_lanes, int *yes) {
+  __shared__ uint64_t mbar;
+  if (threadIdx.x == 0) tc::mbar_init(&mbar);
+  __syncthreads();
+  if (threadIdx.x == 32) {
+    const long long t0 = tc::now_ns();
+    while (tc::now_ns() - t0 < open_after_ns) __nanosleep(1000);
+    tc::mbar_arrive(&mbar);
+  }
+  if (threadIdx.x >= 32) return;
+  const bool give_up = (short_lanes >> threadIdx.x) & 1u;
+  const bool ok = tc::mbar_wait_warp(&mbar, 0, give_up ? 0 : open_after_ns + 1000000000ll);
+  atomicAdd(yes, ok ? 1 : 0);
+}
+
+cudaError_t selftest_mma_wait(long long open_after_ns, uint32_t short_lanes, int *yes_host) {
+  int *yes = nullptr;
+  cudaError_t e = cudaMalloc(&yes, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(yes, 0, sizeof(int));
+  if (e == cudaSuccess) {
+    wait_selftest_kernel<<<1, 64>>>(open_after_ns, short_lanes, yes);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpy(yes_host, yes, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaFree(yes);
+  return e;
+}
 
 int mlp_num_params() { return NPAR; }
 int mlp_num_bf16() { return NBW; }

@@ -78,6 +78,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, long 
   }
 }
 
+// The same by a whole warp, with one answer for all its lanes: true if every lane's wait ended in time.  Each
+// lane reads the clock for itself, so lanes can disagree about a wait that runs out; warp-wide instructions
+// (TMEM loads, the next wait) must not follow in only some of them.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *mbar, uint32_t parity, long long limit_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(mbar, parity, limit_ns));
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+  asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(smem_u32(mbar)) : "memory");
+}
+
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // generic-proxy shared-memory writes become visible to the tensor cores' reads

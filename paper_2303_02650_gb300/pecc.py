@@ -55,6 +55,7 @@ _EXPORTS = ["pecc_config_default", "pecc_create", "pecc_destroy", "pecc_set_radi
             "pecc_check_feasible_noalloc", "pecc_mlp_num_params", "pecc_mlp_create", "pecc_mlp_destroy",
             "pecc_mlp_get_params", "pecc_mlp_set_params", "pecc_mlp_forward", "pecc_mlp_grad", "pecc_mlp_train_step",
             "pecc_features", "pecc_targets", "pecc_warm_start", "pecc_autotune", "pecc_selftest_grid_barrier",
+            "pecc_selftest_mma_wait",
             "pecc_adjust_container", "pecc_sed_config_default", "pecc_sed_create", "pecc_sed_destroy",
             "pecc_sed_last_error", "pecc_sed_set_radius", "pecc_sed_start", "pecc_sed_set_state", "pecc_sed_iterate",
             "pecc_sed_prepare", "pecc_sed_descend", "pecc_sed_select", "pecc_sed_get", "pecc_sed_context",
@@ -107,6 +108,7 @@ def load(build_if_missing: bool = True):
         "pecc_phase_times": (st, [vp, C.POINTER(C.c_float)]),
         "pecc_check_feasible_noalloc": (st, [vp, C.c_int32, C.c_double, C.c_double, C.c_double, vp, vp, vp]),
         "pecc_selftest_grid_barrier": (st, [C.c_int64, C.POINTER(C.c_int32), C.POINTER(C.c_int64)]),
+        "pecc_selftest_mma_wait": (st, [C.c_int64, C.c_uint32, C.POINTER(C.c_int32)]),
         "pecc_adjust_container": (st, [vp, vp, C.c_double, C.c_int32, vp, vp, vp]),
         "pecc_mlp_num_params": (C.c_int32, []),
         "pecc_mlp_create": (st, [C.c_uint64, vp, C.POINTER(vp)]),
@@ -172,6 +174,16 @@ def selftest_grid_barrier(timeout_ns=50_000_000):
     if rc != 0:
         raise PeccError(f"pecc_selftest_grid_barrier: {ERRORS.get(rc, rc)}: {L.pecc_last_error(None).decode()}")
     return f.value, w.value
+
+
+def selftest_mma_wait(open_after_ns, short_lanes):
+    """pecc_selftest_mma_wait: how many of a warp's lanes answered that the wait ended in time."""
+    L = load()
+    yes = C.c_int32()
+    rc = L.pecc_selftest_mma_wait(int(open_after_ns), int(short_lanes), C.byref(yes))
+    if rc != 0:
+        raise PeccError(f"pecc_selftest_mma_wait: {ERRORS.get(rc, rc)}: {L.pecc_last_error(None).decode()}")
+    return yes.value
 
 
 def check_feasible_noalloc(xy, R, l_cut=2.5, tol=1e-9, stream=None):

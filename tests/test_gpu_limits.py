@@ -1,5 +1,5 @@
 """Calls at the limits of what they take (marked gpu): list overflow of any length, shared memory of any
-size, contexts of several host threads."""
+size, contexts of several host threads, waits that run out."""
 import os
 import subprocess
 import sys
@@ -138,3 +138,11 @@ def test_contexts_of_two_host_threads():
     assert not errors, errors
     for v in sizes:
         assert np.array_equal(got[v], alone[v])
+
+
+@pytest.mark.parametrize("short_lanes,yes", [(0, 32), (1, 0), (0x80000000, 0), (0x55555555, 0), (0xFFFFFFFF, 0)])
+def test_a_warp_has_one_answer_to_a_wait(short_lanes, yes):
+    """A wait for the tensor cores that runs out in some lanes of a warp and not in others: all of them
+    hear that it ran out (warp-wide instructions follow)."""
+    torch, pecc = need_gpu()
+    assert pecc.selftest_mma_wait(200_000_000, short_lanes) == yes
