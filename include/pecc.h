@@ -168,8 +168,9 @@ pecc_status pecc_destroy(pecc_ctx *ctx);
  * on the device (the cell tables were allocated at pecc_create for the largest grid an instance
  * can get, max(16, ceil(2 sqrt(n))) cells per side), so R_dev must stay valid until the stream
  * has run the call.  A radius that is not finite and > 0 is not an argument error (it is not read
- * on the host): its instance gets R = NaN, and its energies, descents (status
- * PECC_DESC_NONFINITE) and feasibility checks (max_overlap NaN) say so. */
+ * on the host): its instance gets R = NaN, and its energies and gradients (NaN), descents (status
+ * PECC_DESC_NONFINITE) and feasibility checks (max_overlap NaN, feasible 0) say so.  An instance of 0
+ * circles has nothing to report whatever its radius. */
 pecc_status pecc_set_radius(pecc_ctx *ctx, const double *R_dev);
 
 /* Coordinates: xy_dev = device double[2 * sum n].  FP32 contexts round them to binary32. */
@@ -216,8 +217,8 @@ pecc_status pecc_export_cells(pecc_ctx *ctx, uint32_t *key_dev, int32_t *order_d
  * instances up to PECC_ENERGY_STAGE_BYTES of coordinates); larger instances take one thread
  * per circle and a per-instance reduction.
  * The gradient is gathered (no atomics) and E is summed in a fixed order (deterministic).
- * An instance whose last build overflowed its list capacity (nbr_capacity) gets E = NaN and
- * a NaN gradient. */
+ * An instance whose last build overflowed its list capacity (nbr_capacity), or whose radius was not
+ * accepted (pecc_set_radius), gets E = NaN and a NaN gradient. */
 pecc_status pecc_energy_grad(pecc_ctx *ctx, double *E_dev, void *grad_dev);
 
 /* Same, with an explicit arithmetic: eval = PECC_FP64 (double2 gradient), PECC_FP32
@@ -258,8 +259,8 @@ pecc_status pecc_get_energy(pecc_ctx *ctx, double *E_dev);
  * list with cutoff l_cut > 2 holds every overlapping pair) and largest container overlap
  * depth, in FP64 with correctly rounded operations; feasible_dev (device uint8[num]) is 1
  * where the larger of the two is <= tol, max_overlap_dev (device double[num]) receives it.
- * An instance that cannot be checked (a non-finite coordinate, or more list entries than twice
- * its capacity) gets max_overlap NaN and feasible 0. */
+ * An instance that cannot be checked (a non-finite coordinate, a radius that was not accepted, or
+ * more list entries than twice its capacity) gets max_overlap NaN and feasible 0. */
 pecc_status pecc_check_feasible(pecc_ctx *ctx, double tol, uint8_t *feasible_dev, double *max_overlap_dev);
 
 /* The whole path from host memory: copy R_host (double[num]) to the device, draw the

@@ -77,8 +77,11 @@ __global__ void __launch_bounds__(kDT, 2) dense_kernel(DenseParams P) {
     const InstDesc D = P.desc[q];
     const int n = D.n;
     InstOut *O = P.out + q;
-    if (n == 0) {
-      if (tid == 0) { O->iters = 0; O->status = 0; O->E = 0.0; O->iters32 = 0; O->trials32 = 0; }
+    if (n == 0 || !(D.R > 0.0)) {  // nothing to do, or a radius pecc_set_radius could not accept
+      if (tid == 0) {
+        O->iters = O->iters32 = 0; O->status = O->status32 = n == 0 ? 0 : 5; O->E = 0.0;
+        O->builds = O->trials = O->resets = O->stalls = O->polished = O->trials32 = 0;
+      }
       __syncthreads();
       continue;
     }

@@ -344,6 +344,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
       xb[p] = v;
     }
     clear_cells();
+    bad |= !(D.R > 0.0);  // a radius pecc_set_radius could not accept
     double vb[1] = {(double)bad};
     const int kind[1] = {1};
     ok = grid_reduce<A, 1, double>(S, G, ctl, vb, kind);

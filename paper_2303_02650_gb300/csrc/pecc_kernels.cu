@@ -508,7 +508,9 @@ __global__ void __launch_bounds__(256) energy_grad_kernel(StandaloneParams P, in
   vec_t gx = 0, gy = 0;
   acc_t e = 0;
   const int lo = __ldg(rp + i), hi = __ldg(rp + i + 1);
-  if (__ldg(rp + P.desc[q].n) > P.desc[q].cap) {  // the last build overflowed the list's capacity: no valid list
+  // the last build overflowed the list's capacity (no valid list), or the radius was rejected (NaN; tested
+  // by its bits: binary64 instructions issue slowly)
+  if (__ldg(rp + P.desc[q].n) > P.desc[q].cap || not_finite(Rd)) {
     VV gv; gv.x = gv.y = (vec_t)NAN;
     ((VV *)grad_)[gi] = gv;
     ((acc_t *)ecirc_)[gi] = (acc_t)NAN;
@@ -579,7 +581,9 @@ __global__ void __launch_bounds__(kEgBlock) energy_grad_block_kernel(StandaloneP
   // are in flight together instead of one load round trip per coordinate
   for (int i = threadIdx.x; i < n; i += blockDim.x) cp_async_shared<sizeof(PP)>(xs + i, x + i);
   asm volatile("cp.async.wait_all;\n" ::: "memory");
-  if (end > P.desc[q].cap) {  // the last build overflowed the list's capacity: no valid list
+  // the last build overflowed the list's capacity (no valid list), or the radius was rejected (NaN; tested
+  // by its bits: binary64 instructions issue slowly)
+  if (end > P.desc[q].cap || not_finite(Rd)) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) { VV gv; gv.x = gv.y = (vec_t)NAN; grad[i] = gv; }
     if (threadIdx.x == 0) E[q] = NAN;
     return;
@@ -684,7 +688,8 @@ __device__ __forceinline__ void feasible_result(const StandaloneParams &P, int q
   if (s2 < 4.0) v = fmax(v, __dsub_rn(2.0, __dsqrt_rn(s2)));
   const double d = __dsub_rn(__dadd_rn(__dsqrt_rn(r2), 1.0), R);
   v = fmax(v, d > 0.0 ? d : 0.0);
-  if (P.desc[q].n == 0) v = 0.0;
+  bad |= !(R > 0.0);  // a rejected radius (NaN here) contains nothing, however the circles lie
+  if (P.desc[q].n == 0) { v = 0.0; bad = false; }
   if (bad) v = __longlong_as_double(0x7ff8000000000000ll);  // NaN: not checkable
   const bool ok = !bad && v <= tol;
   if (feasible) feasible[q] = ok ? 1 : 0;

@@ -1,5 +1,6 @@
 """Calls at the limits of what they take (marked gpu): list overflow of any length, shared memory of any
-size, contexts of several host threads, waits that run out."""
+size, contexts of several host threads, waits that run out,
+radii that are not radii."""
 import os
 import subprocess
 import sys
@@ -146,3 +147,47 @@ def test_a_warp_has_one_answer_to_a_wait(short_lanes, yes):
     hear that it ran out (warp-wide instructions follow)."""
     torch, pecc = need_gpu()
     assert pecc.selftest_mma_wait(200_000_000, short_lanes) == yes
+
+
+def _apart(n):
+    """Layouts of circles that do not overlap: squares of side 2.5."""
+    parts = []
+    for v in n:
+        side = int(np.ceil(np.sqrt(v)))
+        g = np.stack(np.meshgrid(np.arange(side), np.arange(side)), -1).reshape(-1, 2)[:v] * 2.5
+        parts.append(g - g.mean(0) if v else g.astype(float))
+    return np.concatenate(parts).astype(np.float32).astype(np.float64)
+
+
+@pytest.mark.parametrize("bad", [-1.0, 0.0, float("nan"), float("inf")])
+def test_rejected_radius_is_reported(orc, bad):
+    """Circles that do not overlap, in containers whose radius is not finite and > 0: not checkable, no energy,
+    no descent, in the block, tile, whole-GPU and explicit-Hessian forms; the instances beside them are
+    unaffected, and one without circles has nothing to report."""
+    torch, pecc = need_gpu()
+    n = np.array([7, 7000, 30, 0, 16500], dtype=np.int32)
+    off = np.concatenate([[0], np.cumsum(n)])
+    xy = _apart(n)
+    R = np.array([bad, bad, 12.0, bad, bad])
+    for prec in (0, 1, 2):
+        with pecc.Context(n, precision=prec) as c:
+            c.set_radius(R)
+            c.set_positions(torch.from_numpy(xy))
+            feas, mo = [t.cpu().numpy() for t in c.check_feasible()]
+            c.rebuild_neighbors(force=True)
+            E, g = [t.cpu().numpy() for t in c.energy_grad()]
+            status = c.descend()[1].cpu().numpy()
+            x1 = c.get_positions().cpu().numpy()
+            assert np.array_equal(c.check_feasible()[0].cpu().numpy(), feas)
+        assert feas.tolist() == [0, 0, 1, 1, 0] and np.isnan(mo[[0, 1, 4]]).all()
+        x2 = xy[off[2]:off[3]]
+        assert mo[2] == orc.max_overlap(x2, 12.0)[0] and mo[3] == 0.0
+        for q in (0, 1, 4):
+            assert np.isnan(E[q]) and np.isnan(g[off[q]:off[q + 1]]).all() and status[q] == 5
+            assert np.array_equal(x1[off[q]:off[q + 1]], xy[off[q]:off[q + 1]])
+        assert E[2] == 0.0 and not g[off[2]:off[3]].any() and E[3] == 0.0 and status[[2, 3]].tolist() == [0, 0]
+    n = n[:4]
+    with pecc.Context(n, precision=0, qn_dense=1) as c:
+        c.set_radius(R[:4])
+        c.set_positions(torch.from_numpy(xy[:off[4]]))
+        assert c.descend()[1].cpu().numpy().tolist() == [5, 5, 0, 0]
