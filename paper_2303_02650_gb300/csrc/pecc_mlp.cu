@@ -48,12 +48,15 @@ __device__ __forceinline__ float2 frame_er(float2 c) {
   return make_float2(__fdiv_rn(c.x, r), __fdiv_rn(c.y, r));
 }
 
-// A lane takes one circle: it collects the circles within 4.5 (at most two cells away: the grid's side
-// is at least 2.5) as positions in a column of its warp's buffer, then keeps the twelve least (squared
-// distance, index) of them as ascending 64-bit keys: the distance's bits, then the index (and, where
-// both fit 16 bits, the sorted position, which gives the coordinates without a search).  Collecting first
-// lets the insertions of a warp's lanes run together.  The warp's 32 rows of 25 values leave through
-// shared memory as one contiguous piece.
+// Cells that 4.5 spans: the grid's side is at least l_cut (1 + 2^-20), l_cut above 2.  (The margin covers
+// the binary32 distances: one below 4.5 is below 4.5 (1 + 2^-22) in exact terms.)
+static int knn_reach(double l_cut) { return l_cut >= 2.25 ? 2 : 3; }
+
+// A lane takes one circle: it collects the circles within 4.5 (at most `reach` cells away) as positions in
+// a column of its warp's buffer, then keeps the twelve least (squared distance, index) of them as ascending
+// 64-bit keys: the distance's bits, then the index (and, where both fit 16 bits, the sorted position, which
+// gives the coordinates without a search).  Collecting first lets the insertions of a warp's lanes run
+// together.  The warp's 32 rows of 25 values leave through shared memory as one contiguous piece.
 constexpr int kKnnBuf = 32;                               // collected per lane before they are inserted
 constexpr int kKnnWarpBytes = 32 * F * (int)sizeof(float);  // the rows of a warp
 static_assert(kKnnWarpBytes >= 32 * kKnnBuf * (int)sizeof(uint16_t), "the rows take the 16-bit buffer's place");
@@ -62,7 +65,7 @@ static_assert(kKnnWarpBytes <= 32 * kKnnBuf * (int)sizeof(int32_t), "and fit the
 // I: type of the sorted order's entries (16-bit: keys carry the position).
 template <typename I>
 __device__ __forceinline__ void feature_rows(const float2 *__restrict__ x, int n, int i, float Rf, int key, int nc,
-                                             const int32_t *start, const float2 *xs, const I *ord, void *scratch,
+                                             int reach, const int32_t *start, const float2 *xs, const I *ord, void *scratch,
                                              float *__restrict__ feat) {
   constexpr bool pack = sizeof(I) == 2;
   const int lane = threadIdx.x & 31;
@@ -97,8 +100,8 @@ __device__ __forceinline__ void feature_rows(const float2 *__restrict__ x, int n
       cnt = 0;
     };
     const int cy = key / nc, cx = key - cy * nc;
-    const int bx0 = max(cx - 2, 0), bx1 = min(cx + 2, nc - 1);
-    for (int yy = max(cy - 2, 0); yy <= min(cy + 2, nc - 1); ++yy) {
+    const int bx0 = max(cx - reach, 0), bx1 = min(cx + reach, nc - 1);
+    for (int yy = max(cy - reach, 0); yy <= min(cy + reach, nc - 1); ++yy) {
       const int lo = start[yy * nc + bx0], hi = start[yy * nc + bx1 + 1];
       for (int q = lo; q < hi; ++q) {
         if (!(dist2(q) < kKnnR2)) continue;
@@ -135,7 +138,7 @@ __device__ __forceinline__ void feature_rows(const float2 *__restrict__ x, int n
 // Instances of at most kCellsBlockN circles, one block each (pecc_cells.cuh).  Bound by instruction issue
 // of the collecting and inserting walks: 142 us for 665 000 circles in 1024 instances, 460 us when cells
 // and lists lay in global memory and every lane inserted as it walked.
-__global__ void __launch_bounds__(256) features_block_kernel(StandaloneParams P, float *feat) {
+__global__ void __launch_bounds__(256) features_block_kernel(StandaloneParams P, int reach, float *feat) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int32_t sh[40];
   const int q = P.eorder[blockIdx.x];
@@ -149,19 +152,20 @@ __global__ void __launch_bounds__(256) features_block_kernel(StandaloneParams P,
   void *scratch = C.extra + (threadIdx.x >> 5) * kKnnWarpBytes;
   for (int i0 = threadIdx.x & ~31; i0 < n; i0 += blockDim.x) {
     const int i = i0 + (threadIdx.x & 31);
-    feature_rows<uint16_t>(X.x, n, i, (float)D.R, i < n ? (int)C.key[i] : 0, D.ncx, C.start, C.xs, C.ord, scratch,
-                           feat + (size_t)D.off * F);
+    feature_rows<uint16_t>(X.x, n, i, (float)D.R, i < n ? (int)C.key[i] : 0, D.ncx, reach, C.start, C.xs, C.ord,
+                           scratch, feat + (size_t)D.off * F);
   }
 }
 
 // Tiles of the larger instances, over the cells that launch_large_cells32 left in the scratch.
-__global__ void __launch_bounds__(kTileRows) features_tile_kernel(StandaloneParams P, LargeTiles L, float *feat) {
+__global__ void __launch_bounds__(kTileRows) features_tile_kernel(StandaloneParams P, LargeTiles L, int reach,
+                                                                  float *feat) {
   __shared__ __align__(16) unsigned char sm[(kTileRows / 32) * 32 * kKnnBuf * 4];
   const int2 t = L.rows[blockIdx.x];
   const InstDesc &D = P.desc[t.x];
   const int n = D.n, i = t.y * kTileRows + threadIdx.x;
   if (i - (int)(threadIdx.x & 31) >= n) return;  // the whole warp
-  feature_rows<int32_t>(P.x32 + D.off, n, i, (float)D.R, i < n ? (int)P.ckey_t[D.off + i] : 0, D.ncx,
+  feature_rows<int32_t>(P.x32 + D.off, n, i, (float)D.R, i < n ? (int)P.ckey_t[D.off + i] : 0, D.ncx, reach,
                         P.cells + D.cell_off, (const float2 *)P.xtmp + D.off, P.corder_t + D.off,
                         sm + (threadIdx.x >> 5) * 32 * kKnnBuf * 4, feat + (size_t)D.off * F);
 }
@@ -846,12 +850,12 @@ cudaError_t mlp_features(const StandaloneParams &p, const LargeTiles &L, int n_s
   if (n_small >= 0) {
     const int block = n_small <= 64 ? 64 : (n_small <= 128 ? 128 : 256);
     const size_t smem = cells_smem(n_small, (size_t)(block / 32) * kKnnWarpBytes, false);
-    features_block_kernel<<<p.num, block, smem, s>>>(p, feat);
+    features_block_kernel<<<p.num, block, smem, s>>>(p, knn_reach(p.l_cut), feat);
   }
   if (L.nrows > 0) {
     cudaError_t e = launch_large_cells32(p, L, s);
     if (e != cudaSuccess) return e;
-    features_tile_kernel<<<L.nrows, kTileRows, 0, s>>>(p, L, feat);
+    features_tile_kernel<<<L.nrows, kTileRows, 0, s>>>(p, L, knn_reach(p.l_cut), feat);
   }
   return cudaGetLastError();
 }

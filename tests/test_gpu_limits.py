@@ -1,6 +1,6 @@
 """Calls at the limits of what they take (marked gpu): list overflow of any length, shared memory of any
 size, contexts of several host threads, waits that run out,
-radii that are not radii."""
+radii that are not radii, cutoffs close to 2."""
 import os
 import subprocess
 import sys
@@ -9,8 +9,9 @@ import threading
 import numpy as np
 import pytest
 
+from oracle import mlp as omlp
 from paper_2303_02650_gb300 import synth
-from gpu_util import need_gpu
+from gpu_util import need_gpu, split
 
 pytestmark = pytest.mark.gpu
 
@@ -191,3 +192,20 @@ def test_rejected_radius_is_reported(orc, bad):
         c.set_radius(R[:4])
         c.set_positions(torch.from_numpy(xy[:off[4]]))
         assert c.descend()[1].cpu().numpy().tolist() == [5, 5, 0, 0]
+
+
+@pytest.mark.parametrize("l_cut", [2.05, 2.1, 2.249, 2.25, 3.0])
+def test_features_reach_over_small_cells(l_cut):
+    """Cells of side l_cut: every circle within 4.5 is found, also where 4.5 spans three cells."""
+    torch, pecc = need_gpu()
+    n = np.array([900, 2600], dtype=np.int32)
+    R = np.array([synth.radius(int(v), 0.3) for v in n])  # about six circles within 4.5: all are kept
+    xy = np.concatenate([synth.random_layout(int(v), float(r), 31 + int(v)) for v, r in zip(n, R)])
+    half = (l_cut - 2.0) / 2.0
+    with pecc.Context(n, precision=1, l_cut=l_cut, rebuild_disp=half, step_max=half) as c:
+        c.set_radius(R)
+        c.set_positions(torch.from_numpy(xy))
+        xy = c.get_positions().cpu().numpy().astype(np.float32)
+        f = c.features().cpu().numpy()
+    for q, (fq, xq) in enumerate(zip(split(f, n), split(xy, n))):
+        assert np.array_equal(fq, omlp.features(xq, float(R[q]))), q
