@@ -98,9 +98,14 @@ __device__ __forceinline__ int cell_coord_fast(V v, float vf, double R, double i
   if (fr > slack && fr < 1.f - slack && f > 0.f && f < (float)nc) return (int)fl;
   return cell_coord((double)v, R, inv, nc);
 }
+// inv for it in binary32: NaN, which leaves every coordinate to binary64, for radii near the end of
+// binary32's range, where v + R would overflow (and inv lose bits).
+__device__ __forceinline__ float fast_inv(float Rf, double inv) {
+  return Rf < 1e37f ? (float)inv : __int_as_float(0x7fc00000);
+}
 template <typename P>
 __device__ __forceinline__ int cell_key_fast(P p, float2 f, double R, double inv, int nc) {
-  const float Rf = (float)R, invf = (float)inv, slack = (float)nc * (1.f / 1048576.f);
+  const float Rf = (float)R, invf = fast_inv(Rf, inv), slack = (float)nc * (1.f / 1048576.f);
   const int cx = cell_coord_fast(p.x, f.x, R, inv, nc, Rf, invf, slack);
   return cell_coord_fast(p.y, f.y, R, inv, nc, Rf, invf, slack) * nc + cx;
 }
@@ -242,7 +247,7 @@ __device__ __forceinline__ uint32_t grid_cell(v2<T> p, const CellGrid &G) {
     cx = !(fx >= 0.f) ? 0 : (fx >= (float)G.nc ? G.nc - 1 : (int)fx);
     cy = !(fy >= 0.f) ? 0 : (fy >= (float)G.nc ? G.nc - 1 : (int)fy);
   } else {
-    const float Rf = (float)G.R, invf = (float)G.inv, slack = (float)G.nc * (1.f / 1048576.f);
+    const float Rf = (float)G.R, invf = fast_inv(Rf, G.inv), slack = (float)G.nc * (1.f / 1048576.f);
     cx = cell_coord_fast(p.x, (float)p.x, G.R, G.inv, G.nc, Rf, invf, slack);
     cy = cell_coord_fast(p.y, (float)p.y, G.R, G.inv, G.nc, Rf, invf, slack);
   }

@@ -1,6 +1,6 @@
 """Calls at the limits of what they take (marked gpu): list overflow of any length, shared memory of any
 size, contexts of several host threads, waits that run out,
-radii that are not radii, cutoffs close to 2."""
+radii that are not radii or past binary32's range, cutoffs close to 2."""
 import os
 import subprocess
 import sys
@@ -209,3 +209,29 @@ def test_features_reach_over_small_cells(l_cut):
         f = c.features().cpu().numpy()
     for q, (fq, xq) in enumerate(zip(split(f, n), split(xy, n))):
         assert np.array_equal(fq, omlp.features(xq, float(R[q]))), q
+
+
+@pytest.mark.parametrize("R0", [1e36, 1e37, 2e38, 1e39, 1e100])
+def test_cells_of_huge_containers(orc, R0):
+    """Radii near and past the largest binary32 value: the cells are those of the binary64 operations."""
+    torch, pecc = need_gpu()
+    n = np.array([300, 2100], dtype=np.int32)
+    R = np.array([R0, R0])
+    xy = np.concatenate([synth.random_layout(int(v), R0, 5 + int(v)) for v in n])
+    xy[:4] = [[0.5, -0.5], [0.5, 1.5], [-R0, R0], [3.0 * R0, 0.0]]
+    with pecc.Context(n, precision=0) as c:
+        c.set_radius(R)
+        c.set_positions(torch.from_numpy(xy))
+        c.rebuild_neighbors(force=True)
+        key, order = [t.cpu().numpy() for t in c.export_cells()]
+        rp, col = [t.cpu().numpy() for t in c.export_neighbors()]
+        mo = c.check_feasible()[1].cpu().numpy()
+    off = np.concatenate([[0], np.cumsum(n)])
+    for q in range(len(n)):
+        a, b = off[q], off[q + 1]
+        kref = orc.cell_keys(xy[a:b], R0, 2.5)
+        assert np.array_equal(key[a:b].astype(np.uint32), kref), q
+        assert np.array_equal(order[a:b], np.argsort(kref, kind="stable")), q
+        rref, cref = orc.neighbors_brute(xy[a:b], 2.5)
+        assert np.array_equal(rp[a:b + 1] - rp[a], rref) and np.array_equal(col[rp[a]:rp[b]] - a, cref), q
+        assert mo[q] == orc.max_overlap(xy[a:b], R0)[0], q
