@@ -227,8 +227,6 @@ pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
   };
   if (cudaGetDevice(&ctx->device) != cudaSuccess) return bail(fail(ctx, PECC_ERR_CUDA, "no CUDA device"));
   cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
-  if (standalone_smem_limits() != cudaSuccess || (cfg->precision != PECC_FP64 && features_smem_limit() != cudaSuccess))
-    return bail(fail(ctx, PECC_ERR_CUDA, "shared-memory limits"));
 
   const int m1 = cfg->lbfgs_m + 1;
   const bool fp64 = cfg->precision == PECC_FP64;
@@ -343,6 +341,9 @@ pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
     for (int t = 0; t < (n + kTileRows - 1) / kTileRows; ++t) row_tiles.push_back(make_int2(q, t));
     for (int64_t t = 0; t < nct; ++t) cell_tiles.push_back(make_int2(q, (int)t));
   }
+  if (standalone_smem_limits(ctx->n_small, ctx->eg_small) != cudaSuccess ||
+      (!fp64 && features_smem_limit(ctx->n_small) != cudaSuccess))
+    return bail(fail(ctx, PECC_ERR_CUDA, "shared-memory limits"));
   if (!row_tiles.empty()) {
     LargeTiles &L = ctx->lt;
     L.nrows = (int)row_tiles.size();

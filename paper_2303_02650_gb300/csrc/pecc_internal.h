@@ -218,8 +218,14 @@ int adjust_max_m();
 // thread's between that and the launch, so every setting is this same one, made when a context is created
 // (the standalone kernels) or plans its descent.  A launch takes what it asks for, whatever the limit.
 cudaError_t raise_smem_limit(const void *kernel);
-cudaError_t standalone_smem_limits();
-cudaError_t features_smem_limit();
+// ... if launches of up to `bytes` need it: 48 KB, static shared memory included, need not be asked for
+// (a context of small instances is created 80 us faster without).
+inline cudaError_t raise_smem_limit(const void *kernel, size_t bytes) {
+  return bytes <= 44 * 1024 ? cudaSuccess : raise_smem_limit(kernel);  // 4 KB: far more than a kernel's own
+}
+// n_small, eg_small: the largest instances that the kernels of one block per instance take (-1: none)
+cudaError_t standalone_smem_limits(int n_small, const int (&eg_small)[3]);
+cudaError_t features_smem_limit(int n_small);
 
 // Largest instance whose coordinates the block energy + gradient kernel stages in shared memory.
 inline int energy_stage_n(int eval) { return (int)(PECC_ENERGY_STAGE_BYTES / (eval == 1 ? 8 : 16)); }

@@ -938,11 +938,18 @@ cudaError_t raise_smem_limit(const void *kernel) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
 }
 
-cudaError_t standalone_smem_limits() {
-  for (const void *k : {(const void *)build_block_kernel<float>, (const void *)build_block_kernel<double>,
-                        (const void *)feasible_block_kernel, (const void *)energy_grad_block_kernel<Arith64>,
-                        (const void *)energy_grad_block_kernel<Arith32>, (const void *)energy_grad_block_kernel<ArithMix>})
-    if (cudaError_t e = raise_smem_limit(k)) return e;
+cudaError_t standalone_smem_limits(int n_small, const int (&eg_small)[3]) {
+  const size_t rows = 16 * (size_t)kBuildWarpBytes;  // of 512 threads
+  const int n = std::max(n_small, 0);
+  const struct { const void *kernel; size_t bytes; } most[] = {
+      {(const void *)build_block_kernel<float>, cells_smem(n, rows, false)},
+      {(const void *)build_block_kernel<double>, cells_smem(n, rows, true)},
+      {(const void *)feasible_block_kernel, cells_smem(n, 0, true)},
+      {(const void *)energy_grad_block_kernel<Arith64>, sizeof(double2) * (size_t)std::max(eg_small[0], 0)},
+      {(const void *)energy_grad_block_kernel<Arith32>, sizeof(float2) * (size_t)std::max(eg_small[1], 0)},
+      {(const void *)energy_grad_block_kernel<ArithMix>, sizeof(double2) * (size_t)std::max(eg_small[2], 0)}};
+  for (const auto &k : most)
+    if (cudaError_t e = raise_smem_limit(k.kernel, k.bytes)) return e;
   return cudaSuccess;
 }
 

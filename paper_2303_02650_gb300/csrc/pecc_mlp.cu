@@ -843,7 +843,10 @@ cudaError_t mlp_sync_bf16(const float *params, bf16 *wb, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t features_smem_limit() { return raise_smem_limit((const void *)features_block_kernel); }
+cudaError_t features_smem_limit(int n_small) {
+  return raise_smem_limit((const void *)features_block_kernel,
+                          cells_smem(std::max(n_small, 0), 8 * (size_t)kKnnWarpBytes, false));
+}
 
 cudaError_t mlp_features(const StandaloneParams &p, const LargeTiles &L, int n_small, float *feat, cudaStream_t s) {
   if (p.num <= 0) return cudaSuccess;
