@@ -272,6 +272,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
 
   // ---- 1. partition: keys, their range, buckets by value, per-bucket (key, index) order
   const int nbk = max(1, n / 4);
+  int32_t *arrived = (int32_t *)dv;  // circles by bucket, in arrival order (scratch: the direction)
   {
     double kmax = -1e300, kmin_neg = -1e300;
     for (int i = gid; i < n; i += gstride) {
@@ -308,32 +309,44 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
     for (int c = gid; c < nbk; c += gstride) bfill[c] = G.bucket[c];
     ok = grid_sync(S, ctl);
     if (ok) {
-      for (int i = gid; i < n; i += gstride) perm[atomicAdd(&bfill[bucket_of(skey[i])], 1)] = i;
+      for (int i = gid; i < n; i += gstride) arrived[atomicAdd(&bfill[bucket_of(skey[i])], 1)] = i;
       ok = grid_sync(S, ctl);
     }
   }
   if (ok) {
-    for (int c = gid; c < nbk; c += gstride) {  // insertion sort of a bucket by (key, index)
-      const int lo = G.bucket[c], hi = G.bucket[c + 1];
-      for (int a = lo + 1; a < hi; ++a) {
-        const int v = perm[a];
-        const uint64_t kv = skey[v];
-        int b = a - 1;
-        while (b >= lo) {
-          const int u = perm[b];
-          const uint64_t ku = skey[u];
-          if (ku < kv || (ku == kv && u < v)) break;
-          perm[b + 1] = u;
-          --b;
-        }
-        perm[b + 1] = v;
+    // (key, index) order: a circle's place in its bucket is the number of smaller ones there.  Buckets
+    // sorted by one thread each took n^2 / 4 serial steps where all keys are equal (circles in one place),
+    // minutes past the other blocks' wait.
+    for (int p = gid; p < n; p += gstride) {
+      const int i = arrived[p];
+      const uint64_t ki = skey[i];
+      const int c = bucket_of(ki), lo = G.bucket[c], hi = G.bucket[c + 1];
+      int r = lo;
+      for (int b = lo; b < hi; ++b) {
+        const int u = arrived[b];
+        const uint64_t ku = skey[u];
+        r += ku < ki || (ku == ki && u < i);
       }
+      perm[r] = i;
     }
     ok = grid_sync(S, ctl);
   }
   // ---- 2. renumber in partition order
   int bad = 0;
-  if (ok) {
+  if (!ok) {  // a barrier failed: perm and xw hold nothing to scatter
+    if (A::kId == 2)  // the layout stays the FP32 descent's
+      for (int i = gid; i < n; i += gstride) {
+        const float2 v = P.x32[D.off + i];
+        P.x64[D.off + i] = make_double2((double)v.x, (double)v.y);
+      }
+    if (gid == 0) {
+      if (A::kId == 1) { O->status32 = 6; O->E32 = 0.0; }
+      if (A::kId != 2) O->iters = O->iters32 = O->trials32 = O->builds = O->changes = O->trials = O->resets = O->stalls = 0;
+      O->status = 6; O->E = 0.0; O->polished = A::kId == 2;
+    }
+    return;
+  }
+  {
     for (int p = gid; p < n; p += gstride) {
       const int i = perm[p];
       PP v;

@@ -235,3 +235,18 @@ def test_cells_of_huge_containers(orc, R0):
         rref, cref = orc.neighbors_brute(xy[a:b], 2.5)
         assert np.array_equal(rp[a:b + 1] - rp[a], rref) and np.array_equal(col[rp[a]:rp[b]] - a, cref), q
         assert mo[q] == orc.max_overlap(xy[a:b], R0)[0], q
+
+
+@pytest.mark.parametrize("n,R0,expect", [(50000, 260.0, 4), (20000, -1.0, 5), (16384, 1.0, 4)])
+def test_whole_gpu_descent_of_coincident_circles(n, R0, expect):
+    """All circles in one place (as pecc_init_random leaves them for R <= 1 or a rejected radius): equal
+    partition keys, one bucket.  The descent ends with its status well before a barrier's time limit."""
+    torch, pecc = need_gpu()
+    with pecc.Context(np.array([n], dtype=np.int32), precision=2) as c:
+        c.set_radius(np.array([R0]))
+        c.init_random(3) if R0 <= 1.0 else c.set_positions(torch.zeros(n, 2, dtype=torch.float64))
+        x0 = c.get_positions()
+        assert not x0.any()
+        iters, status = c.descend()
+        assert int(status.cpu()[0]) == expect and int(iters.cpu()[0]) == 0
+        assert torch.equal(c.get_positions(), x0)
