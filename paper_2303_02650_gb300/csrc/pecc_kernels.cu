@@ -126,12 +126,12 @@ __device__ __forceinline__ void for_neighbors(const Coords<T> &X, int i, int key
 }
 
 // The 32 rows of a warp, once every lane knows where its row starts: buf holds the lane's hits at
-// buf[32 h + lane] (cnt of them when cnt <= kRowHits), row0 is the lane's row start.  Entries at or
-// past cap are not written (an overflowed list).
+// buf[32 h + lane] (cnt of them when cnt <= kRowHits), row0 is the lane's row start.  Called only where the
+// block's rows end within the list's capacity: rows of an overflowed list are not written (nor sorted: in
+// a crowd they can hold every circle).
 template <typename T, typename I>
 __device__ __forceinline__ void write_rows(const Coords<T> &X, bool act, int i, int key, int nc, const int32_t *start,
-                                           const float2 *xs, const I *ord, I *buf, int cnt, int row0, int32_t *col,
-                                           int cap) {
+                                           const float2 *xs, const I *ord, I *buf, int cnt, int row0, int32_t *col) {
   const int lane = threadIdx.x & 31;
   if (__any_sync(0xffffffffu, cnt > kRowHits)) {
     if (act) {
@@ -140,12 +140,9 @@ __device__ __forceinline__ void write_rows(const Coords<T> &X, bool act, int i, 
       int w = row0;
       for_neighbors<T, I>(X, i, key, nc, start, xs, ord, near, [&](int q) {
         const int v = (int)ord[q];
-        if (w < cap) {  // insert in ascending order
-          int t = w - 1;
-          while (t >= row0 && col[t] > v) { col[t + 1] = col[t]; --t; }
-          col[t + 1] = v;
-        }
-        ++w;
+        int t = w++ - 1;
+        while (t >= row0 && col[t] > v) { col[t + 1] = col[t]; --t; }  // insert in ascending order
+        col[t + 1] = v;
       });
     }
     return;
@@ -182,8 +179,7 @@ __device__ __forceinline__ void write_rows(const Coords<T> &X, bool act, int i, 
   for (int u = 0; u < kRowHits; ++u)
     if (u < cnt) buf[row0 - base + rank[u]] = (I)h[u];
   __syncwarp();
-  for (int t = lane; t < total; t += 32)
-    if (base + t < cap) col[base + t] = (int)buf[t];
+  for (int t = lane; t < total; t += 32) col[base + t] = (int)buf[t];
   __syncwarp();  // the next rows' hits go into the same buffer
 }
 
@@ -281,8 +277,8 @@ __global__ void __launch_bounds__(512, 3) build_block_kernel(StandaloneParams P,
     int total;
     const int row0 = run + block_exclusive(cnt, sh, total);
     if (act) rp[i + 1] = row0 + cnt;
-    write_rows<T, uint16_t>(X, act, i, key, nc, C.start, C.xs, C.ord, buf, cnt, row0, col, cap);
     run += total;
+    if (run <= cap) write_rows<T, uint16_t>(X, act, i, key, nc, C.start, C.xs, C.ord, buf, cnt, row0, col);
   }
 }
 
@@ -461,7 +457,8 @@ __global__ void __launch_bounds__(kTileRows) large_rows_kernel(StandaloneParams 
   int32_t *rp = P.rp + D.off + t.x;
   if (act) rp[i + 1] = sat_add(row0, cnt);
   if (i == 0) rp[0] = 0;
-  write_rows<T, int32_t>(X, act, i, key, nc, start, xs, ord, buf, cnt, row0, P.col + D.col_s_off, D.cap);
+  if (sat_add(base, total) <= D.cap)
+    write_rows<T, int32_t>(X, act, i, key, nc, start, xs, ord, buf, cnt, row0, P.col + D.col_s_off);
 }
 
 // Cells, order and sorted coordinates of every large instance (flags in L.go, or all of them).

@@ -250,3 +250,55 @@ def test_whole_gpu_descent_of_coincident_circles(n, R0, expect):
         iters, status = c.descend()
         assert int(status.cpu()[0]) == expect and int(iters.cpu()[0]) == 0
         assert torch.equal(c.get_positions(), x0)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_overflow_of_crowded_cells(orc, prec):
+    """Crowds around the corner of four cells: the lists overflow, and the crowd's rows (every other circle
+    of it, from several cells) are not put in order first.  The rest of the batch is unaffected; a crowd
+    that fits is listed in full."""
+    torch, pecc = need_gpu()
+    n = np.array([2048, 50000, 300, 2048, 3000], dtype=np.int32)
+    crowd = [2048, 50000, 0, 120, 150]
+    R = np.array([synth.radius(int(v), 0.8) for v in n])
+    rng = np.random.default_rng(4)
+    parts = []
+    for v, m, r in zip(n, crowd, R):
+        x = synth.random_layout(int(v), 0.9 * float(r), 3 + int(v))
+        side = 2.5 * (1.0 + 2.0 ** -20)
+        corner = -r + side * np.floor(r / side)
+        x[:m] = corner + rng.uniform(-0.4, 0.4, size=(m, 2))
+        parts.append(x.astype(np.float32).astype(np.float64))
+    off = np.concatenate([[0], np.cumsum(n)])
+    with pecc.Context(n, precision=prec) as c:
+        c.set_radius(R)
+        c.set_positions(torch.from_numpy(np.concatenate(parts)))
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        c.check_feasible()
+        ev[0].record()
+        c.rebuild_neighbors(force=True)
+        ev[1].record()
+        torch.cuda.synchronize()
+        assert ev[0].elapsed_time(ev[1]) < 2000.0
+        with pytest.raises(pecc.PeccError, match="NBR_OVERFLOW"):
+            c.export_neighbors()
+        E, g = [t.cpu().numpy() for t in c.energy_grad()]
+    for q in range(len(n)):
+        if crowd[q] == n[q]:
+            assert np.isnan(E[q]) and np.isnan(g[off[q]:off[q + 1]]).all()
+        else:
+            # binary32: a thread adds up at most about 2400 positive terms, 2^-24 each
+            ref = orc.energy_allpairs(parts[q], float(R[q]))
+            assert abs(E[q] - ref) <= (1e-12 if prec == 0 else 2e-4) * ref
+    keep = [2, 3, 4]
+    with pecc.Context(n[keep], precision=prec) as c:
+        c.set_radius(R[keep])
+        c.set_positions(torch.from_numpy(np.concatenate([parts[q] for q in keep])))
+        c.rebuild_neighbors(force=True)
+        rp, col = [t.cpu().numpy() for t in c.export_neighbors()]
+    a = 0
+    for q in keep:
+        b = a + n[q]
+        rref, cref = orc.neighbors_brute(parts[q], 2.5, prec32=(prec == 1))
+        assert np.array_equal(rp[a:b + 1] - rp[a], rref) and np.array_equal(col[rp[a]:rp[b]] - a, cref), q
+        a = b
