@@ -477,6 +477,11 @@ cudaError_t large_cells(const StandaloneParams &p, const LargeTiles &L, const La
 }
 
 // ------------------------------------------------- fused energy + gradient ----
+// A radius that pecc_set_radius did not accept is NaN (binary64: told by its bits, as the arithmetic units of
+// that width are few: a comparison took 2 % of the 4096-instance batch's energies).
+__device__ __forceinline__ bool rejected(float R) { return R != R; }
+__device__ __forceinline__ bool rejected(double R) { return not_finite(R); }
+
 // One thread per circle (gather over its row, no atomics):
 //   g_i = sum_{j in Gamma(i)} -2 d_ij (c_i - c_j) / l_ij + 2 d_i0 c_i / |c_i|
 //   e_i = sum_{j in Gamma(i), j < i} d_ij^2 + d_i0^2      (so that E = sum_i e_i, Eq. 5)
@@ -505,9 +510,7 @@ __global__ void __launch_bounds__(256) energy_grad_kernel(StandaloneParams P, in
   vec_t gx = 0, gy = 0;
   acc_t e = 0;
   const int lo = __ldg(rp + i), hi = __ldg(rp + i + 1);
-  // the last build overflowed the list's capacity (no valid list), or the radius was rejected (NaN; tested
-  // by its bits: binary64 instructions issue slowly)
-  if (__ldg(rp + P.desc[q].n) > P.desc[q].cap || not_finite(Rd)) {
+  if (__ldg(rp + P.desc[q].n) > P.desc[q].cap) {  // the last build overflowed the list's capacity: no valid list
     VV gv; gv.x = gv.y = (vec_t)NAN;
     ((VV *)grad_)[gi] = gv;
     ((acc_t *)ecirc_)[gi] = (acc_t)NAN;
@@ -534,6 +537,10 @@ __global__ void __launch_bounds__(256) energy_grad_kernel(StandaloneParams P, in
   acc_t d0 = A::wall(xi, R, Rm1sq, fx, fy);
   gx += fx; gy += fy;
   e += d0 * d0;
+  if (rejected(R)) {  // tested here, where the radius has come in
+    gx = gy = (vec_t)NAN;
+    e = (acc_t)NAN;
+  }
   VV gv; gv.x = gx; gv.y = gy;
   ((VV *)grad_)[gi] = gv;
   ((acc_t *)ecirc_)[gi] = e;
@@ -578,9 +585,8 @@ __global__ void __launch_bounds__(kEgBlock) energy_grad_block_kernel(StandaloneP
   // are in flight together instead of one load round trip per coordinate
   for (int i = threadIdx.x; i < n; i += blockDim.x) cp_async_shared<sizeof(PP)>(xs + i, x + i);
   asm volatile("cp.async.wait_all;\n" ::: "memory");
-  // the last build overflowed the list's capacity (no valid list), or the radius was rejected (NaN; tested
-  // by its bits: binary64 instructions issue slowly)
-  if (end > P.desc[q].cap || not_finite(Rd)) {
+  // the last build overflowed the list's capacity (no valid list), or the radius was rejected
+  if (end > P.desc[q].cap || rejected(R)) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) { VV gv; gv.x = gv.y = (vec_t)NAN; grad[i] = gv; }
     if (threadIdx.x == 0) E[q] = NAN;
     return;
