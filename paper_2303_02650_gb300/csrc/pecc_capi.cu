@@ -262,10 +262,10 @@ pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
     rp_off += 2 * (int64_t)(n + 1);
     col_off += 2 * (int64_t)D.cap;
     col_s_off += D.cap;
-    gram_off += (int64_t)k * kBasis * kBasis;
+    gram_off += (int64_t)k * kGram;
     meta_off += (int64_t)k * kMetaInts;
     const int cap_c = cell_grid_cap(n);  // the cell table of the largest grid the instance can get
-    cell_off += 2 * (int64_t)cap_c * cap_c + 2;
+    cell_off += (int64_t)cap_c * cap_c + 1;
   }
   pecc_status s;
 #define ALC(ptr, T, count)                                   \
@@ -324,7 +324,7 @@ pecc_status pecc_create(const pecc_config *cfg, void *stream, pecc_ctx **out) {
     ALC(ctx->gb.ipart, int32_t, ctx->ggrid);
     ALC(ctx->gb.bucket, int32_t, 2 * (size_t)(nmax_big / 4) + 4);
     ALC(ctx->gb.hash, unsigned long long, 1);
-    ALC(p, char, (size_t)ctx->ggrid * kmax * kBasis * kBasis * 8); ctx->gb.gram = p;
+    ALC(p, char, (size_t)ctx->ggrid * kmax * kGram * 8); ctx->gb.gram = p;
     ctx->gb.kmax = kmax;
     ALC(ctx->gctl, GridCtl, 1);
   }

@@ -55,14 +55,11 @@ template <> struct Near<double> {
   double lc2;
   float lc;
   float2 xf;
-  float lo, hi;  // binary32 squared distances below lo are inside, above hi outside
+  float lo, hi;
   __device__ __forceinline__ explicit Near(double l_cut) : lc2(l_cut * l_cut), lc((float)l_cut) {}
   __device__ __forceinline__ void set(float2 x) {
     xf = x;
-    const float m = dist_slack(fabsf(x.x) + fabsf(x.y), lc);
-    const bool ok = m <= 0.25f;  // else (far out, not finite): every distance in binary64
-    lo = ok ? (lc - m) * (lc - m) : -1.f;
-    hi = ok ? (lc + m) * (lc + m) : __int_as_float(0x7f800000);
+    near_bounds(x, lc, lo, hi);
   }
   template <typename I>
   __device__ __forceinline__ bool operator()(int i, float2 xq, const Coords<double> &X, const I *ord, int q) const {

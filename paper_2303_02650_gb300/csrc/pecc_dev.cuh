@@ -31,8 +31,8 @@ struct InstDesc {
   int64_t rp_off;           // 2 * (n + 1) row pointers (two CSR buffers)
   int64_t col_off;          // 2 * cap column entries (descent lists)
   int64_t col_s_off;        // cap column entries (standalone lists; row pointers at off + index)
-  int64_t cell_off;         // 2 * ncell + 2 cell counters
-  int64_t gram_off;         // k * kBasis * kBasis Gram entries
+  int64_t cell_off;         // cell table: cell_grid_cap(n)^2 + 1 counters
+  int64_t gram_off;         // k * kGram Gram entries
   int64_t meta_off;         // k * kMetaInts ring metadata
   double R, inv_cs;
   float inv_f;              // binary32 grid of the FP32 descent: 1 / side, side >= l_cut (1 + 2^-10)
@@ -114,6 +114,15 @@ __device__ __forceinline__ int cell_key_fast(P p, float2 f, double R, double inv
 // distance l: the binary32 distance of the rounded coordinates is off by less than 2^-22 (M + l).
 __device__ __forceinline__ float dist_slack(float M, float l) { return (M + l + 8.f) * (1.f / 1048576.f); }
 
+// Bounds of the binary32 squared distances from a circle at x that decide the predicate for cutoff lc by
+// themselves: below lo inside, above hi outside, the rest in binary64.
+__device__ __forceinline__ void near_bounds(float2 x, float lc, float &lo, float &hi) {
+  const float m = dist_slack(fabsf(x.x) + fabsf(x.y), lc);
+  const bool ok = m <= 0.25f;  // else (far out, not finite): every distance in binary64
+  lo = ok ? (lc - m) * (lc - m) : -1.f;
+  hi = ok ? (lc + m) * (lc + m) : __int_as_float(0x7f800000);
+}
+
 // Neighbor predicate of Sec. 4.3: dx*dx + dy*dy < l_cut^2 with every operation
 // correctly rounded (no contraction), in the coordinates' own precision.
 __device__ __forceinline__ bool nbr_pred(float2 a, float2 b, float lc2) {
@@ -183,10 +192,10 @@ constexpr int32_t kMaxEntries = 0x3fffffff;
 
 __device__ __forceinline__ int32_t sat_add(int32_t a, int32_t b) { return min(a + b, kMaxEntries); }
 
-// Inclusive prefix sum of a[0..len) in place (int32), whole block; copy (may be null) receives the
-// same sums.  SAT: the sums stop at kMaxEntries (entry counts of lists).
+// Inclusive prefix sum of a[0..len) in place (int32), whole block.  SAT: the sums stop at kMaxEntries
+// (entry counts of lists).
 template <bool SAT = false>
-__device__ inline void block_scan_inplace(int32_t *a, int len, int32_t *sh /*>=33 ints*/, int32_t *copy = nullptr) {
+__device__ inline void block_scan_inplace(int32_t *a, int len, int32_t *sh /*>=33 ints*/) {
   const int T = blockDim.x, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = T >> 5;
   auto add = [](int32_t x, int32_t y) { return SAT ? sat_add(x, y) : x + y; };
   int ch = (len + T - 1) / T;
@@ -218,10 +227,7 @@ __device__ inline void block_scan_inplace(int32_t *a, int len, int32_t *sh /*>=3
   } else {
     run += incl - s;
   }
-  if (copy)
-    for (int i = lo; i < hi; ++i) { run = add(run, a[i]); a[i] = run; copy[i] = run; }
-  else
-    for (int i = lo; i < hi; ++i) { run = add(run, a[i]); a[i] = run; }
+  for (int i = lo; i < hi; ++i) { run = add(run, a[i]); a[i] = run; }
   __syncthreads();
 }
 
@@ -269,13 +275,6 @@ __device__ __forceinline__ unsigned long long mix32(uint32_t x) {
   return (unsigned long long)x;
 }
 
-// Cell binning and stable key sort, then CSR rows over the 3x3 cells.  x: n positions of
-// one instance; lists go to rp[0..n], col[0..cap).  cells: nc^2 + 1 int32 of scratch;
-// ckey/corder: n each; xs: n positions of scratch (the coordinates in cell order, so that
-// the three cells of a row of the 3x3 block are one contiguous range).  All pointers may
-// be shared or global memory.  Rows come in cell-scan order (deterministic).  Returns the number of entries (block-uniform); > cap means
-// overflow and the rows are then not written.  hash (shared, may be null) receives an
-// order-independent 64-bit digest of the pair set, used to tell Gamma' from Gamma.
 // Cell binning and stable key sort of one instance (the first half of a list build): ckey[i] = cell
 // of circle i (cx | cy << 16), corder = circles sorted by (cell, index), cells[0..ncell] = cell starts,
 // xs[q] = coordinates of corder[q] rounded to binary32.  tmp: n int32 of scratch.  A circle keeps its
@@ -342,10 +341,7 @@ template <> struct SortedNear<double> {
   __device__ __forceinline__ void set(int q0) {
     a = xs[q0];
     i = order[q0];
-    const float m = dist_slack(fabsf(a.x) + fabsf(a.y), lc);
-    const bool ok = m <= 0.25f;  // else (far out, not finite): every distance in binary64
-    lo = ok ? (lc - m) * (lc - m) : -1.f;
-    hi = ok ? (lc + m) * (lc + m) : __int_as_float(0x7f800000);
+    near_bounds(a, lc, lo, hi);
   }
   __device__ __forceinline__ bool operator()(int qq) const {
     const float2 b = xs[qq];
@@ -356,6 +352,14 @@ template <> struct SortedNear<double> {
   }
 };
 
+// Cell binning and stable key sort of one instance of fewer than kGridMinN circles (its entries fit 32
+// bits), then CSR rows over the 3x3 cells.  x: n positions; lists go to rp[0..n], col[0..cap).  cells:
+// nc^2 + 1 int32 of scratch; ckey/corder: n each; xs_: room for n positions, which takes the binary32
+// coordinates in cell order, so that the three cells of a row of the 3x3 block are one contiguous range.
+// All pointers may be shared or global memory.  Rows come in cell-scan order (deterministic).  Returns the
+// number of entries (block-uniform); > cap means overflow: the rows are then not written, rp holds no list.
+// hash (shared, may be null) receives an order-independent 64-bit digest of the pair set, used to tell
+// Gamma' from Gamma.
 template <typename T, typename IdxT>
 __device__ int cta_build_neighbors(const v2<T> *__restrict__ x, int n, const CellGrid &G, T lc2,
                                    uint32_t *ckey, int32_t *corder, int32_t *cells, v2<T> *xs_, int32_t *rp,

@@ -69,7 +69,6 @@ template <class A> struct GSmem {
   int ring[kMaxK][kRing];
   int32_t sh[40];
   long long iv[2];
-  int flag;
   int rbuf;  // partial buffer of the next grid_reduce (same in every block)
   unsigned barriers;  // grid barriers passed
 };
@@ -487,7 +486,7 @@ __global__ void __launch_bounds__(256, 1) descend_grid_kernel(DescendParams P, i
   }
   for (int u = tid; u < k * kRing; u += blockDim.x) S.ring[u / kRing][u % kRing] = 0;
   // every block keeps identical Gram matrices (built from identical totals) in its own slice
-  vec_t *gram_mine = (vec_t *)G.gram + (size_t)blockIdx.x * G.kmax * kBasis * kBasis;
+  vec_t *gram_mine = (vec_t *)G.gram + (size_t)blockIdx.x * G.kmax * kGram;
   for (int u = tid; u < k * kGram; u += blockDim.x) (k <= kGramOnChip ? S.gram : gram_mine)[u] = vec_t(0);
   __syncthreads();
 

@@ -106,7 +106,7 @@ struct GridBufs {
   int32_t *ipart;           // [grid] block totals of integer scans
   int32_t *bucket;          // [2 (n / 4) + 2] partition buckets
   unsigned long long *hash; // [1] pair-set digest
-  void *gram;               // [grid][kmax][kBasis^2] per-block Gram copies
+  void *gram;               // [grid][kmax][kGram] per-block Gram copies
   int kmax;
 };
 constexpr int kGridMinN = 16384;  // instances this large descend on the whole GPU

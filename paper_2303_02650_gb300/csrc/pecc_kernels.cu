@@ -712,9 +712,8 @@ __device__ __forceinline__ void exact_bounds(float smin, float rmax, float *s_hi
 
 // Visit the circles around sorted position p: f(q, squared distance in binary32) for every other circle
 // of its 3x3 cells.
-template <typename I, typename F>
-__device__ __forceinline__ void for_candidates(int p, int key, int nc, const int32_t *start, const float2 *xs,
-                                               const I *, F f) {
+template <typename F>
+__device__ __forceinline__ void for_candidates(int p, int key, int nc, const int32_t *start, const float2 *xs, F f) {
   const int cy = key / nc, cx = key - cy * nc;
   const int bx0 = max(cx - 1, 0), bx1 = min(cx + 1, nc - 1);
   const float2 a = xs[p];
@@ -756,7 +755,7 @@ __global__ void __launch_bounds__(512, 3) feasible_block_kernel(StandaloneParams
   for (int p = threadIdx.x; p < n; p += blockDim.x) {
     const int i = C.ord[p];
     near.set(C.xs[p]);
-    for_candidates(p, (int)C.key[i], nc, C.start, C.xs, C.ord, [&](int qq, float s) {
+    for_candidates(p, (int)C.key[i], nc, C.start, C.xs, [&](int qq, float s) {
       smin = fminf(smin, s);
       if (s > near.hi) return;
       hits += (s < near.lo) || nbr_pred(X.at(i), X.at(C.ord[qq]), near.lc2);
@@ -787,7 +786,7 @@ __global__ void __launch_bounds__(512, 3) feasible_block_kernel(StandaloneParams
       if (!(a.x * a.x + a.y * a.y < r_lo)) r2 = fmax(r2, norm2_exact(X.at(i)));
       if (pairs) {  // each pair once; in a finished layout every contact lies within the slack
         const double2 xi = X.at(i);
-        for_candidates(p, (int)C.key[i], nc, C.start, C.xs, C.ord, [&](int qq, float s) {
+        for_candidates(p, (int)C.key[i], nc, C.start, C.xs, [&](int qq, float s) {
           if (qq > p && !(s > s_hi))
             sb = min(sb, (unsigned long long)__double_as_longlong(dist2_exact(xi, X.at(C.ord[qq]))));
         });
@@ -823,7 +822,7 @@ __global__ void __launch_bounds__(kTileRows) large_check_kernel(StandaloneParams
       const int i = ord[p];
       Near<double> near(P.l_cut);
       near.set(xs[p]);
-      for_candidates(p, (int)O.ckey[D.off + i], nc, start, xs, ord, [&](int q, float s) {
+      for_candidates(p, (int)O.ckey[D.off + i], nc, start, xs, [&](int q, float s) {
         smin = fminf(smin, s);
         if (s > near.hi) return;
         hits += (s < near.lo) || nbr_pred(X.at(i), X.at(ord[q]), near.lc2);
@@ -845,7 +844,7 @@ __global__ void __launch_bounds__(kTileRows) large_check_kernel(StandaloneParams
     if (!(a.x * a.x + a.y * a.y < r_lo))
       atomicMax(&L.rmax[t.x], (unsigned long long)__double_as_longlong(norm2_exact(X.at(i))));
     unsigned long long sb = 0x7ff0000000000000ull;  // squared distances compare as integers
-    for_candidates(p, (int)O.ckey[D.off + i], nc, start, xs, ord, [&](int q, float s) {
+    for_candidates(p, (int)O.ckey[D.off + i], nc, start, xs, [&](int q, float s) {
       if (q > p && !(s > s_hi))  // each pair once; in a finished layout every contact lies within the slack
         sb = min(sb, (unsigned long long)__double_as_longlong(dist2_exact(X.at(i), X.at(ord[q]))));
     });

@@ -25,8 +25,8 @@ constexpr size_t kOffX = 0;                                   // double2[kMaxN]
 constexpr size_t kOffXs = kOffX + sizeof(double2) * kMaxN;    // double2[kMaxN]
 constexpr size_t kOffKey = kOffXs + sizeof(double2) * kMaxN;  // uint32[kMaxN]
 constexpr size_t kOffOrd = kOffKey + 4 * (size_t)kMaxN;       // int32[kMaxN]
-constexpr size_t kOffCells = kOffOrd + 4 * (size_t)kMaxN;     // int32[2 kMaxNc^2 + 2]
-constexpr size_t kOffRp = kOffCells + 4 * (2 * (size_t)kMaxNc * kMaxNc + 2 + 2);  // int32[kMaxN + 1]
+constexpr size_t kOffCells = kOffOrd + 4 * (size_t)kMaxN;     // int32[kMaxNc^2 + 1]
+constexpr size_t kOffRp = kOffCells + 4 * ((size_t)kMaxNc * kMaxNc + 1 + 3);  // int32[kMaxN + 1]
 constexpr size_t kOffCol = kOffRp + 4 * ((size_t)kMaxN + 4);  // int32[kCap]
 constexpr size_t kScratchBytes = kOffCol + 4 * (size_t)kCap;
 
