@@ -379,7 +379,7 @@ pecc_status pecc_warm_start_ex(pecc_ctx *ctx, pecc_mlp *mlp, int32_t rounds, dou
 /* The feasibility check of pecc_check_feasible for ONE instance, without any device allocation.
  * The paper has no counterpart: this is a service for callers that cannot call cudaMalloc
  * (code running while its stream is captured into a CUDA graph, plug-ins whose host owns all
- * device memory, real-time loops).  Its scratch (about 0.85 MB) is a fixed array in device
+ * device memory, real-time loops).  Its scratch (about 0.77 MB) is a fixed array in device
  * memory that every GPU loading the library holds until the process exits.
  *   xy_dev          device double[2 n], interleaved (x, y)
  *   n               0 .. PECC_NOALLOC_MAX_N circles, else PECC_ERR_ARG (nothing launched)

@@ -222,10 +222,10 @@ template <> __device__ __forceinline__ Coords<double> coords_of<double>(const St
 }
 
 // Instances of at most kCellsBlockN circles, one block each, everything on chip: the coordinates come
-// in once, the rows, cells and order go out once.  What bounds it is the latency of the block's chain
-// (cell counts, two scans, candidate walks).  The 4096-instance batch's new positions, lists, energy and
-// gradient take 215 us with it, about 158 us of them here; 966 us with the kernel it replaced (lists
-// built and sorted in global memory, 901 us).
+// in once, the rows, cells and order go out once.  What bounds it is instruction issue (81 % of the slots)
+// and shared-memory wavefronts (61 %) of the candidate walks.  The 4096-instance batch's new positions,
+// lists, energy and gradient take 209 us with it, 152 us of them here; 966 us with lists built and sorted
+// in global memory (901 us).
 constexpr int kBuildWarpBytes = 32 * kRowHits * (int)sizeof(uint16_t);
 template <typename T>
 __global__ void __launch_bounds__(512, 3) build_block_kernel(StandaloneParams P, int force, int32_t *rebuilt) {
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(512, 3) build_block_kernel(StandaloneParams P,
 
 // ---- larger instances: one kernel per step over tiles of all of them (pecc_cells.cuh); each step reads
 // what the one before it wrote.  One block per instance left the GPU idle: new positions, lists, energy
-// and gradient of 100000 circles took 3842 us, now 88 us, most of it the launches' own latency.  The line
+// and gradient of 100000 circles took 3842 us, now 80 us, most of it the launches' own latency.  The line
 // to the block form is where its shared memory and one block's time end; from 1000 circles on a block
 // takes longer than the eight launches, but a batch of such instances fills the GPU with blocks.
 struct LargeDest { uint32_t *ckey; int32_t *corder; float2 *xs; };  // per circle (offset by the instance)
@@ -673,10 +673,9 @@ __global__ void __launch_bounds__(1024) energy_reduce_kernel(StandaloneParams P,
 // search runs in binary32; the binary64 values are formed for the pairs and circles whose binary32 ones
 // lie within the slack of the extreme.  The entries a list with cutoff l_cut > 2 would hold (it holds
 // every overlapping pair) are counted: past twice the capacity the instance is not checkable.
-// The 4096-instance batch: 150 us (447 us on its finished layouts, where every contact is near the extreme),
-// against 2212 us (2084) for a binary64 list build and a walk over it, which
-// the two binary64 lanes of an SM bound.  40 registers let six 256-thread blocks share an SM (170 us with
-// 64 registers and four).
+// The 4096-instance batch: 149 us (446 us on its finished layouts, where every contact is near the extreme),
+// against 2212 us (2084) for a binary64 list build and a walk over it, which the two binary64 lanes of an
+// SM bound.  40 registers let six 256-thread blocks share an SM (170 us with 64 registers and four).
 __device__ __forceinline__ double dist2_exact(double2 a, double2 b) {
   const double dx = __dsub_rn(a.x, b.x), dy = __dsub_rn(a.y, b.y);
   return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));

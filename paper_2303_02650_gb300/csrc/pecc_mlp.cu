@@ -136,7 +136,7 @@ __device__ __forceinline__ void feature_rows(const float2 *__restrict__ x, int n
 }
 
 // Instances of at most kCellsBlockN circles, one block each (pecc_cells.cuh).  Bound by instruction issue
-// of the collecting and inserting walks: 142 us for 665 000 circles in 1024 instances, 460 us when cells
+// of the collecting and inserting walks: 145 us for 665 000 circles in 1024 instances, 460 us when cells
 // and lists lay in global memory and every lane inserted as it walked.
 __global__ void __launch_bounds__(256) features_block_kernel(StandaloneParams P, int reach, float *feat) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -320,7 +320,7 @@ __device__ __forceinline__ bool tc_wait(uint64_t *mbar, uint32_t &phase) {
 // so that three tiles' epilogues run while another's MMAs do.  A group's tile of inputs and its hidden
 // activations take the same 32 KB (the inputs are dead once the first MMAs are done).  The features of
 // the next tile are loaded, coalesced, while the last layer runs.
-// 665 000 rows: 98 us, bound by shared-memory wavefronts and issue of the epilogues; 283 us with one group
+// 665 000 rows: 96 us, bound by shared-memory wavefronts and issue of the epilogues; 283 us with one group
 // per SM and row-wise feature loads.
 constexpr int kFwdGroups = 4;
 constexpr int kRowLoads = F;  // 32 rows of F floats per warp, one per lane and load
@@ -438,7 +438,7 @@ forward_tc_kernel(const bf16 *__restrict__ wb, const float *__restrict__ params,
 // stage, which then run behind the next epilogue; dZ2 takes H3's room for that.  The accumulators dW1 to
 // dW4 stay in TMEM until the block's last tile; the block then writes its partial gradient to
 // part[block][NPAR] and its loss to loss_part[block].
-// 333 000 rows: 159 us, bound by the chain of six MMA and epilogue stages per tile; 484 us with one
+// 333 000 rows: 161 us, bound by the chain of six MMA and epilogue stages per tile; 484 us with one
 // 128-thread group, the column sums as scalar reads of shared memory and every MMA waited for.
 // bwd_trace (may be null): float[rows][4][128], the bf16 dZ3, dZ2, dZ1 of every row, then its bf16
 // dO (2 values) and its outputs (2 values).
