@@ -1,6 +1,6 @@
 """Calls at the limits of what they take (marked gpu): list overflow of any length, shared memory of any
-size, contexts of several host threads, waits that run out,
-radii that are not radii or past binary32's range, cutoffs close to 2."""
+size, contexts of several host threads, waits that run out, radii that are not radii or past binary32's
+range, cutoffs close to 2, circles in one place or crowded."""
 import os
 import subprocess
 import sys
@@ -94,7 +94,7 @@ def test_first_call_of_a_process(orc, kind, n, others, prec):
     """Sizes whose dynamic shared memory is just below 48 KB, and above it with the kernel's own."""
     need_gpu()
     r = subprocess.run([sys.executable, "-c", FIRST_CALL, kind, str(n), str(others), str(prec)], cwd=ROOT,
-                       env=dict(os.environ, PYTHONPATH=ROOT), capture_output=True, text=True, timeout=300)
+                       capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "first call ok" in r.stdout, r.stdout[-2000:] + r.stderr[-2000:]
 
 
